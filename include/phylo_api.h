@@ -215,15 +215,17 @@ int phylo_gradient_branch_sum(phylo_ctx* ctx, const int32_t* branches, const dou
  * the last check (PHYLO_ENUMERIC) or PHYLO_OK. */
 int phylo_check(phylo_ctx* ctx);
 
-/* Number of kernel launches one evaluation makes (the level schedule's
- * length plus the matrix build and the final reduction); 0 before the
- * tree is set. */
+/* Number of steps of one evaluation (the level schedule's length plus the
+ * matrix build and the final reduction); 0 before the tree is set.  Each step
+ * is one kernel launch, except that with up to 4 states the FP64 path, and
+ * the FP32 path on problems of one wave of blocks, walk all the levels of a
+ * pass in one launch. */
 int phylo_launches_per_evaluation(const phylo_ctx* ctx);
 
-/* Length of the level schedule: the number of post-order launches (tree
+/* Length of the level schedule: the number of post-order steps (tree
  * height, less the heights left empty by fused cherries on the FP32
  * 4-state path; plus one for Eq. 3 at the root on the FP32 path for 65-128
- * states) and of pre-order launches (distinct depths of internal nodes;
+ * states) and of pre-order steps (distinct depths of internal nodes;
  * twice that on the FP32 path for 65-128 states, which runs two kernels per
  * level).  Both 0 before the tree is set. */
 int phylo_level_counts(const phylo_ctx* ctx, int* n_post_levels,

@@ -299,6 +299,7 @@ __device__ __forceinline__ void block_sum2(double& a, double& b,
 // ---------------------------------------------------------------------------
 template <typename T, int SP>
 __global__ void __launch_bounds__(256) pmat_kernel(PmatArgs a) {
+  if constexpr (SP == 4) pdl_release();
   constexpr int UPB = (256 / (SP * SP)) > 0 ? 256 / (SP * SP) : 1;
   __shared__ double she[UPB][SP];
   __shared__ double shd[UPB][SP];
@@ -326,6 +327,7 @@ __global__ void __launch_bounds__(256) pmat_kernel(PmatArgs a) {
   __syncthreads();
   T* P = static_cast<T*>(a.P);
   T* dP = static_cast<T*>(a.dP);
+  constexpr int SQ = SP * SP;
   for (int idx = threadIdx.x; idx < UPB * SP * SP; idx += blockDim.x) {
     const int u = idx / (SP * SP), e = idx % (SP * SP);
     const int unit = unit0 + u;
@@ -340,8 +342,15 @@ __global__ void __launch_bounds__(256) pmat_kernel(PmatArgs a) {
       }
       if (s == t) acc += 1.0;  // P = I + V diag(e^x - 1) Vinv
     }
-    P[(size_t)unit * SP * SP + e] = (T)acc;
-    dP[(size_t)unit * SP * SP + e] = (T)dacc;
+    if constexpr (SP == 4) {  // [P' | dP' | P] per branch
+      T* base = P + ((size_t)(unit / R) * kP4MatKinds * R + unit % R) * SQ;
+      base[t * SP + s] = (T)acc;
+      base[(size_t)R * SQ + t * SP + s] = (T)dacc;
+      base[(size_t)2 * R * SQ + e] = (T)acc;
+    } else {
+      P[(size_t)unit * SQ + e] = (T)acc;
+      dP[(size_t)unit * SQ + e] = (T)dacc;
+    }
   }
 }
 
@@ -1400,6 +1409,7 @@ inline size_t wide_pre_smem(int R) {
 }  // namespace phylo
 
 #include "kernels_p4.cuh"
+#include "kernels_tree.cuh"
 #include "kernels_tc64.cuh"
 #include "kernels_big.cuh"
 #include "kernels_tcb.cuh"
@@ -1413,8 +1423,7 @@ namespace phylo {
 // bounded by registers (the inputs of all NPT nodes are held at once).
 template <typename T, int SP>
 struct SmallNpt {
-  static constexpr int post = (SP == 4) ? 4 : 2;
-  static constexpr int pre = (SP == 4) ? (sizeof(T) == 4 ? 4 : 2) : 1;
+  static constexpr int post = 2, pre = 1;
 };
 
 template <typename T, int SP, int RP, int NPT>
@@ -1496,7 +1505,7 @@ cudaError_t launch_level_impl(const LevelArgs<T>& a, int SP, int RP, bool post,
   switch (SP) {
     case 4:
       if constexpr (std::is_same<T, float>::value) return launch_p4_rp(a, RP, post, st);
-      else return launch_small_rp<T, 4>(a, RP, post, st);
+      else return cudaErrorInvalidValue;  // FP64: launch_tree_pass
     case 20: return launch_small_rp<T, 20>(a, RP, post, st);
     case 64:
       if constexpr (std::is_same<T, float>::value) {
@@ -1518,7 +1527,7 @@ cudaError_t launch_level_impl(const LevelArgs<T>& a, int SP, int RP, bool post,
 
 template <typename T>
 cudaError_t prepare_impl(int SP, int RP) {
-  if (SP == 4) return prepare_small_rp<T, 4>(RP);
+  if (SP == 4) return prepare_tree<T>(RP);
   if (SP == 20) return prepare_small_rp<T, 20>(RP);
   if (SP == 64) {
     if constexpr (std::is_same<T, float>::value) {
@@ -1600,6 +1609,11 @@ cudaError_t launch_pre_finish_impl(const LevelArgs<T>& a, int SP, cudaStream_t s
   cudaError_t launch_pre_level<T>(const LevelArgs<T>& a, int SP, int RP,      \
                                   cudaStream_t st) {                          \
     return launch_level_impl<T>(a, SP, RP, false, st);                        \
+  }                                                                           \
+  template <>                                                                 \
+  cudaError_t launch_tree_pass<T>(const LevelArgs<T>& a, const TreePass& p,   \
+                                  int RP, cudaStream_t st) {                  \
+    return launch_tree<T>(a, p, RP, st);                                      \
   }                                                                           \
   template <>                                                                 \
   cudaError_t launch_pre_finish<T>(const LevelArgs<T>& a, int SP,             \

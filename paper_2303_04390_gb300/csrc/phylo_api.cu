@@ -10,6 +10,7 @@
 // captured once per tree into a CUDA graph and replayed on the caller's
 // stream.  The paper instead launches one kernel per node (post-order and
 // pre-order) plus separate gradient and site-reduction kernels.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -37,8 +38,10 @@ struct Region {
 // Workspace layout of one context (all offsets 256-byte aligned).
 struct Layout {
   int SP = 0, RP = 0, n_tiles = 0;
+  PassMode mode = kByLevel;
   size_t elem = 0;
   Region children, post_nodes, pre_nodes, post_desc, pre_desc;
+  Region post_off, pre_off;  // whole-pass launches: the level offsets
   Region P, dP, post, pre, escale, pre_escale, rterm;
   Region tip_states, tip_partials, tip_has;
   Region pattern_w, V, Vinv, lambda, pi, rates, cat_w, t;
@@ -80,8 +83,9 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
   L.SP = padded_states(S);
   L.RP = lanes_per_pattern(R);
   L.elem = prec == PHYLO_FP64 ? 8 : 4;
-  const int ct = patterns_per_tile(L.SP, R, prec == PHYLO_FP64);
-  L.n_tiles = (C + ct - 1) / ct;
+  L.mode = pass_mode(L.SP, prec == PHYLO_FP64, N, C, R, L.RP);
+  const int ct = patterns_per_tile(L.SP, R, prec == PHYLO_FP64, L.mode);
+  L.n_tiles = (int)(((long long)C + ct - 1) / ct);
   const size_t n_nodes = 2 * (size_t)N - 1, n_br = 2 * (size_t)N - 2;
   const size_t n_int = (size_t)N - 1;
   size_t mat, part, tmp, tmp2;
@@ -91,7 +95,8 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
                          : (size_t)L.SP * L.SP * L.elem * (p4 ? kP4MatKinds : 1);
   if (!mul_ok(n_br * R, unit, &mat)) return "size overflow";
   if (C > (1 << 30)) return "n_patterns too large";
-  const size_t per_node = partial_elems_per_node(L.SP, prec == PHYLO_FP64, C, R, L.n_tiles);
+  const size_t per_node = partial_elems_per_node(L.SP, prec == PHYLO_FP64, C, R, L.n_tiles,
+                                                 L.mode);
   if (!mul_ok(n_int, per_node, &tmp) || !mul_ok(tmp, L.elem, &part)) return "size overflow";
   bool ok = true;
   ok &= add_region(L, L.children, n_nodes * sizeof(int2));
@@ -99,6 +104,10 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
   ok &= add_region(L, L.pre_nodes, n_int * sizeof(int));
   ok &= add_region(L, L.post_desc, n_int * sizeof(int4));
   ok &= add_region(L, L.pre_desc, n_int * sizeof(int4));
+  if (L.mode != kByLevel) {
+    ok &= add_region(L, L.post_off, (n_int + 1) * sizeof(int));
+    ok &= add_region(L, L.pre_off, (n_int + 1) * sizeof(int));
+  }
   ok &= add_region(L, L.P, mat);
   ok &= add_region(L, L.dP, tc || p4 ? 0 : mat);  // else the P region holds dP
   if (uses_tc_big(L.SP, prec == PHYLO_FP64)) {
@@ -118,10 +127,10 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
   } else {
     ok &= add_region(L, L.post, part);
   }
-  ok &= add_region(L, L.pre, part);
+  ok &= add_region(L, L.pre, L.mode == kWalk ? 0 : part);
   if (tc || uses_tc_big(L.SP, prec == PHYLO_FP64)) ok &= add_region(L, L.qt, qt_bytes(L.SP));
-  if (prec == PHYLO_FP32 && (L.SP == 4 || L.SP == 20))  // the U form's Q (FP32, row-major)
-    ok &= add_region(L, L.qmat, (size_t)L.SP * L.SP * sizeof(float));
+  if (uses_tr_layout(L.SP, prec == PHYLO_FP64))  // the U form's Q (row-major)
+    ok &= add_region(L, L.qmat, (size_t)L.SP * L.SP * L.elem);
   if (C > (1 << 30)) return "n_patterns too large";
   const int planes = escale_planes(L.SP, R, prec == PHYLO_FP64);
   if (!mul_ok(n_int * planes, (size_t)round_up(C, 4) * sizeof(int), &tmp))
@@ -192,6 +201,7 @@ struct phylo_ctx {
   std::vector<int2> children;
   std::vector<int> post_nodes, post_off;  // level l: [post_off[l], post_off[l+1])
   std::vector<int> pre_nodes, pre_off;
+  int n_post_levels = 0, n_pre_levels = 0;    // the level schedule's length
   std::vector<char> post_cherry, pre_cherry;  // per level: a node has a fused cherry child
   std::vector<int> height, depth;             // per node
   std::vector<char> cherry;                   // per node: fused into its parent
@@ -300,7 +310,7 @@ LevelArgs<T> level_args(const phylo_ctx* ctx) {
   a.err = reinterpret_cast<int*>(ctx->dev<double>(ctx->L.out) + 2 * ctx->N - 1);
   a.tc_tiles = ctx->L.tc_tiles.bytes ? ctx->dev<unsigned char>(ctx->L.tc_tiles) : nullptr;
   a.qt = ctx->L.qt.bytes ? ctx->dev<unsigned char>(ctx->L.qt) : nullptr;
-  a.qmat = ctx->L.qmat.bytes ? ctx->dev<float>(ctx->L.qmat) : nullptr;
+  a.qmat = ctx->L.qmat.bytes ? ctx->dev<T>(ctx->L.qmat) : nullptr;
   a.rates = ctx->dev<double>(ctx->L.rates);
   a.tip_level = 0;
   return a;
@@ -313,6 +323,21 @@ bool has_tip_level(const phylo_ctx* ctx) {
   for (int v : ctx->tip_has)
     if (v) return true;
   return false;
+}
+
+int widest_level(const std::vector<int>& off) {
+  int w = 0;
+  for (size_t l = 0; l + 1 < off.size(); ++l) w = std::max(w, off[l + 1] - off[l]);
+  return w;
+}
+
+// Warps per block of a kWalk launch with 2^g tiles: one for each (node, tile)
+// of the widest level.
+int walk_warps(const phylo_ctx* ctx, int g) {
+  const int widest = std::max(widest_level(ctx->post_off), widest_level(ctx->pre_off)) << g;
+  int w = 2;
+  while (w < kWalkMaxWarps && w < widest) w *= 2;
+  return w;
 }
 
 int* flag_word(const phylo_ctx* ctx) {
@@ -329,6 +354,30 @@ constexpr int kPhaseLogLOnly = 4;
 constexpr unsigned kSeqEvaluate = 0xf;
 constexpr unsigned kSeqForward = 1u << 0 | 1u << 1 | 1u << kPhaseLogLOnly;
 constexpr unsigned kSeqBackward = 1u << 2 | 1u << 3;
+
+// The post-order (1) and pre-order (2) phases of a kByTile or kWalk problem;
+// together they are one launch for kWalk.
+template <typename T>
+cudaError_t enqueue_tree(phylo_ctx* ctx, bool do_post, bool do_pre, cudaStream_t st) {
+  NvtxRange range(!do_pre    ? "phylo post-order pass (Eq. 2)"
+                  : !do_post ? "phylo pre-order pass (Eqs. 4, 8)"
+                             : "phylo post- and pre-order passes (Eqs. 2, 4, 8)");
+  TreePass p{};
+  for (bool post : {true, false}) {
+    TreeSched& s = post ? p.post : p.pre;
+    s.desc = ctx->dev<int4>(post ? ctx->L.post_desc : ctx->L.pre_desc);
+    s.off = ctx->dev<int>(post ? ctx->L.post_off : ctx->L.pre_off);
+    s.n_levels = (int)(post ? ctx->post_off : ctx->pre_off).size() - 1;
+  }
+  p.do_post = do_post;
+  p.do_pre = do_pre;
+  p.walk = ctx->L.mode == kWalk;
+  if (p.walk) {
+    p.group = walk_group(ctx->precision == PHYLO_FP64, ctx->N, ctx->C, ctx->R, ctx->L.RP);
+    p.warps = walk_warps(ctx, p.group);
+  }
+  return launch_tree_pass<T>(level_args<T>(ctx), p, ctx->L.RP, st);
+}
 
 template <typename T>
 cudaError_t enqueue_phase(phylo_ctx* ctx, int phase, cudaStream_t st) {
@@ -409,8 +458,15 @@ cudaError_t enqueue_phase(phylo_ctx* ctx, int phase, cudaStream_t st) {
 cudaError_t enqueue_phases(phylo_ctx* ctx, unsigned seq, cudaStream_t st) {
   for (int ph = 0; ph <= kPhaseLogLOnly; ++ph) {
     if (!(seq >> ph & 1u)) continue;
-    cudaError_t e = ctx->precision == PHYLO_FP64 ? enqueue_phase<double>(ctx, ph, st)
-                                                 : enqueue_phase<float>(ctx, ph, st);
+    const bool fp64 = ctx->precision == PHYLO_FP64;
+    cudaError_t e;
+    if (ctx->L.mode != kByLevel && (ph == 1 || ph == 2)) {
+      const bool pre = seq >> 2 & 1u, post = ph == 1;
+      e = fp64 ? enqueue_tree<double>(ctx, post, pre, st) : enqueue_tree<float>(ctx, post, pre, st);
+      if (post && pre) ph = 2;
+    } else {
+      e = fp64 ? enqueue_phase<double>(ctx, ph, st) : enqueue_phase<float>(ctx, ph, st);
+    }
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -484,6 +540,7 @@ int upload(phylo_ctx* ctx, const Region& r, const T* host, size_t count,
 int build_schedule(phylo_ctx* ctx) {
   const int N = ctx->N, n = 2 * N - 1, root = n - 1;
   const bool fuse = ctx->precision == PHYLO_FP32 && ctx->L.SP == 4;
+  const bool tree = ctx->L.mode != kByLevel;  // every node has its own step
   const std::vector<int2>& ch = ctx->children;
   ctx->cherry.assign(n, 0);
   if (fuse)
@@ -499,10 +556,13 @@ int build_schedule(phylo_ctx* ctx) {
     D = ctx->depth[v] > D ? ctx->depth[v] : D;
   }
   std::vector<std::vector<int>> by_height(H + 1), by_depth(D + 1);
+  std::vector<char> launched(H + 1, 0);  // heights with an unfused node
   for (int v = N; v < n; ++v) {
-    if (!ctx->cherry[v]) by_height[ctx->height[v]].push_back(v);
+    launched[ctx->height[v]] |= !ctx->cherry[v];
+    if (tree || !ctx->cherry[v]) by_height[ctx->height[v]].push_back(v);
     by_depth[ctx->depth[v]].push_back(v);
   }
+  if (tree) ctx->cherry.assign(n, 0);
   for (int pass = 0; pass < 2; ++pass) {
     std::vector<int>& nodes = pass == 0 ? ctx->post_nodes : ctx->pre_nodes;
     std::vector<int>& off = pass == 0 ? ctx->post_off : ctx->pre_off;
@@ -522,7 +582,16 @@ int build_schedule(phylo_ctx* ctx) {
       flag.push_back(any);
     }
   }
-  int rc = upload(ctx, ctx->L.post_nodes, ctx->post_nodes.data(), ctx->post_nodes.size(),
+  ctx->n_pre_levels = (int)ctx->pre_off.size() - 1;
+  ctx->n_post_levels = 0;
+  for (char any : launched) ctx->n_post_levels += any;
+  int rc = tree ? upload(ctx, ctx->L.post_off, ctx->post_off.data(), ctx->post_off.size(),
+                         "upload schedule")
+                : PHYLO_OK;
+  if (!rc && tree)
+    rc = upload(ctx, ctx->L.pre_off, ctx->pre_off.data(), ctx->pre_off.size(), "upload schedule");
+  if (rc) return rc;
+  rc = upload(ctx, ctx->L.post_nodes, ctx->post_nodes.data(), ctx->post_nodes.size(),
                   "upload schedule");
   if (rc) return rc;
   rc = upload(ctx, ctx->L.pre_nodes, ctx->pre_nodes.data(), ctx->pre_nodes.size(),
@@ -642,7 +711,7 @@ int launch_eval(phylo_ctx* ctx) {
   if (ctx->flags & PHYLO_FLAG_NO_GRAPH) {
     rc = run_phases(ctx, kSeqEvaluate, nullptr);
     if (rc) return rc;
-    ctx->forward_valid = true;
+    ctx->forward_valid = ctx->L.mode != kWalk;  // (a walk keeps no partials)
     ctx->have_grad = true;
     return PHYLO_OK;
   }
@@ -651,7 +720,7 @@ int launch_eval(phylo_ctx* ctx) {
     if (rc) return rc;
   }
   CUDA_TRY(ctx, cudaGraphLaunch(ctx->gexec, ctx->stream), "cudaGraphLaunch");
-  ctx->forward_valid = true;
+  ctx->forward_valid = ctx->L.mode != kWalk;
   ctx->have_grad = true;
   return PHYLO_OK;
 }
@@ -981,9 +1050,9 @@ int phylo_set_eigen(phylo_ctx* ctx, const double* V, const double* Vinv,
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
   }
   if (ctx->L.qmat.bytes) {
-    std::vector<float> qm((size_t)ctx->L.SP * ctx->L.SP);
+    std::vector<double> qm((size_t)ctx->L.SP * ctx->L.SP);
     build_q_matrix(S, ctx->L.SP, V, Vinv, lambda, qm.data());
-    if ((rc = upload(ctx, ctx->L.qmat, qm.data(), qm.size(), "upload Q"))) return rc;
+    if ((rc = upload_typed(ctx, ctx->L.qmat, qm.data(), qm.size(), "upload Q"))) return rc;
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
   }
   if (ctx->L.qt.bytes) {
@@ -1350,7 +1419,7 @@ int phylo_launches_per_evaluation(const phylo_ctx* ctx) {
   int n = 2;  // pmat + final reduction
   if (ctx->C > 0) {
     const bool fp64 = ctx->precision == PHYLO_FP64;
-    n += (int)(ctx->post_off.size() - 1) + (int)(ctx->pre_off.size() - 1);
+    n += ctx->n_post_levels + ctx->n_pre_levels;
     if (uses_tc_terms(ctx->L.SP, fp64)) ++n;  // Eq. 8 ratios
     if (has_tip_level(ctx)) ++n;                // U of the tips with partials
   }
@@ -1360,8 +1429,8 @@ int phylo_launches_per_evaluation(const phylo_ctx* ctx) {
 int phylo_level_counts(const phylo_ctx* ctx, int* n_post_levels,
                        int* n_pre_levels) {
   if (!ctx || !n_post_levels || !n_pre_levels) return PHYLO_EINVAL;
-  *n_post_levels = ctx->have_tree ? (int)ctx->post_off.size() - 1 : 0;
-  *n_pre_levels = ctx->have_tree ? (int)ctx->pre_off.size() - 1 : 0;
+  *n_post_levels = ctx->have_tree ? ctx->n_post_levels : 0;
+  *n_pre_levels = ctx->have_tree ? ctx->n_pre_levels : 0;
   if (ctx->have_tree && ctx->C > 0 && has_tip_level(ctx)) ++*n_post_levels;
   return PHYLO_OK;
 }

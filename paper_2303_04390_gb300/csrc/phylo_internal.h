@@ -74,8 +74,58 @@ inline int tip_state_stride(int C) { return round_up(C, 16); }
 // branch, [P' of every category][dP' of every category][P of every
 // category] (SP x SP floats each; P' rows are the columns of P).  The dP
 // region is then empty.
-inline bool uses_tr_layout(int SP, bool fp64) { return (SP == 4 || SP == 20) && !fp64; }
+inline bool uses_tr_layout(int SP, bool fp64) { return SP == 4 || (SP == 20 && !fp64); }
 constexpr int kP4MatKinds = 3;
+// How a pass of the level schedule runs.
+enum PassMode {
+  kByLevel,  // one launch per level
+  kByTile,   // one launch: a pattern tile walks the tree (kernels_tree.cuh)
+  kWalk      // the same with every partial vector in shared memory
+};
+// Whole-pass launches, 4 padded states: tiles of one warp of (pattern,
+// category) lanes.
+constexpr int kTreeWarps = 8;      // warps per block, kByTile
+constexpr int kWalkMaxWarps = 16;  // warps per block, kWalk
+constexpr int kSms = 152;          // SMs of the GPU: blocks of one wave
+constexpr int kWalkMaxGroup = 2;   // at most 4 tiles per block, kWalk
+constexpr size_t kWalkMaxSmem = 226 * 1024;
+constexpr uint32_t kWalkCopy = 32768;  // bytes per bulk copy of the matrices
+// Shared memory of a kWalk block with 2^g tiles: the matrices of every branch
+// (at offset 0), the nodes' vectors, Q, both schedules (descriptors, level
+// offsets), the tips' states.
+struct WalkPlan {
+  size_t vec, q, desc, off, states, total;
+  __host__ __device__ WalkPlan(int n_tips, int R, int RP, int g, bool fp64) {
+    const size_t elem = fp64 ? 8 : 4, N = n_tips;
+    vec = (2 * N - 2) * kP4MatKinds * R * 16 * elem;
+    q = vec + ((N - 2) << g) * 128 * elem;
+    desc = q + RP * 16 * elem;
+    off = desc + 2 * (N - 1) * 16;
+    states = off + (2 * N * 4 + 15) / 16 * 16;
+    total = states + ((N << g) * (32 / RP) + 15) / 16 * 16;
+  }
+};
+// Tiles per block (log2) of a kWalk launch, -1 if the problem does not fit in
+// one wave of blocks: the smallest group with a block per SM, else the
+// largest that shared memory holds.  A second wave loses: 61 taxa x 5,000
+// patterns took 100 us against 78 level by level, x 2,000 (one wave) 45
+// against 77.
+inline int walk_group(bool fp64, int n_tips, int C, int R, int RP) {
+  const long long tiles = ((long long)C * RP + 31) / 32;
+  auto smem = [&](int g) { return WalkPlan(n_tips, R, RP, g, fp64).total; };
+  auto blocks = [&](int g) { return (tiles + (1 << g) - 1) >> g; };
+  int g = 0;
+  while (g < kWalkMaxGroup && blocks(g) > kSms) ++g;
+  while (g >= 0 && smem(g) > kWalkMaxSmem) --g;
+  if (g < 0) return -1;
+  const int resident = !fp64 && 2 * (smem(g) + 2048) <= 228 * 1024 ? 2 : 1;
+  return blocks(g) <= kSms * resident ? g : -1;
+}
+inline PassMode pass_mode(int SP, bool fp64, int n_tips, int C, int R, int RP) {
+  if (SP != 4) return kByLevel;
+  if (walk_group(fp64, n_tips, C, R, RP) >= 0) return kWalk;
+  return fp64 ? kByTile : kByLevel;
+}
 
 // FP32 with 21..64 states runs on the tensor cores (kernels_tc64.cuh):
 // 128-pattern tiles and one rescale exponent per (node, category, pattern).
@@ -144,16 +194,17 @@ inline bool uses_u_form(int SP, bool fp64) {
   return (SP == 20 || SP == 64 || SP == 128) && !fp64;
 }
 
-// Q = V diag(lambda) Vinv in FP64, rounded once to FP32, row-major SP x SP
+// Q = V diag(lambda) Vinv in FP64, rounded once to T, row-major SP x SP
 // with zero padding (the pre-order step of the 4- and 20-state U form).
+template <typename T>
 inline void build_q_matrix(int S, int SP, const double* V, const double* Vinv,
-                           const double* lambda, float* out) {
-  for (int i = 0; i < SP * SP; ++i) out[i] = 0.f;
+                           const double* lambda, T* out) {
+  for (int i = 0; i < SP * SP; ++i) out[i] = T(0);
   for (int t = 0; t < S; ++t)
     for (int s = 0; s < S; ++s) {
       double q = 0.0;
       for (int m = 0; m < S; ++m) q += V[t * S + m] * lambda[m] * Vinv[m * S + s];
-      out[t * SP + s] = (float)q;
+      out[t * SP + s] = (T)q;
     }
 }
 
@@ -222,7 +273,8 @@ inline int escale_planes(int SP, int R, bool fp64) {
 }
 
 // Patterns of one tile (the unit of the per-tile gradient sums).
-inline int patterns_per_tile(int SP, int R, bool fp64) {
+inline int patterns_per_tile(int SP, int R, bool fp64, PassMode mode = kByLevel) {
+  if (mode != kByLevel) return 32 / lanes_per_pattern(R);
   if (SP == 4 && !fp64) return kP4TilePatterns;
   if (uses_tc_terms(SP, fp64)) return kTcTilePatterns;
   if (SP <= 20) return kSmallThreads / lanes_per_pattern(R);
@@ -234,8 +286,10 @@ inline int patterns_per_tile(int SP, int R, bool fp64) {
 // patterns to whole tiles: FP32 with 4 padded states ([tile][r][32][4]),
 // FP32 with 20 padded states ([tile][chunk][kSmallThreads][4], every lane of
 // the RP-wide category slots present); the others store [C][R][SP].
-inline size_t partial_elems_per_node(int SP, bool fp64, int C, int R, int n_tiles) {
-  if (uses_p4_tiles(SP, fp64)) return (size_t)n_tiles * kP4TilePatterns * R * SP;
+inline size_t partial_elems_per_node(int SP, bool fp64, int C, int R, int n_tiles,
+                                     PassMode mode = kByLevel) {
+  if (mode == kWalk) return (size_t)n_tiles * 32 * SP;
+  if (uses_p4_tiles(SP, fp64) && mode == kByLevel) return (size_t)n_tiles * kP4TilePatterns * R * SP;
   if (SP == 20 && !fp64) return (size_t)n_tiles * kSmallThreads * SP;
   return (size_t)C * R * SP;
 }
@@ -286,7 +340,7 @@ struct LevelArgs {
   const unsigned char* tc_tiles;  // 65..128 states, FP32: the pre-split matrix
                                   // blocks [2N-2][R][kTcbUnitBytes] (else null)
   const unsigned char* qt;     // 21..64 states, FP32: Q' operand (kTcQtBytes)
-  const float* qmat;           // 4 and 20 padded states, FP32: Q row-major [SP][SP]
+  const T* qmat;               // 4 and 20 padded states, U form: Q row-major [SP][SP]
   const double* rates;         // [R] category rates gamma_r
   int tip_level;               // U-form paths: the level's nodes are tips with
                                // partials (their U = P p, before level 1)
@@ -294,6 +348,30 @@ struct LevelArgs {
                                // began (every launch but the first after the
                                // matrix kernel): the level may read P and its
                                // descriptors before griddepcontrol.wait
+};
+
+struct ReduceArgs {
+  const double* gpart;   // [n_branches][n_tiles]; with gpart_pairs each entry
+                         // holds a float pair {hi, lo} (value hi + lo)
+  const double* lpart;   // [n_tiles]
+  int n_tiles, n_branches;
+  int gpart_pairs;       // FP32 with 4 or 20 padded states: tile sums as float
+                         // pairs (no FP64 in those level kernels)
+  double* out;           // [1 + n_branches]
+};
+
+// The level schedule of a pass on the device: descriptors in level order,
+// level l in [off[l], off[l + 1]).
+struct TreeSched {
+  const int4* desc;
+  const int* off;
+  int n_levels;
+};
+struct TreePass {
+  TreeSched post, pre;
+  bool do_post, do_pre;
+  bool walk;
+  int warps, group;  // kWalk: warps per block, log2 of its tiles
 };
 
 struct PmatArgs {
@@ -310,16 +388,6 @@ struct PmatArgs {
   void* tiles;           // 65..128 states, FP32: the matrices written as pre-split
                          // operand blocks instead of P and dP (else null)
   int* err;
-};
-
-struct ReduceArgs {
-  const double* gpart;   // [n_branches][n_tiles]; with gpart_pairs each entry
-                         // holds a float pair {hi, lo} (value hi + lo)
-  const double* lpart;   // [n_tiles]
-  int n_tiles, n_branches;
-  int gpart_pairs;       // FP32 with 4 or 20 padded states: tile sums as float
-                         // pairs (no FP64 in those level kernels)
-  double* out;           // [1 + n_branches]
 };
 
 // Launch with programmatic stream serialisation: the kernel may begin
@@ -354,6 +422,9 @@ cudaError_t launch_post_level(const LevelArgs<T>& a, int SP, int RP,
 template <typename T>
 cudaError_t launch_pre_level(const LevelArgs<T>& a, int SP, int RP,
                              cudaStream_t st);
+// The passes of a kByTile or kWalk problem.
+template <typename T>
+cudaError_t launch_tree_pass(const LevelArgs<T>& a, const TreePass& p, int RP, cudaStream_t st);
 // Work after the last pre-order level (the tensor-core path's Eq. 8
 // ratios); a no-op elsewhere.
 template <typename T>

@@ -90,4 +90,11 @@ __device__ __forceinline__ void pdl_wait_and_release() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The first kernel of an evaluation (the matrix build), which is launched
+// without the attribute: nothing is in flight before it, so it releases its
+// successor at once and that kernel's launch overlaps the build.
+__device__ __forceinline__ void pdl_release() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 }  // namespace phylo
