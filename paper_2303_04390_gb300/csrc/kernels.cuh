@@ -1052,365 +1052,12 @@ constexpr size_t u20_smem(bool post) {
          sizeof(float);
 }
 
-// ---------------------------------------------------------------------------
-// Shared-memory kernels for SP = 64 (S in 21..64): one thread per (pattern
-// group, state s); each thread owns CPG patterns of its group; categories
-// are processed one at a time with that category's matrices staged in a
-// padded (stride SP+1, bank-conflict-free both ways) shared layout.
-// ---------------------------------------------------------------------------
-template <typename T> struct WideCfg;
-template <> struct WideCfg<float> { static constexpr int CT = kWidePatternsF32; };
-template <> struct WideCfg<double> { static constexpr int CT = kWidePatternsF64; };
-
-constexpr int kWideSP = 64;
-constexpr int kWideLD = kWideSP + 1;
-
-template <typename T>
-__device__ __forceinline__ void stage_mat_padded(const T* __restrict__ src,
-                                                 T* dst) {
-  for (int idx = threadIdx.x; idx < kWideSP * kWideSP; idx += blockDim.x) {
-    const int s = idx / kWideSP, t = idx % kWideSP;
-    dst[s * kWideLD + t] = src[idx];
-  }
-}
-
-// Stage child vectors for category r into vin[CT][SP]; tips with compact
-// states store their state in ystate[CT] instead.
-template <typename T>
-__device__ __forceinline__ void stage_child_vec(const LevelArgs<T>& a, int b,
-                                                int c0, int r, T* vin,
-                                                int* ystate) {
-  constexpr int CT = WideCfg<T>::CT;
-  const int C = a.n_patterns, R = a.n_cat;
-  const bool compact =
-      b < a.n_tips && !(a.tip_has_partials && a.tip_has_partials[b]);
-  if (compact) {
-    for (int j = threadIdx.x; j < CT; j += blockDim.x) {
-      const int c = c0 + j;
-      ystate[j] = c < C ? (int)a.tip_states[(size_t)b * a.state_stride + c] : 0;
-    }
-    return;
-  }
-  for (int idx = threadIdx.x; idx < CT * kWideSP; idx += blockDim.x) {
-    const int j = idx / kWideSP, s = idx % kWideSP, c = c0 + j;
-    T v = T(0);
-    if (c < C) {
-      if (b < a.n_tips)
-        v = a.tip_partials[((size_t)b * C + c) * kWideSP + s];
-      else
-        v = a.post[(((size_t)(b - a.n_tips) * C + c) * R + r) * kWideSP + s];
-    }
-    vin[j * kWideSP + s] = v;
-  }
-  if (threadIdx.x < CT) ystate[threadIdx.x] = -1;
-}
-
-// u = M v for state s of pattern j (M padded in smem).
-template <typename T>
-__device__ __forceinline__ T wide_up(const T* M, const T* vin, const int* ys,
-                                     int j, int s, int S) {
-  const int y = ys[j];
-  if (y >= 0) {
-    if (y < S) return M[s * kWideLD + y];
-    return s < S ? T(1) : T(0);
-  }
-  const T* v = vin + j * kWideSP;
-  T acc = T(0);
-#pragma unroll 16
-  for (int t = 0; t < kWideSP; ++t) acc = fma(M[s * kWideLD + t], v[t], acc);
-  return acc;
-}
-
-template <typename T>
-__device__ __forceinline__ T wide_up_gap_d(const int* ys, int j, int S,
-                                           T dval) {
-  // derivative of a gap tip's all-ones vector is exactly 0
-  const int y = ys[j];
-  return (y >= S) ? T(0) : dval;
-}
-
-template <typename T>
-struct WideSmemPost {
-  T mat[2][kWideSP * kWideLD];
-  T vin[2][WideCfg<T>::CT * kWideSP];
-  T pk[8][WideCfg<T>::CT * kWideSP];
-  int ys[2][WideCfg<T>::CT];
-  T redm[WideCfg<T>::CT][kWideThreads / 32];
-  double redl[kWideThreads / 32][2];
-};
-
-template <typename T>
-__global__ void __launch_bounds__(kWideThreads) post_wide_kernel(LevelArgs<T> a) {
-  pdl_wait_and_release();
-  constexpr int CT = WideCfg<T>::CT;
-  constexpr int NT = kWideThreads;
-  constexpr int GROUPS = NT / kWideSP;  // 4
-  constexpr int CPG = CT / GROUPS;      // patterns per thread
-  extern __shared__ __align__(16) unsigned char smraw[];
-  WideSmemPost<T>& sm = *reinterpret_cast<WideSmemPost<T>*>(smraw);
-  const int k = a.level_nodes[blockIdx.y];
-  const int2 ch = a.children[k];
-  const int R = a.n_cat, C = a.n_patterns, S = a.n_states;
-  const int c0 = blockIdx.x * CT;
-  const int g = threadIdx.x / kWideSP, s = threadIdx.x % kWideSP;
-  int eacc[CPG];
-#pragma unroll
-  for (int jj = 0; jj < CPG; ++jj) eacc[jj] = 0;
-  for (int r = 0; r < R; ++r) {
-    __syncthreads();
-    stage_mat_padded<T>(a.P + ((size_t)ch.x * R + r) * kWideSP * kWideSP,
-                        sm.mat[0]);
-    stage_mat_padded<T>(a.P + ((size_t)ch.y * R + r) * kWideSP * kWideSP,
-                        sm.mat[1]);
-    stage_child_vec<T>(a, ch.x, c0, r, sm.vin[0], sm.ys[0]);
-    stage_child_vec<T>(a, ch.y, c0, r, sm.vin[1], sm.ys[1]);
-    __syncthreads();
-#pragma unroll
-    for (int jj = 0; jj < CPG; ++jj) {
-      const int j = g * CPG + jj;
-      const T ui = wide_up<T>(sm.mat[0], sm.vin[0], sm.ys[0], j, s, S);
-      const T uj = wide_up<T>(sm.mat[1], sm.vin[1], sm.ys[1], j, s, S);
-      sm.pk[r][j * kWideSP + s] = ui * uj;
-    }
-  }
-  __syncthreads();
-  // exponents of the children (internal ones)
-  for (int jj = 0; jj < CPG; ++jj) {
-    const int j = g * CPG + jj, c = c0 + j;
-    int e = 0;
-    if (c < C) {
-      if (ch.x >= a.n_tips) e += a.escale[(size_t)(ch.x - a.n_tips) * a.escale_stride + c];
-      if (ch.y >= a.n_tips) e += a.escale[(size_t)(ch.y - a.n_tips) * a.escale_stride + c];
-    }
-    eacc[jj] = e;
-  }
-  // max over (r, s) per pattern: 64 threads of the group = 2 warps
-  const int warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int jj = 0; jj < CPG; ++jj) {
-    const int j = g * CPG + jj;
-    T m = T(0);
-    for (int r = 0; r < R; ++r) m = tmax(m, fabs(sm.pk[r][j * kWideSP + s]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = tmax(m, __shfl_xor_sync(kFull, m, o));
-    if ((threadIdx.x & 31) == 0) sm.redm[j][warp] = m;
-  }
-  __syncthreads();
-  double lterm = 0.0;
-#pragma unroll
-  for (int jj = 0; jj < CPG; ++jj) {
-    const int j = g * CPG + jj, c = c0 + j;
-    const T m = tmax(sm.redm[j][2 * g], sm.redm[j][2 * g + 1]);
-    int e = 0;
-    if (c < C) {
-      if (!(m > T(0)) || !isfinite(m)) atomicOr(a.err, ERR_ZERO_PARTIAL);
-      else (void)frexp(m, &e);
-    }
-    const T f = ldexp(T(1), -e);
-    const int etot = e + eacc[jj];
-    if (k != a.root) {
-      if (c < C) {
-        const size_t slot = (size_t)(k - a.n_tips);
-        for (int r = 0; r < R; ++r)
-          a.post[((slot * C + c) * R + r) * kWideSP + s] =
-              sm.pk[r][j * kWideSP + s] * f;
-        if (s == 0) a.escale[slot * a.escale_stride + c] = etot;
-      }
-    } else {
-      // root: sum_r w_r pi' p over the group's 64 threads
-      double lr = 0.0;
-      if (c < C && s < S)
-        for (int r = 0; r < R; ++r)
-          lr += a.cat_w[r] * a.root_pi[s] *
-                (double)(sm.pk[r][j * kWideSP + s] * f);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) lr += __shfl_xor_sync(kFull, lr, o);
-      // combine the group's two warps through shared memory
-      __syncthreads();
-      if ((threadIdx.x & 31) == 0) sm.redl[warp][0] = lr;
-      __syncthreads();
-      if (s == 0 && c < C) {
-        const double L = sm.redl[2 * g][0] + sm.redl[2 * g + 1][0];
-        if (!(L > 0.0) || !isfinite(L)) atomicOr(a.err, ERR_ZERO_PARTIAL);
-        lterm += a.pattern_w[c] * (log(L) + (double)etot * 0.69314718055994530942);
-      }
-    }
-  }
-  if (k == a.root) {
-    __syncthreads();
-    double unused = 0.0;
-    block_sum2<NT>(lterm, unused, sm.redl);
-    if (threadIdx.x == 0) a.lpart[blockIdx.x] = lterm;
-  }
-}
-
-template <typename T>
-struct WideSmemPre {
-  T mat[4][kWideSP * kWideLD];   // P_i, P_j, dP_i, dP_j for one r
-  T vin[2][WideCfg<T>::CT * kWideSP];
-  T qk[WideCfg<T>::CT * kWideSP];
-  T av[2][WideCfg<T>::CT * kWideSP];
-  int ys[2][WideCfg<T>::CT];
-  T redm[2][WideCfg<T>::CT][kWideThreads / 32];
-  typename Acc<T>::type red[kWideThreads / 32][2];
-  T redg[3][WideCfg<T>::CT][kWideThreads / 32];
-};
-
-template <typename T>
-__global__ void __launch_bounds__(kWideThreads) pre_wide_kernel(LevelArgs<T> a) {
-  pdl_wait_and_release();
-  constexpr int CT = WideCfg<T>::CT;
-  constexpr int NT = kWideThreads;
-  constexpr int GROUPS = NT / kWideSP;
-  constexpr int CPG = CT / GROUPS;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  WideSmemPre<T>& sm = *reinterpret_cast<WideSmemPre<T>*>(smraw);
-  T* qout = reinterpret_cast<T*>(smraw + sizeof(WideSmemPre<T>));  // [2][R][CT][SP]
-  const int k = a.level_nodes[blockIdx.y];
-  const int2 ch = a.children[k];
-  const int R = a.n_cat, C = a.n_patterns, S = a.n_states;
-  const int c0 = blockIdx.x * CT;
-  const int g = threadIdx.x / kWideSP, s = threadIdx.x % kWideSP;
-  const bool int_i = ch.x >= a.n_tips, int_j = ch.y >= a.n_tips;
-  T ni[CPG], nj[CPG], dd[CPG];
-#pragma unroll
-  for (int jj = 0; jj < CPG; ++jj) { ni[jj] = T(0); nj[jj] = T(0); dd[jj] = T(0); }
-  for (int r = 0; r < R; ++r) {
-    __syncthreads();
-    stage_mat_padded<T>(a.P + ((size_t)ch.x * R + r) * kWideSP * kWideSP, sm.mat[0]);
-    stage_mat_padded<T>(a.P + ((size_t)ch.y * R + r) * kWideSP * kWideSP, sm.mat[1]);
-    stage_mat_padded<T>(a.dP + ((size_t)ch.x * R + r) * kWideSP * kWideSP, sm.mat[2]);
-    stage_mat_padded<T>(a.dP + ((size_t)ch.y * R + r) * kWideSP * kWideSP, sm.mat[3]);
-    stage_child_vec<T>(a, ch.x, c0, r, sm.vin[0], sm.ys[0]);
-    stage_child_vec<T>(a, ch.y, c0, r, sm.vin[1], sm.ys[1]);
-    for (int idx = threadIdx.x; idx < CT * kWideSP; idx += NT) {
-      const int j = idx / kWideSP, ss = idx % kWideSP, c = c0 + j;
-      T v = T(0);
-      if (c < C) {
-        if (k == a.root) v = ss < S ? (T)a.root_pi[ss] : T(0);
-        else v = a.pre[(((size_t)(k - a.n_tips) * C + c) * R + r) * kWideSP + ss];
-      }
-      sm.qk[idx] = v;
-    }
-    __syncthreads();
-    const T wr = a.cat_wt[r];
-#pragma unroll
-    for (int jj = 0; jj < CPG; ++jj) {
-      const int j = g * CPG + jj;
-      const T ui = wide_up<T>(sm.mat[0], sm.vin[0], sm.ys[0], j, s, S);
-      const T uj = wide_up<T>(sm.mat[1], sm.vin[1], sm.ys[1], j, s, S);
-      const T vi = wide_up_gap_d<T>(sm.ys[0], j, S,
-                                   wide_up<T>(sm.mat[2], sm.vin[0], sm.ys[0], j, s, S));
-      const T vj = wide_up_gap_d<T>(sm.ys[1], j, S,
-                                   wide_up<T>(sm.mat[3], sm.vin[1], sm.ys[1], j, s, S));
-      const T q = sm.qk[j * kWideSP + s];
-      const T ai = q * uj, aj = q * ui;
-      ni[jj] = fma(wr, ai * vi, ni[jj]);
-      nj[jj] = fma(wr, aj * vj, nj[jj]);
-      dd[jj] = fma(wr, ai * ui, dd[jj]);
-      sm.av[0][j * kWideSP + s] = ai;
-      sm.av[1][j * kWideSP + s] = aj;
-    }
-    __syncthreads();
-    // q_child[t = s] = sum_s' P[s'][t] a[s'] for this r (unscaled)
-#pragma unroll
-    for (int jj = 0; jj < CPG; ++jj) {
-      const int j = g * CPG + jj;
-      for (int x = 0; x < 2; ++x) {
-        if (!(x == 0 ? int_i : int_j)) continue;
-        const T* M = sm.mat[x];
-        const T* av = sm.av[x] + j * kWideSP;
-        T acc = T(0);
-#pragma unroll 16
-        for (int sp = 0; sp < kWideSP; ++sp) acc = fma(M[sp * kWideLD + s], av[sp], acc);
-        qout[((x * R + r) * CT + j) * kWideSP + s] = acc;
-      }
-    }
-  }
-  // Gradient ratio per pattern: reduce ni, nj, dd over the group's 64 states.
-  const int warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int jj = 0; jj < CPG; ++jj) {
-    const int j = g * CPG + jj;
-    T x0 = ni[jj], x1 = nj[jj], x2 = dd[jj];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      x0 += __shfl_xor_sync(kFull, x0, o);
-      x1 += __shfl_xor_sync(kFull, x1, o);
-      x2 += __shfl_xor_sync(kFull, x2, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      sm.redg[0][j][warp] = x0; sm.redg[1][j][warp] = x1; sm.redg[2][j][warp] = x2;
-    }
-  }
-  // Max of each child's unscaled q over (r, s) per pattern.
-  __syncthreads();
-#pragma unroll
-  for (int jj = 0; jj < CPG; ++jj) {
-    const int j = g * CPG + jj;
-    for (int x = 0; x < 2; ++x) {
-      T m = T(0);
-      if (x == 0 ? int_i : int_j)
-        for (int r = 0; r < R; ++r)
-          m = tmax(m, fabs(qout[((x * R + r) * CT + j) * kWideSP + s]));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = tmax(m, __shfl_xor_sync(kFull, m, o));
-      if ((threadIdx.x & 31) == 0) sm.redm[x][j][warp] = m;
-    }
-  }
-  __syncthreads();
-  using A = Acc<T>;
-  typename A::type gi = A::zero(), gj = A::zero();
-#pragma unroll
-  for (int jj = 0; jj < CPG; ++jj) {
-    const int j = g * CPG + jj, c = c0 + j;
-    if (c >= C) continue;
-    if (s == 0) {
-      const T Ni = sm.redg[0][j][2 * g] + sm.redg[0][j][2 * g + 1];
-      const T Nj = sm.redg[1][j][2 * g] + sm.redg[1][j][2 * g + 1];
-      const T D = sm.redg[2][j][2 * g] + sm.redg[2][j][2 * g + 1];
-      if (!(D > T(0)) || !isfinite(D)) {
-        atomicOr(a.err, ERR_BAD_RATIO);
-      } else {
-        gi = A::add(gi, A::prod(a.pattern_wt[c], Ni / D));
-        gj = A::add(gj, A::prod(a.pattern_wt[c], Nj / D));
-      }
-    }
-    for (int x = 0; x < 2; ++x) {
-      const int b = x == 0 ? ch.x : ch.y;
-      if (b < a.n_tips) continue;
-      const T m = tmax(sm.redm[x][j][2 * g], sm.redm[x][j][2 * g + 1]);
-      int e = 0;
-      if (!(m > T(0)) || !isfinite(m)) atomicOr(a.err, ERR_ZERO_PARTIAL);
-      else (void)frexp(m, &e);
-      const T f = ldexp(T(1), -e);
-      const size_t slot = (size_t)(b - a.n_tips);
-      for (int r = 0; r < R; ++r)
-        a.pre[((slot * C + c) * R + r) * kWideSP + s] =
-            qout[((x * R + r) * CT + j) * kWideSP + s] * f;
-    }
-  }
-  __syncthreads();
-  block_sum_acc<T, NT>(gi, gj, sm.red, 1);
-  if (threadIdx.x == 0) {
-    a.gpart[(size_t)ch.x * a.n_tiles + blockIdx.x] = A::to_double(gi);
-    a.gpart[(size_t)ch.y * a.n_tiles + blockIdx.x] = A::to_double(gj);
-  }
-}
-
-template <typename T>
-inline size_t wide_post_smem() { return sizeof(WideSmemPost<T>); }
-template <typename T>
-inline size_t wide_pre_smem(int R) {
-  return sizeof(WideSmemPre<T>) +
-         (size_t)2 * R * WideCfg<T>::CT * kWideSP * sizeof(T);
-}
-
 }  // namespace phylo
 
 #include "kernels_p4.cuh"
 #include "kernels_tree.cuh"
 #include "kernels_tc64.cuh"
+#include "kernels_tcd.cuh"
 #include "kernels_big.cuh"
 #include "kernels_tcb.cuh"
 
@@ -1511,11 +1158,7 @@ cudaError_t launch_level_impl(const LevelArgs<T>& a, int SP, int RP, bool post,
       if constexpr (std::is_same<T, float>::value) {
         return launch_tc64(a, post, st);
       } else {
-        dim3 grid(a.n_tiles, a.n_level);
-        if (post)
-          return launch_pdl(post_wide_kernel<T>, grid, kWideThreads, wide_post_smem<T>(), st, a);
-        return launch_pdl(pre_wide_kernel<T>, grid, kWideThreads, wide_pre_smem<T>(a.n_cat), st,
-                          a);
+        return launch_tcd(a, post, st);
       }
     case 128:
       if constexpr (std::is_same<T, float>::value) return launch_tcb(a, post, st);
@@ -1533,13 +1176,7 @@ cudaError_t prepare_impl(int SP, int RP) {
     if constexpr (std::is_same<T, float>::value) {
       return prepare_tc64();
     } else {
-      cudaError_t e = cudaFuncSetAttribute(
-          post_wide_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-          (int)wide_post_smem<T>());
-      if (e != cudaSuccess) return e;
-      return cudaFuncSetAttribute(pre_wide_kernel<T>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)wide_pre_smem<T>(8));
+      return prepare_tcd();
     }
   }
   if (SP == 128) {
@@ -1569,7 +1206,7 @@ cudaError_t launch_pmat_impl(const PmatArgs& a, int SP, cudaStream_t st) {
       break;
     case 64:
       if constexpr (std::is_same<T, float>::value) return launch_pmat_tc64(a, st);
-      else pmat_kernel<T, 64><<<units, 256, 0, st>>>(a);
+      else return launch_pmat_tcd(a, st);
       break;
     case 128:
       if constexpr (std::is_same<T, float>::value) return launch_pmat_tcb(a, st);
@@ -1588,6 +1225,8 @@ template <typename T>
 cudaError_t launch_pre_finish_impl(const LevelArgs<T>& a, int SP, cudaStream_t st) {
   if constexpr (std::is_same<T, float>::value) {
     if (SP == 64 || SP == 128) return launch_ratio_tc64(a, st);
+  } else if (SP == 64) {
+    return launch_ratio_tcd(a, st);
   }
   return cudaSuccess;
 }

@@ -47,7 +47,8 @@ struct Layout {
   Region pattern_w, V, Vinv, lambda, pi, rates, cat_w, t;
   Region vsplit;  // tensor-core path: eigenvectors as double-float tables
   Region tc_tiles;  // 65..128 states, FP32: pre-split matrix blocks
-  Region qt;        // 21..128 states, FP32: Q' as a tensor-core operand
+  Region qt;        // 21..128 states, FP32, and 21..64, FP64: Q' as a tensor-core operand
+  Region vdigits;   // 21..64 states, FP64: the digits of Vinv'
   Region qmat;      // 4 and 20 padded states, FP32: Q row-major
   Region tip_desc;  // U-form paths with tip partials: descriptors of the tips
                     // whose U = P p the first post-order launch forms
@@ -91,7 +92,9 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
   size_t mat, part, tmp, tmp2;
   const bool tc = uses_tensor_cores(L.SP, prec == PHYLO_FP64);
   const bool p4 = uses_tr_layout(L.SP, prec == PHYLO_FP64);
+  const bool tcd = uses_tcd(L.SP, prec == PHYLO_FP64);
   const size_t unit = tc ? kTcUnitBytes
+                      : tcd ? kTcdUnitBytes
                          : (size_t)L.SP * L.SP * L.elem * (p4 ? kP4MatKinds : 1);
   if (!mul_ok(n_br * R, unit, &mat)) return "size overflow";
   if (C > (1 << 30)) return "n_patterns too large";
@@ -109,7 +112,7 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
     ok &= add_region(L, L.pre_off, (n_int + 1) * sizeof(int));
   }
   ok &= add_region(L, L.P, mat);
-  ok &= add_region(L, L.dP, tc || p4 ? 0 : mat);  // else the P region holds dP
+  ok &= add_region(L, L.dP, tc || tcd || p4 ? 0 : mat);  // else the P region holds dP
   if (uses_tc_big(L.SP, prec == PHYLO_FP64)) {
     // the matrix kernel writes the operand blocks instead of P and dP
     L.P.bytes = L.dP.bytes = 0;
@@ -129,6 +132,10 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
   }
   ok &= add_region(L, L.pre, L.mode == kWalk ? 0 : part);
   if (tc || uses_tc_big(L.SP, prec == PHYLO_FP64)) ok &= add_region(L, L.qt, qt_bytes(L.SP));
+  if (tcd) {
+    ok &= add_region(L, L.qt, kTcdModelBytes);
+    ok &= add_region(L, L.vdigits, kTcdModelBytes);
+  }
   if (uses_tr_layout(L.SP, prec == PHYLO_FP64))  // the U form's Q (row-major)
     ok &= add_region(L, L.qmat, (size_t)L.SP * L.SP * L.elem);
   if (C > (1 << 30)) return "n_patterns too large";
@@ -138,7 +145,7 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
   ok &= add_region(L, L.escale, tmp);
   if (uses_tc_terms(L.SP, prec == PHYLO_FP64)) {
     ok &= add_region(L, L.pre_escale, tmp);
-    if (!mul_ok(n_int * C, (size_t)R * 16, &tmp)) return "size overflow";
+    if (!mul_ok(n_int * C, (size_t)R * (tcd ? 32 : 16), &tmp)) return "size overflow";
     ok &= add_region(L, L.rterm, tmp);
   }
   if (!mul_ok((size_t)N, (size_t)tip_state_stride(C), &tmp)) return "size overflow";
@@ -388,6 +395,8 @@ cudaError_t enqueue_phase(phylo_ctx* ctx, int phase, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     PmatArgs pa{};
     pa.vsplit = ctx->L.vsplit.bytes ? ctx->dev<float>(ctx->L.vsplit) : nullptr;
+    pa.vdigits = ctx->L.vdigits.bytes ? ctx->dev<void>(ctx->L.vdigits) : nullptr;
+    pa.n_tips = ctx->N;
     pa.reversible = ctx->eig_reversible;
     pa.V = ctx->dev<double>(ctx->L.V);
     pa.Vinv = ctx->dev<double>(ctx->L.Vinv);
@@ -1055,7 +1064,17 @@ int phylo_set_eigen(phylo_ctx* ctx, const double* V, const double* Vinv,
     if ((rc = upload_typed(ctx, ctx->L.qmat, qm.data(), qm.size(), "upload Q"))) return rc;
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
   }
-  if (ctx->L.qt.bytes) {
+  if (ctx->L.vdigits.bytes) {
+    std::vector<double> q((size_t)S * S);  // Q, row-major
+    build_q_matrix(S, S, V, Vinv, lambda, q.data());
+    std::vector<unsigned char> tile(kTcdModelBytes);
+    build_digits(S, [&](int n, int k) { return q[(size_t)k * S + n]; }, tile.data());
+    if ((rc = upload(ctx, ctx->L.qt, tile.data(), tile.size(), "upload Q operand"))) return rc;
+    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+    build_digits(S, [&](int n, int k) { return Vinv[(size_t)k * S + n]; }, tile.data());
+    if ((rc = upload(ctx, ctx->L.vdigits, tile.data(), tile.size(), "upload V operand"))) return rc;
+    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+  } else if (ctx->L.qt.bytes) {
     std::vector<unsigned char> qt(qt_bytes(ctx->L.SP));
     build_qt_tile(S, ctx->L.SP, V, Vinv, lambda, qt.data());
     if ((rc = upload(ctx, ctx->L.qt, qt.data(), qt.size(), "upload Q operand"))) return rc;

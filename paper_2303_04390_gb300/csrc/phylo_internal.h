@@ -2,6 +2,7 @@
 // translation units (kernels_fp32.cu, kernels_fp64.cu).  Not installed.
 #pragma once
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 #include <cstring>
@@ -44,10 +45,6 @@ inline int lanes_per_pattern(int R) {
 
 // Threads per block of the register kernels (one thread per (pattern, r)).
 constexpr int kSmallThreads = 128;
-// Patterns per block of the shared-memory kernels for S_pad = 64.
-constexpr int kWideThreads = 256;
-constexpr int kWidePatternsF32 = 16;
-constexpr int kWidePatternsF64 = 8;
 // Patterns per block of the kernels for S_pad = 128 and 256 (kernels_big.cuh).
 constexpr int kBigPatternsF32 = 16;
 constexpr int kBigPatternsF64 = 8;
@@ -137,6 +134,46 @@ constexpr int kTcTilePatterns = 128;
 constexpr size_t kTcUnitBytes = 65536;
 constexpr size_t kTcQtBytes = 3 * 64 * 128;
 
+// FP64 with 21..64 states runs on the tensor cores as well, in exact integer
+// arithmetic on base-256 digits (kernels_tcd.cuh): per (branch, category) an
+// internal branch's P and P' as eight-digit operands and the exponents of the
+// rows of P', a tip's P' and dP' in FP64.
+inline bool uses_tcd(int SP, bool fp64) { return SP == 64 && fp64; }
+constexpr uint32_t kTcdDigits = 8 * 64 * 128;           // one 64 x 64 operand
+constexpr size_t kTcdUnitBytes = 2 * (size_t)kTcdDigits + 64 * sizeof(int);
+constexpr size_t kTcdModelBytes = kTcdDigits + 64 * sizeof(int);
+
+// The digits of a 64 x 64 operand with rows M(n, k), n, k < S (zero beyond),
+// row n scaled by 2^-e_n to magnitudes below 1: digit i of element (n, k) of
+// round(M 2^(62 - e_n)) = sum_i a_i 256^(7 - i) as an FP16 integer in slice i
+// (8 KB), K-major 128-byte swizzle; then e_n as 64 ints.  out: kTcdModelBytes.
+template <typename F>
+inline void build_digits(int S, F M, unsigned char* out) {
+  std::memset(out, 0, kTcdModelBytes);
+  for (int n = 0; n < S; ++n) {
+    double mx = 0.0;
+    for (int k = 0; k < S; ++k) mx = std::fmax(mx, std::fabs(M(n, k)));
+    int e = 0;
+    (void)std::frexp(mx, &e);
+    std::memcpy(out + kTcdDigits + n * sizeof(int), &e, sizeof(int));
+    for (int k = 0; k < S; ++k) {
+      const long long v = std::llrint(std::ldexp(M(n, k), 62 - e));
+      const uint64_t t = (uint64_t)v + 0x8080808080808080ull;
+      for (int i = 0; i < 8; ++i) {
+        const int digit = (int)(t >> (56 - 8 * i) & 0xff) - 128;
+        uint16_t h = 0;  // FP16 of an integer below 2^11
+        if (digit) {
+          int ex;
+          const double f = std::frexp(std::fabs((double)digit), &ex);
+          h = (uint16_t)((digit < 0 ? 0x8000 : 0) + ((ex + 13) << 10) + (int)(f * 2048.0));
+        }
+        const size_t off = (size_t)n * 128 + ((size_t)((k >> 3) ^ (n & 7)) << 4) + (k & 7) * 2;
+        std::memcpy(out + (size_t)i * 64 * 128 + off, &h, 2);
+      }
+    }
+  }
+}
+
 // Round-to-nearest-even BF16 of a finite float, and back (host side).
 inline uint16_t host_bf16(float x) {
   uint32_t u;
@@ -225,7 +262,7 @@ __host__ __device__ constexpr size_t tcb_block(int kind, int jn, int jk) {
 // Paths with per-category exponents and Eq. 8 terms combined by the ratio
 // kernel (both tensor-core paths).
 inline bool uses_tc_terms(int SP, bool fp64) {
-  return uses_tensor_cores(SP, fp64) || uses_tc_big(SP, fp64);
+  return uses_tensor_cores(SP, fp64) || uses_tc_big(SP, fp64) || uses_tcd(SP, fp64);
 }
 
 // The eigenvectors as double-float pairs for the tensor-core path's matrix
@@ -278,8 +315,7 @@ inline int patterns_per_tile(int SP, int R, bool fp64, PassMode mode = kByLevel)
   if (SP == 4 && !fp64) return kP4TilePatterns;
   if (uses_tc_terms(SP, fp64)) return kTcTilePatterns;
   if (SP <= 20) return kSmallThreads / lanes_per_pattern(R);
-  if (SP >= 128) return fp64 ? kBigPatternsF64 : kBigPatternsF32;
-  return fp64 ? kWidePatternsF64 : kWidePatternsF32;
+  return fp64 ? kBigPatternsF64 : kBigPatternsF32;
 }
 
 // Partial-vector elements stored per node.  Tile-blocked paths pad the
@@ -339,7 +375,7 @@ struct LevelArgs {
   int* err;                    // numeric flags
   const unsigned char* tc_tiles;  // 65..128 states, FP32: the pre-split matrix
                                   // blocks [2N-2][R][kTcbUnitBytes] (else null)
-  const unsigned char* qt;     // 21..64 states, FP32: Q' operand (kTcQtBytes)
+  const unsigned char* qt;     // 21..128 states: Q' operand (FP64: kTcdModelBytes)
   const T* qmat;               // 4 and 20 padded states, U form: Q row-major [SP][SP]
   const double* rates;         // [R] category rates gamma_r
   int tip_level;               // U-form paths: the level's nodes are tips with
@@ -376,6 +412,8 @@ struct TreePass {
 
 struct PmatArgs {
   const float* vsplit;   // tensor-core path: build_eigen_split's table
+  const void* vdigits;   // FP64, 21..64 states: the digits of Vinv' (build_digits)
+  int n_tips;
   int reversible;        // tensor-core path: the table's decomposition is symmetric
   const double* V;       // [S][S]
   const double* Vinv;    // [S][S]
