@@ -1224,7 +1224,8 @@ cudaError_t launch_pmat_impl(const PmatArgs& a, int SP, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_pre_finish_impl(const LevelArgs<T>& a, int SP, cudaStream_t st) {
   if constexpr (std::is_same<T, float>::value) {
-    if (SP == 64 || SP == 128) return launch_ratio_tc64(a, st);
+    if (SP == 64) return launch_ratio_tc64<64>(a, st);
+    if (SP == 128) return launch_ratio_tc64<128>(a, st);
   } else if (SP == 64) {
     return launch_ratio_tcd(a, st);
   }

@@ -85,6 +85,7 @@ constexpr size_t kPostUSmem = 1024 + kOp128 + kOp64;
 #endif
 // FP32 P' of one (branch, r): the compact-tip lookup table, staged by bulk copy.
 constexpr uint32_t kPt32Bytes = 64 * 64 * 4;
+constexpr size_t kTipqSmem = 1024 + kOp128 + kOp64;
 constexpr size_t kPreUSmem = 1024 + kOp128 + 2 * kOp64;
 
 __device__ __forceinline__ float pow2i(int d) {  // 2^d for d <= 0 (0 below 2^-126)
@@ -418,6 +419,78 @@ __global__ void __launch_bounds__(kPmatTcThreads) pmat_tc_kernel(PmatArgs a) {
 }
 
 // ---------------------------------------------------------------------------
+// Tables of the compact tips: G = Q P per (tip, category), stored by columns
+// (row y of G' = column y), FP32, in place of the tip's operand P, which only
+// tips with partial vectors use.  A tip's Eq. 8 numerator a' dP e_y =
+// gamma_r a . (G e_y) is then a lookup in its sibling's pre-order unit instead
+// of a contraction per pattern tile.  Two units (64 rows each) per CTA.
+// ---------------------------------------------------------------------------
+template <typename T>  // float only
+__global__ void __launch_bounds__(kTcThreads) tipq_tc_kernel(PmatArgs a) {
+  static_assert(std::is_same<T, float>::value, "tensor-core path is FP32");
+  extern __shared__ unsigned char smraw[];
+  unsigned char* A = align1024(smraw);
+  unsigned char* B = A + kOp128;
+  __shared__ uint64_t bar_tma, bar_mma;
+  __shared__ uint32_t tmem_slot;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int row = tid & (kTcRows - 1), h = tid / kTcRows;
+  const int R = a.n_cat, units = a.n_tips * R, u0 = 2 * blockIdx.x;
+  unsigned char* base = static_cast<unsigned char*>(a.P);
+  pdl_wait_and_release();
+  if (tid == 0) {
+    mbar_init_fenced(&bar_tma, 1);
+    mbar_init_fenced(&bar_mma, 1);
+    const int n = min(2, units - u0);  // (rows of a missing unit are not read back)
+    mbar_expect_tx(&bar_tma, kOp64 + n * kOp64);
+    bulk_g2s(B, a.qn, kOp64, &bar_tma);
+    for (int u = 0; u < n; ++u)
+      for (int t = 0; t < 3; ++t)
+        bulk_g2s(A + t * kTerm128 + u * kTerm64,
+                 base + (size_t)(u0 + u) * kTcUnitBytes + kUnitPt + t * kTerm64, kTerm64,
+                 &bar_tma);
+  }
+  if (warp == 0) tc::alloc(&tmem_slot, 64);
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = tmem_slot;
+  uint32_t ptma = 0, pmma = 0;
+  int pend_tma = -1, pend_mma = -1;
+  bool ok = tc_block_wait(&bar_tma, ptma, pend_tma, a.err);
+  if (ok) {
+    if (tid == 0) {
+      tc::fence_after();
+      uint32_t ta[3], tb[3];
+      term_addrs(A, kTerm128, ta);
+      term_addrs(B, kTerm64, tb);
+      tc::mma_split_bf16x3<64>(tmem, ta, tb);
+      tc::commit(&bar_mma);
+    }
+    ok = tc_block_wait(&bar_mma, pmma, pend_mma, a.err);
+  }
+  if (ok) {
+    float w[32];
+    tc::ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + 32 * h, w);
+    const int unit = u0 + (row >> 6);
+    if (unit < units && !(a.tip_has && a.tip_has[unit / R])) {
+      float4* out = reinterpret_cast<float4*>(
+          reinterpret_cast<float*>(base + (size_t)unit * kTcUnitBytes + kUnitP) +
+          (row & 63) * 64 + 32 * h);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        out[i] = make_float4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+    }
+  }
+  if (tid == 0) {
+    if (pend_tma >= 0) (void)mbar_wait(&bar_tma, (uint32_t)pend_tma);
+    if (pend_mma >= 0) (void)mbar_wait(&bar_mma, (uint32_t)pend_mma);
+  }
+  tc::fence_before();
+  __syncthreads();
+  if (warp == 0) tc::dealloc(tmem, 64);
+}
+
+// ---------------------------------------------------------------------------
 // Stored U rows and their exponents
 // ---------------------------------------------------------------------------
 // U slot of node x: internal nodes in slot x - N, tips with partial
@@ -715,13 +788,17 @@ __global__ void __launch_bounds__(kTcRows) root_u_kernel(LevelArgs<T> a) {
 
 // ---------------------------------------------------------------------------
 // Pre-order level (Eq. 4) with the per-category Eq. 8 terms: one CTA per
-// (tile, node k, category r, child x); blockIdx.z = 2 r + x.
+// (tile, unit, category).  A unit (pre_units) is a node k with a child x to
+// contract; a compact tip's numerator needs no contraction, a_y . (G_y e) with
+// a_y = q_k o U_x, so it is formed in its sibling's unit from the rows loaded
+// there.  Against one CTA per child, with a contraction W_x = a_x Q for tips
+// too, that is half as many CTAs.
 // ---------------------------------------------------------------------------
 template <typename T>  // float only
 __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
   static_assert(std::is_same<T, float>::value, "tensor-core path is FP32");
   static_assert(kStageBytes <= kOp128 && kStageBytes <= 2 * kOp64, "staging fits");
-  static_assert(kPt32Bytes <= kOp64, "a lookup table fits in the P' buffer");
+  static_assert(2 * kPt32Bytes <= kOp128, "the sibling's tables fit in the operand buffer");
   extern __shared__ unsigned char smraw[];
   unsigned char* base = align1024(smraw);
   unsigned char* A = base;                     // a_x as three BF16 terms
@@ -729,22 +806,21 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
   unsigned char* Bq = base + kOp128 + kOp64;   // Q' (rows = columns of Q)
   float* stW = reinterpret_cast<float*>(A);    // W_x rows, after the MMAs
   float* stQ = reinterpret_cast<float*>(Bp);   // q_x rows, after the MMAs
-  // lookup tables of compact children (FP32 P'): the sibling's in A until
-  // the split, the child's own in Bp (unused by a tip child's MMA)
-  const float* pt32x = reinterpret_cast<const float*>(Bp);
+  // a compact sibling's tables (columns of P and of G = Q P, FP32) in A until
+  // the split
   const float* pt32y = reinterpret_cast<const float*>(A);
+  const float* gy = reinterpret_cast<const float*>(A + kPt32Bytes);
   __shared__ uint64_t bar_tma, bar_mma;
   __shared__ uint32_t tmem_slot;
   __shared__ int eexp[kTcRows];      // each row's rescale exponent of q_x
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, j = lane & 7;
   const int row = tid & (kTcRows - 1), h = tid / kTcRows;
   const int R = a.n_cat, C = a.n_patterns, S = a.n_states;
-  const int4 d = a.level_desc[blockIdx.y];
-  const int k = d.x, x = (int)(blockIdx.z & 1), r = (int)(blockIdx.z >> 1);
-  const TcChild cx = tc_child(a.n_tips, x ? d.z : d.y,
-                              d.w & (x ? kDescFlagCompact1 : kDescFlagCompact0));
-  const TcChild cy = tc_child(a.n_tips, x ? d.y : d.z,
-                              d.w & (x ? kDescFlagCompact0 : kDescFlagCompact1));
+  const int4 d = a.level_desc[blockIdx.z];
+  const int k = d.x, r = (int)blockIdx.y;
+  const int x = (d.w & kUnitSecond) ? 1 : 0;  // x's place among k's children
+  const TcChild cx = tc_child(a.n_tips, d.y, false);
+  const TcChild cy = tc_child(a.n_tips, d.z, d.w & kUnitCompactY);
   const bool root = k == a.root;
   const size_t kslot = (size_t)(k - a.n_tips);
   const int c0 = blockIdx.x * kTcRows;
@@ -757,13 +833,13 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
     mbar_init_fenced(&bar_tma, 1);
     mbar_init_fenced(&bar_mma, 1);
     mbar_expect_tx(&bar_tma, kOp64 + (cx.internal ? kOp64 : 0) +
-                                 (cx.compact ? kPt32Bytes : 0) + (cy.compact ? kPt32Bytes : 0));
+                                 (cy.compact ? 2 * kPt32Bytes : 0));
     bulk_g2s(Bq, a.qt, kOp64, &bar_tma);
     if (cx.internal) bulk_g2s(Bp, unit_tiles(a, cx.b, r) + kUnitPt, kOp64, &bar_tma);
-    if (cx.compact)
-      bulk_g2s(Bp, unit_tiles(a, cx.b, r) + kUnitPt32, kPt32Bytes, &bar_tma);
-    if (cy.compact)
+    if (cy.compact) {
       bulk_g2s(A, unit_tiles(a, cy.b, r) + kUnitPt32, kPt32Bytes, &bar_tma);
+      bulk_g2s(A + kPt32Bytes, unit_tiles(a, cy.b, r) + kUnitP, kPt32Bytes, &bar_tma);
+    }
   };
   const double cw = a.cat_w[r], rate = a.rates[r];  // used in the epilogue
   const float wr = a.cat_wt[r];
@@ -807,16 +883,25 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
   uint32_t ptma = 0, pmma = 0;
   int pend_tma = -1, pend_mma = -1;
   bool ok = tc_block_wait(&bar_tma, ptma, pend_tma, a.err);
-  float den[4];
+  const float wg = (float)(cw * rate);
+  float* rt = reinterpret_cast<float*>(a.rterm);
+  float den[4], ny[4];  // this lane's parts of the rows' sums
   if (ok) {
-    coop_child_u_finish(fx, cx.compact, pt32x, S);
     coop_child_u_finish(fy, cy.compact, pt32y, S);
-    // a_x = q_k o U_y (into q) and den = a_x . U_x per row
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
+      // a_y = q_k o U_x: den = a_y . U_y and a tip sibling's numerator;
+      // then a_x = q_k o U_y (into q)
+      const float4 b0 = mul4(q[2 * it], fx.v[2 * it]), b1 = mul4(q[2 * it + 1], fx.v[2 * it + 1]);
+      den[it] = dot4(b1, fy.v[2 * it + 1], dot4(b0, fy.v[2 * it], 0.f));
+      ny[it] = 0.f;
+      const int y = fy.y[it];
+      if (cy.compact && y >= 0 && y < S) {
+        const float4* g = reinterpret_cast<const float4*>(gy + y * 64 + 8 * j);
+        ny[it] = dot4(b1, g[1], dot4(b0, g[0], 0.f));
+      }
       q[2 * it] = mul4(q[2 * it], fy.v[2 * it]);
       q[2 * it + 1] = mul4(q[2 * it + 1], fy.v[2 * it + 1]);
-      den[it] = row_sum8(dot4(q[2 * it + 1], fx.v[2 * it + 1], dot4(q[2 * it], fx.v[2 * it], 0.f)));
     }
     __syncthreads();  // every lookup in A is done before the split overwrites it
     coop_put(A, q);
@@ -833,6 +918,22 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
         tc::mma_split_bf16x3<64>(tmem, ta, tb);
       }
       tc::commit(&bar_mma);
+    }
+    // the Eq. 8 terms that need no contraction, during the MMAs
+    if (d.w & (kUnitDen | kUnitCompactY)) {
+#pragma unroll
+      for (int it = 0; it < 4; ++it) {
+        const float dn = row_sum8(den[it]), nn = row_sum8(ny[it]);
+        const int c = c0 + coop_row(it);
+        if (c < C && j == 0) {
+          float* t4 = rt + ((kslot * C + c) * R + r) * 4;
+          if (cy.compact) t4[1 - x] = wg * nn;
+          if (d.w & kUnitDen) {
+            t4[2] = wr * dn;
+            t4[3] = __int_as_float(eq[it] + fx.E[it] + fy.E[it]);
+          }
+        }
+      }
     }
     ok = tc_block_wait(&bar_mma, pmma, pend_mma, a.err);
   }
@@ -864,22 +965,14 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
     }
     __syncthreads();
     // num_x = W_x . U_x per row; the Eq. 8 terms of this category
-    const float wg = (float)(cw * rate);
-    float* rt = reinterpret_cast<float*>(a.rterm);
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
       const int rr = coop_row(it), c = c0 + rr;
       const float4 w0 = *reinterpret_cast<const float4*>(stW + rr * kStageLd + 8 * j);
       const float4 w1 = *reinterpret_cast<const float4*>(stW + rr * kStageLd + 8 * j + 4);
-      float num = row_sum8(dot4(w1, fx.v[2 * it + 1], dot4(w0, fx.v[2 * it], 0.f)));
-      if (cx.compact && fx.y[it] >= S) num = 0.f;  // d/dt of the all-ones vector is 0
+      const float num = row_sum8(dot4(w1, fx.v[2 * it + 1], dot4(w0, fx.v[2 * it], 0.f)));
       if (c < C && j == 0) {
-        float* t4 = rt + ((kslot * C + c) * R + r) * 4;
-        t4[x] = wg * num;
-        if (x == 0) {
-          t4[2] = wr * den[it];
-          t4[3] = __int_as_float(eq[it] + fx.E[it] + fy.E[it]);
-        }
+        rt[((kslot * C + c) * R + r) * 4 + x] = wg * num;
         if (cx.internal)  // q_x = P_x' (q_k o U_y): exponents of q_k and of U_y
           a.pre_escale[((size_t)(cx.b - a.n_tips) * R + r) * estr + c] =
               eexp[rr] + eq[it] + fy.E[it];
@@ -897,6 +990,84 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
   __syncthreads();
   if (warp == 0) tc::dealloc(tmem, 128);
 }
+
+// ---------------------------------------------------------------------------
+// Nodes whose children are both compact tips: the Eq. 8 terms from the tips'
+// columns of P and of G = Q P, after the last level.  One block per (tile,
+// node, category), cooperative layout, the tables read through L1.
+//   Cols: (a, b, r, y, kb, j, lo, hi) gives entries 64 kb + 8 j .. + 7 of
+//   column y; col<false> of P (a gap: ones), col<true> of G (a gap: zeros).
+// ---------------------------------------------------------------------------
+template <int SP, class Cols>
+__global__ void __launch_bounds__(kTcThreads) cherry_kernel(LevelArgs<float> a) {
+  pdl_wait_and_release();
+  const int R = a.n_cat, C = a.n_patterns, S = a.n_states, j = threadIdx.x & 7;
+  const int4 d = a.level_desc[blockIdx.z];
+  const int k = d.x, r = (int)blockIdx.y, c0 = blockIdx.x * kTcRows;
+  const bool root = k == a.root;
+  const size_t kslot = (size_t)(k - a.n_tips);
+  const float wg = (float)(a.cat_w[r] * a.rates[r]), wr = a.cat_wt[r];
+#pragma unroll
+  for (int it = 0; it < 4; ++it) {
+    const int c = c0 + coop_row(it);
+    const bool on = c < C;
+    const size_t row = (kslot * C + (on ? c : 0)) * R + r;
+    const int yi = on ? (int)a.tip_states[(size_t)d.y * a.state_stride + c] : -1;
+    const int yj = on ? (int)a.tip_states[(size_t)d.z * a.state_stride + c] : -1;
+    float den = 0.f, ni = 0.f, nj = 0.f;
+#pragma unroll
+    for (int kb = 0; kb < SP / 64; ++kb) {
+      float4 q0, q1, u0, u1, v0, v1, g0, g1;
+      if (root) {
+        const int s = 64 * kb + 8 * j;
+        float p[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) p[i] = s + i < S ? a.root_pit[s + i] : 0.f;
+        q0 = make_float4(p[0], p[1], p[2], p[3]);
+        q1 = make_float4(p[4], p[5], p[6], p[7]);
+      } else {
+        const float4* src = reinterpret_cast<const float4*>(a.pre + row * SP + 64 * kb + 8 * j);
+        q0 = __ldg(src);
+        q1 = __ldg(src + 1);
+      }
+      Cols::template col<false>(a, d.y, r, yi, kb, j, u0, u1);
+      Cols::template col<false>(a, d.z, r, yj, kb, j, v0, v1);
+      const float4 b0 = mul4(q0, u0), b1 = mul4(q1, u1);  // a_j = q_k o U_i
+      den = dot4(b1, v1, dot4(b0, v0, den));
+      Cols::template col<true>(a, d.z, r, yj, kb, j, g0, g1);
+      nj = dot4(b1, g1, dot4(b0, g0, nj));
+      Cols::template col<true>(a, d.y, r, yi, kb, j, g0, g1);
+      ni = dot4(mul4(q1, v1), g1, dot4(mul4(q0, v0), g0, ni));
+    }
+    den = row_sum8(den);
+    ni = row_sum8(ni);
+    nj = row_sum8(nj);
+    if (on && j == 0) {  // (the tips' exponents are 0)
+      const int eq = root ? 0 : a.pre_escale[(kslot * R + r) * a.escale_stride + c];
+      *reinterpret_cast<float4*>(static_cast<float*>(a.rterm) + row * 4) =
+          make_float4(wg * ni, wg * nj, wr * den, __int_as_float(eq));
+    }
+  }
+}
+
+// Ones up to S (a gap's U; zeros for its G and past the last pattern).
+__device__ __forceinline__ void tc_gap8(int s, int S, float g, float4& lo, float4& hi) {
+  lo = make_float4(s < S ? g : 0.f, s + 1 < S ? g : 0.f, s + 2 < S ? g : 0.f, s + 3 < S ? g : 0.f);
+  hi = make_float4(s + 4 < S ? g : 0.f, s + 5 < S ? g : 0.f, s + 6 < S ? g : 0.f,
+                   s + 7 < S ? g : 0.f);
+}
+
+struct Cols64 {
+  template <bool G>
+  __device__ __forceinline__ static void col(const LevelArgs<float>& a, int b, int r, int y, int,
+                                             int j, float4& lo, float4& hi) {
+    if (y < 0 || y >= a.n_states) return tc_gap8(8 * j, a.n_states, !G && y >= 0 ? 1.f : 0.f, lo, hi);
+    const float4* t = reinterpret_cast<const float4*>(unit_tiles(a, b, r) +
+                                                      (G ? kUnitP : kUnitPt32)) + y * 16 + 2 * j;
+    lo = __ldg(t);
+    hi = __ldg(t + 1);
+  }
+};
 
 // ---------------------------------------------------------------------------
 // Eq. 8 ratios and their per-tile sums (Eq. 7) for both children of every
@@ -956,15 +1127,8 @@ inline cudaError_t launch_tc64(const LevelArgs<float>& a, bool post, cudaStream_
   if (post)
     return launch_pdl(post_u_kernel<float>, dim3(a.n_tiles, a.n_level, a.n_cat), kTcThreads,
                       kPostUSmem, st, a);
-  return launch_pdl(pre_u_kernel<float>, dim3(a.n_tiles, a.n_level, 2 * a.n_cat), kTcThreads,
+  return launch_pdl(pre_u_kernel<float>, dim3(a.n_tiles, a.n_cat, a.n_level), kTcThreads,
                     kPreUSmem, st, a);
-}
-
-template <typename T = float>
-inline cudaError_t launch_ratio_tc64(const LevelArgs<float>& a, cudaStream_t st) {
-  if (a.n_tiles <= 0 || a.n_tips < 2) return cudaSuccess;
-  dim3 grid(a.n_tiles, a.n_tips - 1);
-  return launch_pdl(ratio_tc_kernel<float>, grid, kTcRows, 0, st, a);
 }
 
 template <typename T = float>
@@ -973,7 +1137,10 @@ inline cudaError_t launch_pmat_tc64(const PmatArgs& a, cudaStream_t st) {
   if (units <= 0) return cudaSuccess;
   // the reversible form has 136 blocks of (s, t) per unit: 5 warps
   pmat_tc_kernel<float><<<units, a.reversible ? 160 : kPmatTcThreads, kPmatTcSmem, st>>>(a);
-  return cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_pdl(tipq_tc_kernel<float>, dim3((a.n_tips * a.n_cat + 1) / 2), kTcThreads,
+                    kTipqSmem, st, a);
 }
 
 template <typename T = float>
@@ -984,6 +1151,9 @@ inline cudaError_t prepare_tc64() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(pre_u_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kPreUSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(tipq_tc_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kTipqSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(pmat_tc_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kPmatTcSmem);

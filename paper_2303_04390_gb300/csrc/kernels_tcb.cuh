@@ -120,40 +120,20 @@ __device__ __forceinline__ void tcb_child_rows(float4 (&v)[2][8], int (&E)[4], i
     for (int it = 0; it < 4; ++it) tcb_col8(a, x.b, r, y[it], kb, j, v[kb][2 * it], v[kb][2 * it + 1]);
 }
 
-// This thread's half row (states 64 h .. 64 h + 63) of a child's U, for
-// pattern c: stored, or for a compact tip (state y) its column of P.
+// This thread's half row (states 64 h .. 64 h + 63) of a child's stored U, for
+// pattern c.
 __device__ __forceinline__ void tcb_child_half(float (&u)[64], const LevelArgs<float>& a,
-                                               const TcChild& x, int r, int c, int h, int y) {
-  if (c >= a.n_patterns) {
+                                               const TcChild& x, int r, int c, int h) {
+  const bool on = c < a.n_patterns;
+  const float4* src = reinterpret_cast<const float4*>(
+      tcb_u_rows(a, x.b, r) + (size_t)(on ? c : 0) * a.n_cat * kTcbSP + 64 * h);
 #pragma unroll
-    for (int i = 0; i < 64; ++i) u[i] = 0.f;
-    return;
-  }
-  if (!x.compact) {
-    const float4* src = reinterpret_cast<const float4*>(tcb_u_rows(a, x.b, r) +
-                                                        (size_t)c * a.n_cat * kTcbSP + 64 * h);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const float4 f = __ldg(src + i);
-      u[4 * i] = f.x;
-      u[4 * i + 1] = f.y;
-      u[4 * i + 2] = f.z;
-      u[4 * i + 3] = f.w;
-    }
-    return;
-  }
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    float4 lo, hi;
-    tcb_col8(a, x.b, r, y, h, j, lo, hi);
-    u[8 * j] = lo.x;
-    u[8 * j + 1] = lo.y;
-    u[8 * j + 2] = lo.z;
-    u[8 * j + 3] = lo.w;
-    u[8 * j + 4] = hi.x;
-    u[8 * j + 5] = hi.y;
-    u[8 * j + 6] = hi.z;
-    u[8 * j + 7] = hi.w;
+  for (int i = 0; i < 16; ++i) {
+    const float4 f = on ? __ldg(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    u[4 * i] = f.x;
+    u[4 * i + 1] = f.y;
+    u[4 * i + 2] = f.z;
+    u[4 * i + 3] = f.w;
   }
 }
 
@@ -301,6 +281,65 @@ __device__ __forceinline__ bool tcb_rounds(unsigned char* A0, unsigned char* B0,
   for (int i = n >= 2 ? n - 2 : 0; i < n; ++i)
     if (!tcb_wait(bars, ph, 2 + (i & 1), err)) return false;
   return true;
+}
+
+// ---------------------------------------------------------------------------
+// Tables of the compact tips, as on the 64-state path (tipq_tc_kernel): G = Q P
+// of one (tip, category) per CTA, stored by columns in FP32 ([128][128]) in
+// place of the tip's P blocks.
+// ---------------------------------------------------------------------------
+static_assert(kTcbSP * kTcbSP * 4 <= kTcbNB * kTcbNB * kTcbBlock, "a table fits in the P blocks");
+
+template <typename T>  // float only
+__global__ void __launch_bounds__(kTcThreads) tipq_tcb_kernel(PmatArgs a) {
+  static_assert(std::is_same<T, float>::value, "tensor-core path is FP32");
+  pdl_wait_and_release();
+  const int unit = blockIdx.x;
+  if (a.tip_has && a.tip_has[unit / a.n_cat]) return;  // block-uniform
+  TCB_PROLOGUE(128)
+  unsigned char* U = static_cast<unsigned char*>(a.tiles) + (size_t)unit * kTcbUnitBytes;
+  auto round_of = [=, &a](int kb) {
+    return TcbRound{a.qn + tcb_block(0, 0, kb), kb, tmem, kb > 0};
+  };
+  if (tid == 0) {  // A: P' (rows = columns of P), both K-blocks, on round 0's barrier
+    mbar_expect_tx(&bars[0], 2 * kTcbBlock + 2 * kOp128);
+    ph.issue(0);
+    for (int kb = 0; kb < kTcbNB; ++kb)
+      for (int jn = 0; jn < kTcbNB; ++jn)
+        for (int t = 0; t < 3; ++t)
+          bulk_g2s(tcb_a(A0, kb) + t * kTerm128 + jn * kTerm64,
+                   U + tcb_block(1, jn, kb) + t * kTerm64, kTerm64, &bars[0]);
+    bulk_g2s(tcb_b(B0, 0), round_of(0).bsrc, 2 * kTcbBlock, &bars[0]);
+  }
+  tcb_issue_b(B0, bars, ph, 1, round_of(1).bsrc);
+  if (tcb_rounds(A0, B0, bars, ph, kTcbNB, round_of, a.err)) {
+    float* st = reinterpret_cast<float*>(base);  // A is free: every MMA is done
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float w[32];
+      tc::ld32(trow + 64 * h + 32 * q, w);
+#pragma unroll
+      for (int i = 0; i < 32; i += 4)
+        *reinterpret_cast<float4*>(st + row * kTcbLd + 64 * h + 32 * q + i) =
+            make_float4(w[i], w[i + 1], w[i + 2], w[i + 3]);
+    }
+    __syncthreads();
+    tcb_store_rows(reinterpret_cast<float*>(U + tcb_block(0, 0, 0)), kTcbSP, 0, kTcbSP, st);
+  }
+  TCB_EPILOGUE(128)
+}
+
+// Floats 64 kb + 8 j .. + 7 of row y of a tip's table (zeros for a gap or past
+// the last pattern: the derivative of the all-ones vector is 0).
+__device__ __forceinline__ void tcb_gtab8(const LevelArgs<float>& a, int b, int r, int y, int kb,
+                                          int j, float4& lo, float4& hi) {
+  lo = hi = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (y < 0 || y >= a.n_states) return;
+  const float4* g = reinterpret_cast<const float4*>(
+      reinterpret_cast<const float*>(tcb_unit(a, b, r) + tcb_block(0, 0, 0)) + y * kTcbSP +
+      64 * kb + 8 * j);
+  lo = __ldg(g);
+  hi = __ldg(g + 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -456,7 +495,8 @@ __global__ void __launch_bounds__(kTcRows) root_tcb_kernel(LevelArgs<T> a) {
 
 // ---------------------------------------------------------------------------
 // Pre-order level (Eq. 4) with the per-category Eq. 8 terms: one CTA per
-// (tile, node k, category r, child x); blockIdx.z = 2 r + x.
+// (tile, unit (pre_units), category): as on the 64-state path, a compact tip's
+// numerator is formed in its sibling's unit from the table G_y.
 // ---------------------------------------------------------------------------
 template <typename T>  // float only
 __global__ void __launch_bounds__(kTcThreads) pre_tcb_kernel(LevelArgs<T> a) {
@@ -465,13 +505,12 @@ __global__ void __launch_bounds__(kTcThreads) pre_tcb_kernel(LevelArgs<T> a) {
   TCB_PROLOGUE(256)
   __shared__ float xn[2][kTcRows], xm[2][kTcRows];  // the halves' num and q maximum
   const int R = a.n_cat, C = a.n_patterns, S = a.n_states;
-  const int4 d = a.level_desc[blockIdx.y];
-  const int k = d.x, x = (int)(blockIdx.z & 1), r = (int)(blockIdx.z >> 1);
+  const int4 d = a.level_desc[blockIdx.z];
+  const int k = d.x, r = (int)blockIdx.y;
+  const int x = (d.w & kUnitSecond) ? 1 : 0;  // x's place among k's children
   const int lane = tid & 31, j = lane & 7;
-  const TcChild cx = tc_child(a.n_tips, x ? d.z : d.y,
-                              d.w & (x ? kDescFlagCompact1 : kDescFlagCompact0));
-  const TcChild cy = tc_child(a.n_tips, x ? d.y : d.z,
-                              d.w & (x ? kDescFlagCompact0 : kDescFlagCompact1));
+  const TcChild cx = tc_child(a.n_tips, d.y, false);
+  const TcChild cy = tc_child(a.n_tips, d.z, d.w & kUnitCompactY);
   const bool root = k == a.root;
   const size_t kslot = (size_t)(k - a.n_tips);
   const int c0 = blockIdx.x * kTcRows, c = c0 + row;
@@ -487,11 +526,10 @@ __global__ void __launch_bounds__(kTcThreads) pre_tcb_kernel(LevelArgs<T> a) {
   tcb_issue_b(B0, bars, ph, 0, round_of(0).bsrc);
   tcb_issue_b(B0, bars, ph, 1, round_of(1).bsrc);
   // row-layout values of this thread's row for the epilogue
-  int eq_row = 0, ey_row = 0, yx_row = -1;
+  int eq_row = 0, ey_row = 0;
   if (c < C) {
     if (!root) eq_row = a.pre_escale[(kslot * R + r) * estr + c];
     if (cy.internal) ey_row = a.escale[((size_t)(cy.b - a.n_tips) * R + r) * estr + c];
-    if (cx.compact) yx_row = a.tip_states[(size_t)cx.b * a.state_stride + c];
   }
   // a_x = q_k o U_y in the cooperative layout, split into A
   float4 q[2][8];
@@ -526,19 +564,29 @@ __global__ void __launch_bounds__(kTcThreads) pre_tcb_kernel(LevelArgs<T> a) {
     for (int it = 0; it < 4; ++it) eq[it] = 0;
   }
   int Ey[4], Ex[4], yy[4], yxc[4];
+  float4 qg[2][8];  // q_k o G_y e_y of a tip sibling (its numerator is qg . U_x)
   {
     float4 uy[2][8];
     tcb_child_rows(uy, Ey, yy, a, cy, r, c0);
 #pragma unroll
     for (int kb = 0; kb < kTcbNB; ++kb)
 #pragma unroll
-      for (int i = 0; i < 8; ++i) q[kb][i] = mul4(q[kb][i], uy[kb][i]);
+      for (int it = 0; it < 4; ++it) {
+        if (cy.compact) {
+          float4 lo, hi;
+          tcb_gtab8(a, cy.b, r, yy[it], kb, j, lo, hi);
+          qg[kb][2 * it] = mul4(q[kb][2 * it], lo);
+          qg[kb][2 * it + 1] = mul4(q[kb][2 * it + 1], hi);
+        }
+        q[kb][2 * it] = mul4(q[kb][2 * it], uy[kb][2 * it]);
+        q[kb][2 * it + 1] = mul4(q[kb][2 * it + 1], uy[kb][2 * it + 1]);
+      }
   }
 #pragma unroll
   for (int kb = 0; kb < kTcbNB; ++kb) coop_put(tcb_a(A0, kb), q[kb]);
   tc::fence_smem_for_async();
   // den = a_x . U_x per row (U_x loads in flight during the MMAs)
-  float den[4];
+  float den[4], ny[4];
   {
     float4 ux[2][8];
     tcb_child_rows(ux, Ex, yxc, a, cx, r, c0);
@@ -550,6 +598,13 @@ __global__ void __launch_bounds__(kTcThreads) pre_tcb_kernel(LevelArgs<T> a) {
       for (int kb = 0; kb < kTcbNB; ++kb)
         s = dot4(q[kb][2 * it + 1], ux[kb][2 * it + 1], dot4(q[kb][2 * it], ux[kb][2 * it], s));
       den[it] = row_sum8(s);
+      if (!cy.compact) continue;
+      s = 0.f;
+#pragma unroll
+      for (int kb = 0; kb < kTcbNB; ++kb)
+        s = dot4(qg[kb][2 * it + 1], ux[kb][2 * it + 1],
+                 dot4(qg[kb][2 * it], ux[kb][2 * it], s));
+      ny[it] = row_sum8(s);
     }
     if (!ok0) {
       TCB_EPILOGUE(256)
@@ -560,7 +615,7 @@ __global__ void __launch_bounds__(kTcThreads) pre_tcb_kernel(LevelArgs<T> a) {
   float num = 0.f, m = 0.f;
   {
     float u[64];
-    tcb_child_half(u, a, cx, r, c, h, yx_row);
+    tcb_child_half(u, a, cx, r, c, h);
 #pragma unroll
     for (int qq = 0; qq < 2; ++qq) {
       float w[32];
@@ -581,19 +636,20 @@ __global__ void __launch_bounds__(kTcThreads) pre_tcb_kernel(LevelArgs<T> a) {
   __syncthreads();
   num += xn[1 - h][row];
   m = fmaxf(m, xm[1 - h][row]);
-  if (cx.compact && yx_row >= S) num = 0.f;  // d/dt of the all-ones vector is 0
   float* rt = reinterpret_cast<float*>(a.rterm);
-  if (c < C && h == 0) {
-    rt[((kslot * C + c) * R + r) * 4 + x] = (float)(a.cat_w[r] * a.rates[r]) * num;
-  }
-  if (x == 0) {  // den and the exponent of the Eq. 8 terms, from the cooperative layout
+  const float wg = (float)(a.cat_w[r] * a.rates[r]);
+  if (c < C && h == 0) rt[((kslot * C + c) * R + r) * 4 + x] = wg * num;
+  if (d.w & (kUnitDen | kUnitCompactY)) {  // the other terms, from the cooperative layout
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
       const int cc = c0 + coop_row(it);
       if (cc < C && j == 0) {
         float* t4 = rt + ((kslot * C + cc) * R + r) * 4;
-        t4[2] = a.cat_wt[r] * den[it];
-        t4[3] = __int_as_float(eq[it] + Ex[it] + Ey[it]);
+        if (cy.compact) t4[1 - x] = wg * ny[it];
+        if (d.w & kUnitDen) {
+          t4[2] = a.cat_wt[r] * den[it];
+          t4[3] = __int_as_float(eq[it] + Ex[it] + Ey[it]);
+        }
       }
     }
   }
@@ -617,18 +673,44 @@ __global__ void __launch_bounds__(kTcThreads) pre_tcb_kernel(LevelArgs<T> a) {
 #undef TCB_PROLOGUE
 #undef TCB_EPILOGUE
 
+struct Cols128 {
+  template <bool G>
+  __device__ __forceinline__ static void col(const LevelArgs<float>& a, int b, int r, int y,
+                                             int kb, int j, float4& lo, float4& hi) {
+    if (G) tcb_gtab8(a, b, r, y, kb, j, lo, hi);
+    else tcb_col8(a, b, r, y, kb, j, lo, hi);
+  }
+};
+
+// The nodes whose children are both compact tips (level_desc), then the ratios.
+template <int SP>
+inline cudaError_t launch_ratio_tc64(const LevelArgs<float>& a, cudaStream_t st) {
+  if (a.n_tiles <= 0 || a.n_tips < 2) return cudaSuccess;
+  if (a.n_level > 0) {
+    const cudaError_t e =
+        launch_pdl(SP == 64 ? cherry_kernel<64, Cols64> : cherry_kernel<128, Cols128>,
+                   dim3(a.n_tiles, a.n_cat, a.n_level), kTcThreads, 0, st, a);
+    if (e != cudaSuccess) return e;
+  }
+  dim3 grid(a.n_tiles, a.n_tips - 1);
+  return launch_pdl(ratio_tc_kernel<float>, grid, kTcRows, 0, st, a);
+}
+
 inline cudaError_t launch_tcb(const LevelArgs<float>& a, bool post, cudaStream_t st) {
   if (post) {
     if (a.root_level) return launch_pdl(root_tcb_kernel<float>, dim3(a.n_tiles), kTcRows, 0, st, a);
     dim3 grid(a.n_tiles, a.n_level, a.n_cat);
     return launch_pdl(post_tcb_kernel<float>, grid, kTcThreads, kTcbSmem, st, a);
   }
-  dim3 grid(a.n_tiles, a.n_level, 2 * a.n_cat);
+  dim3 grid(a.n_tiles, a.n_cat, a.n_level);
   return launch_pdl(pre_tcb_kernel<float>, grid, kTcThreads, kTcbSmem, st, a);
 }
 
 inline cudaError_t launch_pmat_tcb(const PmatArgs& a, cudaStream_t st) {
-  return launch_pmat_big<kTcbSP>(a, st);  // (writes the operand blocks: a.tiles is set)
+  // (writes the operand blocks: a.tiles is set)
+  const cudaError_t e = launch_pmat_big<kTcbSP>(a, st);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(tipq_tcb_kernel<float>, dim3(a.n_tips * a.n_cat), kTcThreads, kTcbSmem, st, a);
 }
 
 inline cudaError_t prepare_tcb() {
@@ -637,6 +719,9 @@ inline cudaError_t prepare_tcb() {
                                        (int)kTcbSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(pre_tcb_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kTcbSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(tipq_tcb_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kTcbSmem);
   return e;
 }

@@ -48,6 +48,7 @@ struct Layout {
   Region vsplit;  // tensor-core path: eigenvectors as double-float tables
   Region tc_tiles;  // 65..128 states, FP32: pre-split matrix blocks
   Region qt;        // 21..128 states, FP32, and 21..64, FP64: Q' as a tensor-core operand
+  Region qn;        // 21..128 states, FP32: Q as a tensor-core operand
   Region vdigits;   // 21..64 states, FP64: the digits of Vinv'
   Region qmat;      // 4 and 20 padded states, FP32: Q row-major
   Region tip_desc;  // U-form paths with tip partials: descriptors of the tips
@@ -106,7 +107,9 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
   ok &= add_region(L, L.post_nodes, n_int * sizeof(int));
   ok &= add_region(L, L.pre_nodes, n_int * sizeof(int));
   ok &= add_region(L, L.post_desc, n_int * sizeof(int4));
-  ok &= add_region(L, L.pre_desc, n_int * sizeof(int4));
+  // (units on the tensor-core paths: up to two per node)
+  ok &= add_region(L, L.pre_desc,
+                   n_int * sizeof(int4) * (uses_tc_terms(L.SP, prec == PHYLO_FP64) ? 2 : 1));
   if (L.mode != kByLevel) {
     ok &= add_region(L, L.post_off, (n_int + 1) * sizeof(int));
     ok &= add_region(L, L.pre_off, (n_int + 1) * sizeof(int));
@@ -131,7 +134,10 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
     ok &= add_region(L, L.post, part);
   }
   ok &= add_region(L, L.pre, L.mode == kWalk ? 0 : part);
-  if (tc || uses_tc_big(L.SP, prec == PHYLO_FP64)) ok &= add_region(L, L.qt, qt_bytes(L.SP));
+  if (tc || uses_tc_big(L.SP, prec == PHYLO_FP64)) {
+    ok &= add_region(L, L.qt, qt_bytes(L.SP));
+    ok &= add_region(L, L.qn, qt_bytes(L.SP));
+  }
   if (tcd) {
     ok &= add_region(L, L.qt, kTcdModelBytes);
     ok &= add_region(L, L.vdigits, kTcdModelBytes);
@@ -208,6 +214,8 @@ struct phylo_ctx {
   std::vector<int2> children;
   std::vector<int> post_nodes, post_off;  // level l: [post_off[l], post_off[l+1])
   std::vector<int> pre_nodes, pre_off;
+  std::vector<int> unit_off;  // tensor-core paths: the same offsets in pre-order
+                              // units, then the nodes with two compact tips
   int n_post_levels = 0, n_pre_levels = 0;    // the level schedule's length
   std::vector<char> post_cherry, pre_cherry;  // per level: a node has a fused cherry child
   std::vector<int> height, depth;             // per node
@@ -397,6 +405,8 @@ cudaError_t enqueue_phase(phylo_ctx* ctx, int phase, cudaStream_t st) {
     pa.vsplit = ctx->L.vsplit.bytes ? ctx->dev<float>(ctx->L.vsplit) : nullptr;
     pa.vdigits = ctx->L.vdigits.bytes ? ctx->dev<void>(ctx->L.vdigits) : nullptr;
     pa.n_tips = ctx->N;
+    pa.qn = ctx->L.qn.bytes ? ctx->dev<unsigned char>(ctx->L.qn) : nullptr;
+    pa.tip_has = has_tip_level(ctx) ? ctx->dev<int>(ctx->L.tip_has) : nullptr;
     pa.reversible = ctx->eig_reversible;
     pa.V = ctx->dev<double>(ctx->L.V);
     pa.Vinv = ctx->dev<double>(ctx->L.Vinv);
@@ -435,20 +445,29 @@ cudaError_t enqueue_phase(phylo_ctx* ctx, int phase, cudaStream_t st) {
     }
     // P may be staged before the wait on the previous launch unless that
     // launch is the matrix kernel itself (the first post-order launch).
-    bool after_pmat = post && !(ctx->L.tip_desc.bytes && a.tip_partials);
+    // (The tips' tables are built by a launch of their own in between.)
+    bool after_pmat =
+        post && !ctx->L.qn.bytes && !(ctx->L.tip_desc.bytes && a.tip_partials);
+    const bool units = !post && uses_tc_terms(ctx->L.SP, ctx->precision == PHYLO_FP64);
     for (size_t l = 0; l + 1 < off.size(); ++l) {
       NvtxRange range(post ? "phylo post-order level (Eq. 2)"
                            : "phylo pre-order level (Eqs. 4, 8)", (int)l);
       a.mats_ready = after_pmat ? 0 : 1;
       after_pmat = false;
       a.level_nodes = nodes + off[l];
-      a.level_desc = desc + off[l];
-      a.n_level = off[l + 1] - off[l];
+      const std::vector<int>& doff = units ? ctx->unit_off : off;
+      a.level_desc = desc + doff[l];
+      a.n_level = doff[l + 1] - doff[l];
+      if (a.n_level == 0) continue;  // (its nodes' children are all compact tips)
       a.root_level = post && l + 2 == off.size();  // the last post level is the root
       a.level_cherry = (post ? ctx->post_cherry : ctx->pre_cherry)[l];
       e = post ? launch_post_level<T>(a, ctx->L.SP, ctx->L.RP, st)
                : launch_pre_level<T>(a, ctx->L.SP, ctx->L.RP, st);
       if (e != cudaSuccess) return e;
+    }
+    if (units) {
+      a.level_desc = desc + ctx->unit_off[off.size() - 1];
+      a.n_level = ctx->unit_off[off.size()] - ctx->unit_off[off.size() - 1];
     }
     if (!post && ctx->C > 0) return launch_pre_finish<T>(a, ctx->L.SP, st);
     return cudaSuccess;
@@ -625,15 +644,37 @@ int upload_descriptors(phylo_ctx* ctx) {
   for (int pass = 0; pass < 2; ++pass) {
     const std::vector<int>& nodes = pass == 0 ? ctx->post_nodes : ctx->pre_nodes;
     std::vector<int4> desc(nodes.size());
-    for (size_t i = 0; i < nodes.size(); ++i) {
-      const int k = nodes[i];
-      const int2 ch = ctx->children[k];
-      int flags = 0;
-      if (ch.x < ctx->N && !ctx->tip_has[ch.x]) flags |= kDescFlagCompact0;
-      if (ch.y < ctx->N && !ctx->tip_has[ch.y]) flags |= kDescFlagCompact1;
-      if (ch.x >= ctx->N && ctx->cherry[ch.x]) flags |= kDescFlagCherry0;
-      if (ch.y >= ctx->N && ctx->cherry[ch.y]) flags |= kDescFlagCherry1;
-      desc[i] = make_int4(k, ch.x, ch.y, flags);
+    if (pass == 1 && uses_tc_terms(ctx->L.SP, ctx->precision == PHYLO_FP64)) {
+      desc.clear();
+      ctx->unit_off.assign(1, 0);
+      for (size_t l = 0; l + 1 < ctx->pre_off.size(); ++l) {
+        for (int i = ctx->pre_off[l]; i < ctx->pre_off[l + 1]; ++i) {
+          const int2 ch = ctx->children[nodes[i]];
+          int4 u[2];
+          const int n = pre_units(nodes[i], ch.x, ch.y, ch.x < ctx->N && !ctx->tip_has[ch.x],
+                                  ch.y < ctx->N && !ctx->tip_has[ch.y], u);
+          desc.insert(desc.end(), u, u + n);
+        }
+        ctx->unit_off.push_back((int)desc.size());
+      }
+      // then the nodes whose children are both compact tips
+      for (int k : nodes) {
+        const int2 ch = ctx->children[k];
+        if (ch.x < ctx->N && ch.y < ctx->N && !ctx->tip_has[ch.x] && !ctx->tip_has[ch.y])
+          desc.push_back(make_int4(k, ch.x, ch.y, 0));
+      }
+      ctx->unit_off.push_back((int)desc.size());
+    } else {
+      for (size_t i = 0; i < nodes.size(); ++i) {
+        const int k = nodes[i];
+        const int2 ch = ctx->children[k];
+        int flags = 0;
+        if (ch.x < ctx->N && !ctx->tip_has[ch.x]) flags |= kDescFlagCompact0;
+        if (ch.y < ctx->N && !ctx->tip_has[ch.y]) flags |= kDescFlagCompact1;
+        if (ch.x >= ctx->N && ctx->cherry[ch.x]) flags |= kDescFlagCherry0;
+        if (ch.y >= ctx->N && ctx->cherry[ch.y]) flags |= kDescFlagCherry1;
+        desc[i] = make_int4(k, ch.x, ch.y, flags);
+      }
     }
     if (!desc.empty()) {
       int rc = upload(ctx, pass == 0 ? ctx->L.post_desc : ctx->L.pre_desc, desc.data(),
@@ -1079,6 +1120,9 @@ int phylo_set_eigen(phylo_ctx* ctx, const double* V, const double* Vinv,
     build_qt_tile(S, ctx->L.SP, V, Vinv, lambda, qt.data());
     if ((rc = upload(ctx, ctx->L.qt, qt.data(), qt.size(), "upload Q operand"))) return rc;
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+    build_qt_tile(S, ctx->L.SP, V, Vinv, lambda, qt.data(), true);
+    if ((rc = upload(ctx, ctx->L.qn, qt.data(), qt.size(), "upload Q operand"))) return rc;
+    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
   }
   if ((rc = upload(ctx, ctx->L.lambda, lambda, (size_t)S, "upload lambda"))) return rc;
   if ((rc = upload(ctx, ctx->L.pi, pi, (size_t)S, "upload pi"))) return rc;
@@ -1440,6 +1484,7 @@ int phylo_launches_per_evaluation(const phylo_ctx* ctx) {
     const bool fp64 = ctx->precision == PHYLO_FP64;
     n += ctx->n_post_levels + ctx->n_pre_levels;
     if (uses_tc_terms(ctx->L.SP, fp64)) ++n;  // Eq. 8 ratios
+    if (ctx->L.qn.bytes) ++n;                 // tables of the compact tips
     if (has_tip_level(ctx)) ++n;                // U of the tips with partials
   }
   return n;

@@ -17,6 +17,31 @@ namespace phylo {
 constexpr int kDescFlagCompact0 = 1, kDescFlagCompact1 = 2;
 constexpr int kDescFlagCherry0 = 4, kDescFlagCherry1 = 8;
 
+// Pre-order units of the tensor-core paths: {k, child x, sibling y, flags}.
+// A unit contracts the a of a child that is internal or has partial vectors;
+// a compact tip's numerator is a table lookup in its sibling's unit.  A node
+// whose children are both compact tips has none: its terms are lookups only,
+// which nothing waits for, and follow after the last level, for all such nodes
+// in one launch.
+constexpr int kUnitCompactY = 1;  // y is a compact tip
+constexpr int kUnitSecond = 2;    // x is child 1 of k
+constexpr int kUnitDen = 4;       // writes the denominator
+// The units of node k with children (i, j); returns their number (0 to 2).
+inline int pre_units(int k, int i, int j, bool compact_i, bool compact_j, int4 (&out)[2]) {
+  if (compact_i && compact_j) return 0;
+  if (compact_j) {
+    out[0] = make_int4(k, i, j, kUnitCompactY | kUnitDen);
+    return 1;
+  }
+  if (compact_i) {
+    out[0] = make_int4(k, j, i, kUnitCompactY | kUnitSecond | kUnitDen);
+    return 1;
+  }
+  out[0] = make_int4(k, i, j, kUnitDen);
+  out[1] = make_int4(k, j, i, kUnitSecond);
+  return 2;
+}
+
 // Device-side numeric flags (bit mask in the workspace's error word).
 enum : int {
   ERR_ZERO_PARTIAL = 1,  // a partial vector was all zero / NaN for a pattern
@@ -201,8 +226,10 @@ inline size_t qt_bytes(int SP) { return (size_t)(SP / 64) * (SP / 64) * kTcQtByt
 // in the K-major 128-byte-swizzle layout the MMAs read (element (row, k) of
 // a term at row * 128 + (((k / 8) ^ (row % 8)) * 16) + (k % 8) * 2, terms
 // 8 KB apart).  Rows and columns past S are zero.  out: qt_bytes(SP).
+// With `rows` the operand holds Q itself (row s = row s of Q; the tips' tables
+// Q P).
 inline void build_qt_tile(int S, int SP, const double* V, const double* Vinv,
-                          const double* lambda, unsigned char* out) {
+                          const double* lambda, unsigned char* out, bool rows = false) {
   std::memset(out, 0, qt_bytes(SP));
   const size_t term = 64 * 128;
   const int NB = SP / 64;
@@ -211,8 +238,9 @@ inline void build_qt_tile(int S, int SP, const double* V, const double* Vinv,
       double q = 0.0;  // Q[t][s]
       for (int m = 0; m < S; ++m) q += V[t * S + m] * lambda[m] * Vinv[m * S + s];
       float rem = (float)q;
-      const int n = s & 63, k = t & 63;
-      const size_t blk = ((size_t)(t >> 6) * NB + (s >> 6)) * kTcQtBytes;
+      const int on = rows ? t : s, ok = rows ? s : t;  // the entry's row and column
+      const int n = on & 63, k = ok & 63;
+      const size_t blk = ((size_t)(ok >> 6) * NB + (on >> 6)) * kTcQtBytes;
       const size_t off = blk + (size_t)n * 128 + ((size_t)((k >> 3) ^ (n & 7)) << 4) + (k & 7) * 2;
       for (int i = 0; i < 3; ++i) {
         const uint16_t b = host_bf16(rem);
@@ -337,8 +365,9 @@ template <typename T>
 struct LevelArgs {
   const int2* children;        // [2N-1]; (-1,-1) for tips
   const int* level_nodes;      // internal nodes of this level
-  const int4* level_desc;      // per level node: {k, child 0, child 1, flags}
-  int n_level;                 // number of nodes in the level
+  const int4* level_desc;      // per level node: {k, child 0, child 1, flags}; the
+                               // pre-order pass of the tensor-core paths: units
+  int n_level;                 // number of nodes (units) in the level
   int root_level;              // 1 if the level is the root alone
   int level_cherry;            // 1 if a node of the level has a fused cherry child
   int n_tips, n_patterns, n_states, n_cat, root;
@@ -412,6 +441,9 @@ struct TreePass {
 
 struct PmatArgs {
   const float* vsplit;   // tensor-core path: build_eigen_split's table
+  const unsigned char* qn;  // 21..128 states, FP32: Q as an operand (its rows), for the
+                            // tables Q P of compact tips
+  const int* tip_has;    // [N] or nullptr: tips with partial vectors (no table)
   const void* vdigits;   // FP64, 21..64 states: the digits of Vinv' (build_digits)
   int n_tips;
   int reversible;        // tensor-core path: the table's decomposition is symmetric

@@ -33,7 +33,13 @@ constexpr int kMaxNoAllocTips = 512;
 constexpr int kMaxDevices = 64;
 constexpr size_t kAlignNA = 256;
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
+// Beyond the problem's buffers (limited to kNoAllocScratchBytes) the array
+// holds the pre-order units and Q's operand of the tensor-core path.
+constexpr size_t kNoAllocExtraBytes =
+    2 * kMaxNoAllocTips * sizeof(int4) + kTcQtBytes + 2 * kAlignNA;
+
+static __device__ __align__(256) unsigned char
+    g_noalloc_scratch[kNoAllocScratchBytes + kNoAllocExtraBytes];
 
 std::mutex g_noalloc_mutex;
 void* g_scratch_ptr[kMaxDevices] = {};
@@ -60,6 +66,7 @@ struct NaLayout {
       pre_escale, rterm;
   NaRegion tip_states, pattern_w, V, Vinv, lambda, pi, rates, cat_w, t, vsplit, qt, qmat;
   NaRegion gpart, lpart, out, pattern_wt, cat_wt, pi_t;
+  NaRegion units, qn;  // tensor-core path, past `total`
   size_t total = 0;
 };
 
@@ -117,6 +124,12 @@ void na_layout(int N, int C, int S, int R, NaLayout* Lp) {
   na_add(L, L.pattern_wt, (size_t)C * sizeof(float));
   na_add(L, L.cat_wt, (size_t)R * sizeof(float));
   na_add(L, L.pi_t, (size_t)S * sizeof(float));
+  if (tc) {
+    const size_t total = L.total;
+    na_add(L, L.units, 2 * n_int * sizeof(int4));
+    na_add(L, L.qn, kTcQtBytes);
+    L.total = total;
+  }
   *Lp = L;
 }
 
@@ -289,6 +302,7 @@ int phylo_evaluate_noalloc(int N, int C, int S, int R, const int32_t* parent,
   NA_TRY(up(L.children, ch, n * sizeof(int2)), "upload tree");
   NA_TRY(up(L.post_nodes, post_nodes, (size_t)post_off[n_post] * sizeof(int)), "upload schedule");
   NA_TRY(up(L.pre_nodes, pre_nodes, (size_t)pre_off[n_pre] * sizeof(int)), "upload schedule");
+  int unit_end = 0, n_cherries = 0;
   {  // level-node descriptors {k, child 0, child 1, flags}; every tip is compact
     int4 desc[kMaxNoAllocTips];
     for (int pass = 0; pass < 2; ++pass) {
@@ -302,6 +316,28 @@ int phylo_evaluate_noalloc(int N, int C, int S, int R, const int32_t* parent,
       NA_TRY(up(pass == 0 ? L.post_desc : L.pre_desc, desc, (size_t)count * sizeof(int4)),
              "upload descriptors");
       // the host array is reused: finish this copy first
+      NA_TRY(cudaStreamSynchronize(st), "cudaStreamSynchronize");
+    }
+    if (L.units.bytes) {  // the pre-order pass runs in units: offsets in units too
+      int4 units[2 * kMaxNoAllocTips];
+      int n_units = 0;
+      for (int l = 0; l < n_pre; ++l) {
+        const int end = pre_off[l + 1];
+        for (int i = l ? unit_end : 0; i < end; ++i) {
+          const int2 c2 = ch[pre_nodes[i]];
+          int4 u[2];
+          const int m = pre_units(pre_nodes[i], c2.x, c2.y, c2.x < N, c2.y < N, u);
+          for (int v = 0; v < m; ++v) units[n_units++] = u[v];
+        }
+        unit_end = end;
+        pre_off[l + 1] = n_units;
+      }
+      for (int i = 0; i < N - 1; ++i) {  // then the nodes with two tips
+        const int2 c2 = ch[pre_nodes[i]];
+        if (c2.x < N && c2.y < N) units[n_units++] = make_int4(pre_nodes[i], c2.x, c2.y, 0);
+      }
+      n_cherries = n_units - pre_off[n_pre];
+      NA_TRY(up(L.units, units, (size_t)n_units * sizeof(int4)), "upload units");
       NA_TRY(cudaStreamSynchronize(st), "cudaStreamSynchronize");
     }
   }
@@ -325,10 +361,12 @@ int phylo_evaluate_noalloc(int N, int C, int S, int R, const int32_t* parent,
     build_q_matrix(S, L.SP, V, Vinv, lambda, qmat);
     NA_TRY(up(L.qmat, qmat, L.qmat.bytes), "upload Q");
   }
-  static thread_local unsigned char qt[kTcQtBytes];
+  static thread_local unsigned char qt[2][kTcQtBytes];
   if (L.qt.bytes) {
-    build_qt_tile(S, L.SP, V, Vinv, lambda, qt);
-    NA_TRY(up(L.qt, qt, kTcQtBytes), "upload Q operand");
+    build_qt_tile(S, L.SP, V, Vinv, lambda, qt[0]);
+    build_qt_tile(S, L.SP, V, Vinv, lambda, qt[1], true);
+    NA_TRY(up(L.qt, qt[0], kTcQtBytes), "upload Q operand");
+    NA_TRY(up(L.qn, qt[1], kTcQtBytes), "upload Q operand");
   }
   NA_TRY(up(L.lambda, lambda, (size_t)S * 8), "upload lambda");
   NA_TRY(up(L.pi, root_freqs, (size_t)S * 8), "upload pi");
@@ -361,6 +399,8 @@ int phylo_evaluate_noalloc(int N, int C, int S, int R, const int32_t* parent,
   pa.n_branches = 2 * N - 2;
   pa.n_states = S;
   pa.n_cat = R;
+  pa.n_tips = N;
+  pa.qn = L.qn.bytes ? reinterpret_cast<const unsigned char*>(ws + L.qn.off) : nullptr;
   pa.P = ws + L.P.off;
   pa.dP = ws + L.dP.off;
   pa.err = flag;
@@ -401,7 +441,8 @@ int phylo_evaluate_noalloc(int N, int C, int S, int R, const int32_t* parent,
   const int* dpost = reinterpret_cast<const int*>(ws + L.post_nodes.off);
   const int* dpre = reinterpret_cast<const int*>(ws + L.pre_nodes.off);
   const int4* dpostd = reinterpret_cast<const int4*>(ws + L.post_desc.off);
-  const int4* dpred = reinterpret_cast<const int4*>(ws + L.pre_desc.off);
+  const int4* dpred =
+      reinterpret_cast<const int4*>(ws + (L.units.bytes ? L.units.off : L.pre_desc.off));
   for (int l = 0; l < n_post; ++l) {
     a.level_nodes = dpost + post_off[l];
     a.level_desc = dpostd + post_off[l];
@@ -414,8 +455,11 @@ int phylo_evaluate_noalloc(int N, int C, int S, int R, const int32_t* parent,
     a.level_nodes = dpre + pre_off[l];
     a.level_desc = dpred + pre_off[l];
     a.n_level = pre_off[l + 1] - pre_off[l];
+    if (a.n_level == 0) continue;
     NA_TRY(launch_pre_level<float>(a, L.SP, L.RP, st), "pre-order level");
   }
+  a.level_desc = dpred + pre_off[n_pre];
+  a.n_level = n_cherries;
   if (C > 0) NA_TRY(launch_pre_finish<float>(a, L.SP, st), "gradient ratios");
   ReduceArgs ra{};
   ra.gpart = a.gpart;
