@@ -643,11 +643,11 @@ __global__ void __launch_bounds__(256) pmat_big_df_kernel(PmatArgs a) {
       }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      put_split3_4(U + tcb_block(0, sb, tb), kTerm64, ls + i, lt,
+      put_split3_4(U + tcb_block(0, sb, tb), kTerm128, ls + i, lt,
                    make_float4(p[i][0], p[i][1], p[i][2], p[i][3]));
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      put_split3_4(U + tcb_block(1, tb, sb), kTerm64, lt + j, ls,
+      put_split3_4(U + tcb_block(1, tb, sb), kTerm128, lt + j, ls,
                    make_float4(p[0][j], p[1][j], p[2][j], p[3][j]));
     if (rev && sb != tb) {  // mirror: P[t][s] = delta + K_st pi_s
 #pragma unroll
@@ -657,11 +657,11 @@ __global__ void __launch_bounds__(256) pmat_big_df_kernel(PmatArgs a) {
           p[i][j] = df_round(df_mul(accP[i][j], DF{pi_h[s0 + i], pi_l[s0 + i]}), false);
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        put_split3_4(U + tcb_block(0, tb, sb), kTerm64, lt + j, ls,
+        put_split3_4(U + tcb_block(0, tb, sb), kTerm128, lt + j, ls,
                      make_float4(p[0][j], p[1][j], p[2][j], p[3][j]));
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        put_split3_4(U + tcb_block(1, sb, tb), kTerm64, ls + i, lt,
+        put_split3_4(U + tcb_block(1, sb, tb), kTerm128, ls + i, lt,
                      make_float4(p[i][0], p[i][1], p[i][2], p[i][3]));
     }
     return;

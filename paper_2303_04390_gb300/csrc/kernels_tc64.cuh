@@ -75,8 +75,8 @@ static_assert(kTcQtBytes == kOp64, "Q' operand size");
 
 // Dynamic shared memory (+1024 for the alignment of the swizzled tiles):
 //   post: p_k (128-row operand, later the U_k staging) | P_k (64 rows)
-//   pre:  a_x (128-row operand, later the W_x staging) | P_x' | Q' (64 rows
-//         each; later the q_x staging)
+//   pre:  a_x (128-row operand, later the W_x staging) | [P_x' | Q'] (128 rows;
+//         later the q_x staging)
 constexpr size_t kPostUSmem = 1024 + kOp128 + kOp64;
 // Resident CTAs per SM the post-order kernel's registers are bounded for
 // (its shared memory admits three; bounding the registers for three spills and measured slower).
@@ -802,10 +802,11 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
   extern __shared__ unsigned char smraw[];
   unsigned char* base = align1024(smraw);
   unsigned char* A = base;                     // a_x as three BF16 terms
-  unsigned char* Bp = base + kOp128;           // P_x' (rows = columns of P_x)
-  unsigned char* Bq = base + kOp128 + kOp64;   // Q' (rows = columns of Q)
+  // [P_x' | Q'] as one 128-row operand (rows = columns of P_x, then of Q): one
+  // chain of N = 128 MMAs where two of N = 64 took as many clocks each
+  unsigned char* B = base + kOp128;
   float* stW = reinterpret_cast<float*>(A);    // W_x rows, after the MMAs
-  float* stQ = reinterpret_cast<float*>(Bp);   // q_x rows, after the MMAs
+  float* stQ = reinterpret_cast<float*>(B);    // q_x rows, after the MMAs
   // a compact sibling's tables (columns of P and of G = Q P, FP32) in A until
   // the split
   const float* pt32y = reinterpret_cast<const float*>(A);
@@ -834,8 +835,12 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
     mbar_init_fenced(&bar_mma, 1);
     mbar_expect_tx(&bar_tma, kOp64 + (cx.internal ? kOp64 : 0) +
                                  (cy.compact ? 2 * kPt32Bytes : 0));
-    bulk_g2s(Bq, a.qt, kOp64, &bar_tma);
-    if (cx.internal) bulk_g2s(Bp, unit_tiles(a, cx.b, r) + kUnitPt, kOp64, &bar_tma);
+    for (int t = 0; t < 3; ++t) {
+      bulk_g2s(B + t * kTerm128 + kTerm64, a.qt + t * kTerm64, kTerm64, &bar_tma);
+      if (cx.internal)
+        bulk_g2s(B + t * kTerm128, unit_tiles(a, cx.b, r) + kUnitPt + t * kTerm64, kTerm64,
+                 &bar_tma);
+    }
     if (cy.compact) {
       bulk_g2s(A, unit_tiles(a, cy.b, r) + kUnitPt32, kPt32Bytes, &bar_tma);
       bulk_g2s(A + kPt32Bytes, unit_tiles(a, cy.b, r) + kUnitP, kPt32Bytes, &bar_tma);
@@ -911,11 +916,12 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
       tc::fence_after();
       uint32_t ta[3], tb[3];
       term_addrs(A, kTerm128, ta);
-      term_addrs(Bq, kTerm64, tb);
-      tc::mma_split_bf16x3<64>(tmem + 64, ta, tb);
       if (cx.internal) {
-        term_addrs(Bp, kTerm64, tb);
-        tc::mma_split_bf16x3<64>(tmem, ta, tb);
+        term_addrs(B, kTerm128, tb);
+        tc::mma_split_bf16x3<128>(tmem, ta, tb);
+      } else {
+        term_addrs(B + kTerm64, kTerm128, tb);
+        tc::mma_split_bf16x3<64>(tmem + 64, ta, tb);
       }
       tc::commit(&bar_mma);
     }

@@ -34,10 +34,9 @@ namespace phylo {
 
 constexpr int kTcbSP = 128;                  // padded states of this path
 constexpr int kTcbNB = kTcbSP / 64;          // 64-blocks per dimension
-constexpr uint32_t kTcbBlock = 3 * kTerm64;  // one 64 x 64 three-term block
-static_assert(kTcbUnitBytes == 2 * kTcbNB * kTcbNB * kTcbBlock, "tile block size");
+static_assert(kTcbUnitBytes == 2 * kTcbNB * kOp128, "matrix block size");
 // Shared memory: A 2 x 48 KB (both K-blocks), B ring 2 x 48 KB (+1024 for alignment).
-constexpr size_t kTcbSmem = 1024 + 2 * (size_t)kOp128 + 4 * (size_t)kTcbBlock;
+constexpr size_t kTcbSmem = 1024 + 4 * (size_t)kOp128;
 constexpr int kTcbLd = kTcbSP + 4;           // output staging row stride (floats)
 static_assert((size_t)kTcRows * kTcbLd * 4 <= 2 * (size_t)kOp128, "staging fits in A");
 
@@ -69,8 +68,8 @@ __device__ __forceinline__ void tcb_col8(const LevelArgs<float>& a, int b, int r
   const unsigned char* blk = tcb_unit(a, b, r) + tcb_block(1, y >> 6, kb);
   const uint32_t off = tc::b16_chunk(y & 63, j);
   const uint4 t0 = __ldg(reinterpret_cast<const uint4*>(blk + off));
-  const uint4 t1 = __ldg(reinterpret_cast<const uint4*>(blk + kTerm64 + off));
-  const uint4 t2 = __ldg(reinterpret_cast<const uint4*>(blk + 2 * kTerm64 + off));
+  const uint4 t1 = __ldg(reinterpret_cast<const uint4*>(blk + kTerm128 + off));
+  const uint4 t2 = __ldg(reinterpret_cast<const uint4*>(blk + 2 * kTerm128 + off));
   const uint32_t w0[4] = {t0.x, t0.y, t0.z, t0.w}, w1[4] = {t1.x, t1.y, t1.z, t1.w},
                  w2[4] = {t2.x, t2.y, t2.z, t2.w};
   float v[8];
@@ -137,18 +136,14 @@ __device__ __forceinline__ void tcb_child_half(float (&u)[64], const LevelArgs<f
   }
 }
 
-// D (+)= A B' for the two 64-column blocks jn of one K-block (the MMAs of
-// one round): B holds the two blocks (jn = 0, 1) back to back.
+// D (+)= A B' for one K-block (the MMAs of one round).  N = 128 in one chain:
+// two chains of N = 64 took 27 clocks per MMA for half the work.
 __device__ __forceinline__ void tcb_mma_round(uint32_t d_tmem, const unsigned char* A,
                                               const unsigned char* B, bool accumulate) {
-  uint32_t ta[3];
+  uint32_t ta[3], tb[3];
   term_addrs(A, kTerm128, ta);
-#pragma unroll
-  for (int jn = 0; jn < kTcbNB; ++jn) {
-    uint32_t tb[3];
-    term_addrs(B + jn * kTcbBlock, kTerm64, tb);
-    tc::mma_split_bf16x3_acc<64>(d_tmem + 64 * jn, ta, tb, accumulate);
-  }
+  term_addrs(B, kTerm128, tb);
+  tc::mma_split_bf16x3_acc<128>(d_tmem, ta, tb, accumulate);
 }
 
 // Coalesced store of staged 128-float rows (a quarter warp writes one
@@ -228,8 +223,8 @@ __device__ __forceinline__ void tcb_drain(uint64_t* bars, const TcbPhases& ph) {
   __syncthreads();                                                           \
   if (warp == 0) tc::dealloc(tmem, COLS);
 
-// One round of a contraction: the two matrix blocks at bsrc (blocks jn = 0,
-// 1 of one K-block) times A buffer ab (that K-block of the A operand) into
+// One round of a contraction: the matrix operand at bsrc (one K-block) times
+// A buffer ab (that K-block of the A operand) into
 // d_tmem.
 struct TcbRound {
   const unsigned char* bsrc;
@@ -238,21 +233,21 @@ struct TcbRound {
   bool accumulate;
 };
 
-// A buffers at A0 + ab kOp128, B buffers at B0 + b 2 kTcbBlock.
+// A buffers at A0 + ab kOp128, B buffers at B0 + b kOp128.
 __device__ __forceinline__ unsigned char* tcb_a(unsigned char* A0, int ab) {
   return A0 + (size_t)ab * kOp128;
 }
 __device__ __forceinline__ unsigned char* tcb_b(unsigned char* B0, int b) {
-  return B0 + (size_t)b * 2 * kTcbBlock;
+  return B0 + (size_t)b * kOp128;
 }
 
 __device__ __forceinline__ void tcb_issue_b(unsigned char* B0, uint64_t* bars, TcbPhases& ph,
                                             int i, const unsigned char* bsrc) {
   if (threadIdx.x == 0) {
     const int b = i & 1;
-    mbar_expect_tx(&bars[b], 2 * kTcbBlock);
+    mbar_expect_tx(&bars[b], kOp128);
     ph.issue(b);
-    bulk_g2s(tcb_b(B0, b), bsrc, 2 * kTcbBlock, &bars[b]);
+    bulk_g2s(tcb_b(B0, b), bsrc, kOp128, &bars[b]);
   }
 }
 
@@ -288,7 +283,7 @@ __device__ __forceinline__ bool tcb_rounds(unsigned char* A0, unsigned char* B0,
 // of one (tip, category) per CTA, stored by columns in FP32 ([128][128]) in
 // place of the tip's P blocks.
 // ---------------------------------------------------------------------------
-static_assert(kTcbSP * kTcbSP * 4 <= kTcbNB * kTcbNB * kTcbBlock, "a table fits in the P blocks");
+static_assert(kTcbSP * kTcbSP * 4 <= kTcbNB * kOp128, "a table fits in the P blocks");
 
 template <typename T>  // float only
 __global__ void __launch_bounds__(kTcThreads) tipq_tcb_kernel(PmatArgs a) {
@@ -302,14 +297,11 @@ __global__ void __launch_bounds__(kTcThreads) tipq_tcb_kernel(PmatArgs a) {
     return TcbRound{a.qn + tcb_block(0, 0, kb), kb, tmem, kb > 0};
   };
   if (tid == 0) {  // A: P' (rows = columns of P), both K-blocks, on round 0's barrier
-    mbar_expect_tx(&bars[0], 2 * kTcbBlock + 2 * kOp128);
+    mbar_expect_tx(&bars[0], (1 + kTcbNB) * kOp128);
     ph.issue(0);
     for (int kb = 0; kb < kTcbNB; ++kb)
-      for (int jn = 0; jn < kTcbNB; ++jn)
-        for (int t = 0; t < 3; ++t)
-          bulk_g2s(tcb_a(A0, kb) + t * kTerm128 + jn * kTerm64,
-                   U + tcb_block(1, jn, kb) + t * kTerm64, kTerm64, &bars[0]);
-    bulk_g2s(tcb_b(B0, 0), round_of(0).bsrc, 2 * kTcbBlock, &bars[0]);
+      bulk_g2s(tcb_a(A0, kb), U + tcb_block(1, 0, kb), kOp128, &bars[0]);
+    bulk_g2s(tcb_b(B0, 0), round_of(0).bsrc, kOp128, &bars[0]);
   }
   tcb_issue_b(B0, bars, ph, 1, round_of(1).bsrc);
   if (tcb_rounds(A0, B0, bars, ph, kTcbNB, round_of, a.err)) {

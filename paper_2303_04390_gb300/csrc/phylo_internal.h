@@ -221,11 +221,10 @@ inline size_t qt_bytes(int SP) { return (size_t)(SP / 64) * (SP / 64) * kTcQtByt
 // Eq. 8 numerator through dP = gamma Q P): row s holds column s of
 // Q = V diag(lambda) Vinv (FP64, rounded once to FP32), each FP32 value
 // split as x = t0 + t1 + t2 with t_i the round-to-nearest BF16 of the
-// remainder, cut into 64 x 64 blocks (block (jn, jk) holds rows 64 jn ..,
-// columns 64 jk ..; blocks of one K-block jk adjacent, jn fastest) stored
+// remainder, cut into K-blocks of 64 columns, each an operand of SP rows stored
 // in the K-major 128-byte-swizzle layout the MMAs read (element (row, k) of
 // a term at row * 128 + (((k / 8) ^ (row % 8)) * 16) + (k % 8) * 2, terms
-// 8 KB apart).  Rows and columns past S are zero.  out: qt_bytes(SP).
+// SP * 128 bytes apart).  Rows and columns past S are zero.  out: qt_bytes(SP).
 // With `rows` the operand holds Q itself (row s = row s of Q; the tips' tables
 // Q P).
 inline void build_qt_tile(int S, int SP, const double* V, const double* Vinv,
@@ -240,11 +239,11 @@ inline void build_qt_tile(int S, int SP, const double* V, const double* Vinv,
       float rem = (float)q;
       const int on = rows ? t : s, ok = rows ? s : t;  // the entry's row and column
       const int n = on & 63, k = ok & 63;
-      const size_t blk = ((size_t)(ok >> 6) * NB + (on >> 6)) * kTcQtBytes;
+      const size_t blk = (size_t)(ok >> 6) * NB * kTcQtBytes + (size_t)(on >> 6) * term;
       const size_t off = blk + (size_t)n * 128 + ((size_t)((k >> 3) ^ (n & 7)) << 4) + (k & 7) * 2;
       for (int i = 0; i < 3; ++i) {
         const uint16_t b = host_bf16(rem);
-        std::memcpy(out + i * term + off, &b, 2);
+        std::memcpy(out + i * NB * term + off, &b, 2);
         rem = rem - host_bf16_value(b);
       }
     }
@@ -281,11 +280,12 @@ inline bool uses_tc_big(int SP, bool fp64) { return SP == 128 && !fp64; }
 constexpr size_t kTcbUnitBytes = 2 * 2 * 2 * (3 * 64 * 128);
 // Offset of block (kind, jn, jk) in a (branch, category) unit: kind 0 = P,
 // 1 = P' (its rows are the columns of P); block row n, column k
-// holds M[64 jn + n][64 jk + k] as three BF16 terms of 8 KB each, in the
-// K-major 128-byte-swizzle layout of tc.cuh.  The blocks of one K-block jk
-// are adjacent (jn fastest), so one bulk copy stages a contraction round.
+// holds M[64 jn + n][64 jk + k] as three BF16 terms in the K-major
+// 128-byte-swizzle layout of tc.cuh.  The two row blocks of a K-block jk are
+// one 128-row operand (terms 16 KB apart), which one bulk copy stages and one
+// chain of N = 128 MMAs reads.
 __host__ __device__ constexpr size_t tcb_block(int kind, int jn, int jk) {
-  return (((size_t)kind * 2 + jk) * 2 + jn) * (3 * 64 * 128);
+  return ((size_t)kind * 2 + jk) * (3 * 128 * 128) + (size_t)jn * (64 * 128);
 }
 // Paths with per-category exponents and Eq. 8 terms combined by the ratio
 // kernel (both tensor-core paths).
