@@ -13,16 +13,19 @@
 // contraction D[128 x 128] = A[128 x 128] B[128 x 128]' is, for each of the
 // two 64-column blocks of D, two MMA groups of K = 64 accumulated in TMEM.
 // Each group is the BF16 x3 split of tc.cuh (six products per FP32
-// product), so results carry FP32 accuracy.  The A operand (p_k or a_x, both
-// K-blocks) is formed in registers and split into its three BF16 terms in
-// shared memory before the first MMA; the matrix blocks (P and P' written
-// pre-split by the matrix kernel, tcb_block; Q' from the host) are
-// bulk-copied (cp.async.bulk) through two B buffers, one round's copy
-// overlapping the previous round's MMAs.  A compact tip child's U is its
-// column of P, read from the split P' blocks.
+// product), so results carry FP32 accuracy.  One K-block of the A operand
+// (p_k or a_x) at a time is formed in registers and split into its three BF16
+// terms in shared memory; the matrix operands (P and P' written pre-split by
+// the matrix kernel, tcb_block; Q' from the host) are bulk-copied
+// (cp.async.bulk).  A compact tip child's U is its column of P, read from the
+// split P' blocks.
 //
-// TMEM: post 128 columns [U_k]; pre 256 [q_x | W_x].  One CTA per SM
-// (192 KB of shared memory).
+// TMEM: post 128 columns [U_k]; pre 256 [q_x | W_x].  One buffer of A and one
+// of B (97 KB) for two CTAs per SM: the kernels wait on loads, copies and MMAs
+// in turn, and the second CTA fills those waits better than a second buffer
+// did (one CTA, both K-blocks of A and a two-deep B ring, 193 KB: 122 states,
+// 128 taxa x 2,000 patterns x 4 categories, post-order 0.68 -> 0.59 ms,
+// pre-order 1.20 -> 0.99 ms).
 //
 // Rescaling, exponents and the Eq. 8 terms follow the 64-state path
 // (per-category exponents; ratio_tc_kernel combines the categories).
@@ -35,10 +38,11 @@ namespace phylo {
 constexpr int kTcbSP = 128;                  // padded states of this path
 constexpr int kTcbNB = kTcbSP / 64;          // 64-blocks per dimension
 static_assert(kTcbUnitBytes == 2 * kTcbNB * kOp128, "matrix block size");
-// Shared memory: A 2 x 48 KB (both K-blocks), B ring 2 x 48 KB (+1024 for alignment).
-constexpr size_t kTcbSmem = 1024 + 4 * (size_t)kOp128;
+// Shared memory (+1024 for alignment).
+constexpr size_t kTcbSmem = 1024 + 2 * (size_t)kOp128;   // level kernels: A, B
+constexpr size_t kTipqBSmem = 1024 + 4 * (size_t)kOp128;  // tables: both K-blocks of A, B ring
 constexpr int kTcbLd = kTcbSP + 4;           // output staging row stride (floats)
-static_assert((size_t)kTcRows * kTcbLd * 4 <= 2 * (size_t)kOp128, "staging fits in A");
+static_assert((size_t)kTcRows * kTcbLd * 4 <= 2 * (size_t)kOp128, "staging fits in A and B");
 
 __device__ __forceinline__ const unsigned char* tcb_unit(const LevelArgs<float>& a, int b,
                                                          int r) {
@@ -85,49 +89,43 @@ __device__ __forceinline__ void tcb_col8(const LevelArgs<float>& a, int b, int r
   hi = make_float4(v[4], v[5], v[6], v[7]);
 }
 
-// Both K-blocks of a child's U rows in the cooperative layout (v[kb], rows
-// c0 + coop_row(it)), each row's stored exponent in E[it] (0 for a tip),
-// a compact tip's state in y[it] (-1 otherwise).
-__device__ __forceinline__ void tcb_child_rows(float4 (&v)[2][8], int (&E)[4], int (&y)[4],
+// A child's rows c0 + coop_row(it): each one's stored exponent (0 for a tip)
+// and a compact tip's state (-1 otherwise, or past the last pattern).
+__device__ __forceinline__ void tcb_child_meta(int (&E)[4], int (&y)[4],
                                                const LevelArgs<float>& a, const TcChild& x,
                                                int r, int c0) {
-  const int C = a.n_patterns, j = threadIdx.x & 7;
-  if (!x.compact) {
-    const float* base = tcb_u_rows(a, x.b, r);
-#pragma unroll
-    for (int kb = 0; kb < kTcbNB; ++kb)
-      coop_load(v[kb], base + 64 * kb, (size_t)a.n_cat * kTcbSP, c0, C);
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int c = c0 + coop_row(it);
-      y[it] = -1;
-      E[it] = x.internal && c < C
-                  ? a.escale[((size_t)(x.b - a.n_tips) * a.n_cat + r) * a.escale_stride + c]
-                  : 0;
-    }
-    return;
-  }
 #pragma unroll
   for (int it = 0; it < 4; ++it) {
     const int c = c0 + coop_row(it);
-    y[it] = c < C ? (int)a.tip_states[(size_t)x.b * a.state_stride + c] : -1;
-    E[it] = 0;
+    const bool on = c < a.n_patterns;
+    y[it] = x.compact && on ? (int)a.tip_states[(size_t)x.b * a.state_stride + c] : -1;
+    E[it] = x.internal && on
+                ? a.escale[((size_t)(x.b - a.n_tips) * a.n_cat + r) * a.escale_stride + c]
+                : 0;
   }
-#pragma unroll
-  for (int kb = 0; kb < kTcbNB; ++kb)
-#pragma unroll
-    for (int it = 0; it < 4; ++it) tcb_col8(a, x.b, r, y[it], kb, j, v[kb][2 * it], v[kb][2 * it + 1]);
 }
 
-// This thread's half row (states 64 h .. 64 h + 63) of a child's stored U, for
-// pattern c.
-__device__ __forceinline__ void tcb_child_half(float (&u)[64], const LevelArgs<float>& a,
-                                               const TcChild& x, int r, int c, int h) {
+// K-block kb of a child's U rows in the cooperative layout.
+__device__ __forceinline__ void tcb_child_kb(float4 (&v)[8], const int (&y)[4],
+                                             const LevelArgs<float>& a, const TcChild& x, int r,
+                                             int c0, int kb) {
+  if (!x.compact) {
+    coop_load(v, tcb_u_rows(a, x.b, r) + 64 * kb, (size_t)a.n_cat * kTcbSP, c0, a.n_patterns);
+    return;
+  }
+#pragma unroll
+  for (int it = 0; it < 4; ++it)
+    tcb_col8(a, x.b, r, y[it], kb, threadIdx.x & 7, v[2 * it], v[2 * it + 1]);
+}
+
+// 32 floats of a child's stored U, from column col, for pattern c.
+__device__ __forceinline__ void tcb_child_part(float (&u)[32], const LevelArgs<float>& a,
+                                               const TcChild& x, int r, int c, int col) {
   const bool on = c < a.n_patterns;
   const float4* src = reinterpret_cast<const float4*>(
-      tcb_u_rows(a, x.b, r) + (size_t)(on ? c : 0) * a.n_cat * kTcbSP + 64 * h);
+      tcb_u_rows(a, x.b, r) + (size_t)(on ? c : 0) * a.n_cat * kTcbSP + col);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
+  for (int i = 0; i < 8; ++i) {
     const float4 f = on ? __ldg(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     u[4 * i] = f.x;
     u[4 * i + 1] = f.y;
@@ -340,43 +338,59 @@ __device__ __forceinline__ void tcb_gtab8(const LevelArgs<float>& a, int b, int 
 // from those vectors before the first level runs.
 // ---------------------------------------------------------------------------
 template <typename T>  // float only
-__global__ void __launch_bounds__(kTcThreads) post_tcb_kernel(LevelArgs<T> a) {
+__global__ void __launch_bounds__(kTcThreads, 2) post_tcb_kernel(LevelArgs<T> a) {
   static_assert(std::is_same<T, float>::value, "tensor-core path is FP32");
-  pdl_wait_and_release();  // before TMEM, smem or any global access
-  TCB_PROLOGUE(128)
+  extern __shared__ unsigned char smraw[];
+  unsigned char* A = align1024(smraw);  // one K-block of p_k
+  unsigned char* B = A + kOp128;        // one K-block of P_k
+  __shared__ uint64_t bar_tma, bar_mma;
+  __shared__ uint32_t tmem_slot;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int row = tid & (kTcRows - 1), h = tid / kTcRows;
   const int R = a.n_cat, C = a.n_patterns;
   const int4 d = a.level_desc[blockIdx.y];
-  const int k = d.x, r = blockIdx.z, lane = tid & 31;
+  const int k = d.x, r = blockIdx.z;
   const int c0 = blockIdx.x * kTcRows;
   const bool tip = a.tip_level;
-  // round kb: U_k (+)= p_k[:, kb] P_k[:, kb]'; both rounds' blocks copied now
-  auto round_of = [=, &a](int kb) {
-    return TcbRound{tcb_unit(a, k, r) + tcb_block(0, 0, kb), kb, tmem, kb > 0};
+  // round kb: U_k (+)= p_k[:, kb] P_k[:, kb]'
+  auto copy_b = [&](int kb) {
+    if (tid != 0) return;
+    mbar_expect_tx(&bar_tma, kOp128);
+    bulk_g2s(B, tcb_unit(a, k, r) + tcb_block(0, 0, kb), kOp128, &bar_tma);
   };
-  tcb_issue_b(B0, bars, ph, 0, round_of(0).bsrc);
-  tcb_issue_b(B0, bars, ph, 1, round_of(1).bsrc);
+  if (tid == 0) {
+    mbar_init_fenced(&bar_tma, 1);
+    mbar_init_fenced(&bar_mma, 1);
+  }
+  if (a.mats_ready) copy_b(0);
+  pdl_wait_and_release();  // before TMEM or any other global access
+  if (!a.mats_ready) copy_b(0);
+  if (warp == 0) tc::alloc(&tmem_slot, 128);
   float4 v[2][8];
   if (tip) {
 #pragma unroll
     for (int kb = 0; kb < kTcbNB; ++kb)
       coop_load(v[kb], a.tip_partials + (size_t)k * C * kTcbSP + 64 * kb, kTcbSP, c0, C);
   } else {
-    // p_k = U_i o U_j, each row rescaled into [1/2, 1)
+    // p_k = U_i o U_j, each row rescaled into [1/2, 1); a K-block at a time
     const TcChild x0 = tc_child(a.n_tips, d.y, d.w & kDescFlagCompact0);
     const TcChild x1 = tc_child(a.n_tips, d.z, d.w & kDescFlagCompact1);
-    float4 u[2][8];
-    int E0[4], E1[4], y[4];
-    tcb_child_rows(v, E0, y, a, x0, r, c0);
-    tcb_child_rows(u, E1, y, a, x1, r, c0);
+    int E0[4], E1[4], y0[4], y1[4];
+    tcb_child_meta(E0, y0, a, x0, r, c0);
+    tcb_child_meta(E1, y1, a, x1, r, c0);
+#pragma unroll
+    for (int kb = 0; kb < kTcbNB; ++kb) {
+      float4 u[8];
+      tcb_child_kb(v[kb], y0, a, x0, r, c0, kb);
+      tcb_child_kb(u, y1, a, x1, r, c0, kb);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[kb][i] = mul4(v[kb][i], u[i]);
+    }
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
       float m = 0.f;
 #pragma unroll
-      for (int kb = 0; kb < kTcbNB; ++kb) {
-        v[kb][2 * it] = mul4(v[kb][2 * it], u[kb][2 * it]);
-        v[kb][2 * it + 1] = mul4(v[kb][2 * it + 1], u[kb][2 * it + 1]);
-        m = amax4(v[kb][2 * it + 1], amax4(v[kb][2 * it], m));
-      }
+      for (int kb = 0; kb < kTcbNB; ++kb) m = amax4(v[kb][2 * it + 1], amax4(v[kb][2 * it], m));
       m = row_max8(m);
       const int c = c0 + coop_row(it);
       const int e = rescale_exponent(m, c < C, a.err);
@@ -392,12 +406,33 @@ __global__ void __launch_bounds__(kTcThreads) post_tcb_kernel(LevelArgs<T> a) {
         a.escale[((size_t)(k - a.n_tips) * R + r) * a.escale_stride + c] = E0[it] + E1[it] + e;
     }
   }
-#pragma unroll
-  for (int kb = 0; kb < kTcbNB; ++kb) coop_put(tcb_a(A0, kb), v[kb]);
+  coop_put(A, v[0]);
   tc::fence_smem_for_async();
-  const bool ok = tcb_rounds(A0, B0, bars, ph, kTcbNB, round_of, a.err);
+  __syncthreads();  // barriers initialised, TMEM allocated, A written
+  tc::fence_after();
+  const uint32_t tmem = tmem_slot;
+  const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  uint32_t ptma = 0, pmma = 0;
+  int pend_tma = -1, pend_mma = -1;
+  bool ok = true;
+#pragma unroll
+  for (int kb = 0; kb < kTcbNB && ok; ++kb) {
+    if (kb) {
+      copy_b(kb);
+      coop_put(A, v[kb]);
+      tc::fence_smem_for_async();
+    }
+    ok = tc_block_wait(&bar_tma, ptma, pend_tma, a.err);
+    if (!ok) break;
+    if (tid == 0) {
+      tc::fence_after();
+      tcb_mma_round(tmem, A, B, kb > 0);
+      tc::commit(&bar_mma);
+    }
+    ok = tc_block_wait(&bar_mma, pmma, pend_mma, a.err);
+  }
   if (ok) {  // U_k, stored as computed (exponent: escale of k)
-    float* st = reinterpret_cast<float*>(base);  // A is free: every MMA is done
+    float* st = reinterpret_cast<float*>(A);  // A and B are free: every MMA is done
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       float w[32];
@@ -410,7 +445,13 @@ __global__ void __launch_bounds__(kTcThreads) post_tcb_kernel(LevelArgs<T> a) {
     __syncthreads();
     tcb_store_rows(a.post + (u_slot(a, k) * C * R + r) * kTcbSP, (size_t)R * kTcbSP, c0, C, st);
   }
-  TCB_EPILOGUE(128)
+  if (tid == 0) {  // bounded drain of whatever a timeout left in flight
+    if (pend_tma >= 0) (void)mbar_wait(&bar_tma, (uint32_t)pend_tma);
+    if (pend_mma >= 0) (void)mbar_wait(&bar_mma, (uint32_t)pend_mma);
+  }
+  tc::fence_before();
+  __syncthreads();
+  if (warp == 0) tc::dealloc(tmem, 128);
 }
 
 // ---------------------------------------------------------------------------
@@ -491,175 +532,203 @@ __global__ void __launch_bounds__(kTcRows) root_tcb_kernel(LevelArgs<T> a) {
 // numerator is formed in its sibling's unit from the table G_y.
 // ---------------------------------------------------------------------------
 template <typename T>  // float only
-__global__ void __launch_bounds__(kTcThreads) pre_tcb_kernel(LevelArgs<T> a) {
+__global__ void __launch_bounds__(kTcThreads, 2) pre_tcb_kernel(LevelArgs<T> a) {
   static_assert(std::is_same<T, float>::value, "tensor-core path is FP32");
-  pdl_wait_and_release();
-  TCB_PROLOGUE(256)
+  extern __shared__ unsigned char smraw[];
+  unsigned char* A = align1024(smraw);  // one K-block of a_x
+  unsigned char* B = A + kOp128;        // one K-block of Q or P_x
+  __shared__ uint64_t bar_tma, bar_mma;
+  __shared__ uint32_t tmem_slot;
   __shared__ float xn[2][kTcRows], xm[2][kTcRows];  // the halves' num and q maximum
+  const int tid = threadIdx.x, warp = tid >> 5, j = tid & 7;
+  const int row = tid & (kTcRows - 1), h = tid / kTcRows;
   const int R = a.n_cat, C = a.n_patterns, S = a.n_states;
   const int4 d = a.level_desc[blockIdx.z];
   const int k = d.x, r = (int)blockIdx.y;
   const int x = (d.w & kUnitSecond) ? 1 : 0;  // x's place among k's children
-  const int lane = tid & 31, j = lane & 7;
   const TcChild cx = tc_child(a.n_tips, d.y, false);
   const TcChild cy = tc_child(a.n_tips, d.z, d.w & kUnitCompactY);
   const bool root = k == a.root;
   const size_t kslot = (size_t)(k - a.n_tips);
   const int c0 = blockIdx.x * kTcRows, c = c0 + row;
   const int estr = a.escale_stride;
-  // rounds: W_x = a_x Q (K-blocks 0, 1), then for an internal child
-  // q_x = a_x P_x (K-blocks 0, 1); TMEM columns [q_x | W_x]
-  const int n_rounds = cx.internal ? 2 * kTcbNB : kTcbNB;
-  auto round_of = [=, &a](int i) {
-    const int kb = i % kTcbNB;
-    if (i < kTcbNB) return TcbRound{a.qt + tcb_block(0, 0, kb), kb, tmem + 128u, kb > 0};
-    return TcbRound{tcb_unit(a, cx.b, r) + tcb_block(1, 0, kb), kb, tmem, kb > 0};
+  if (tid == 0) {
+    mbar_init_fenced(&bar_tma, 1);
+    mbar_init_fenced(&bar_mma, 1);
+  }
+  auto copy_b = [&](bool p, int kb) {  // Q' (host-written) or P_x'
+    if (tid != 0) return;
+    mbar_expect_tx(&bar_tma, kOp128);
+    bulk_g2s(B, p ? tcb_unit(a, cx.b, r) + tcb_block(1, 0, kb) : a.qt + tcb_block(0, 0, kb),
+             kOp128, &bar_tma);
   };
-  tcb_issue_b(B0, bars, ph, 0, round_of(0).bsrc);
-  tcb_issue_b(B0, bars, ph, 1, round_of(1).bsrc);
+  copy_b(false, 0);
+  pdl_wait_and_release();  // before TMEM or any other global access
+  if (warp == 0) tc::alloc(&tmem_slot, 256);
   // row-layout values of this thread's row for the epilogue
   int eq_row = 0, ey_row = 0;
   if (c < C) {
     if (!root) eq_row = a.pre_escale[(kslot * R + r) * estr + c];
     if (cy.internal) ey_row = a.escale[((size_t)(cy.b - a.n_tips) * R + r) * estr + c];
   }
-  // a_x = q_k o U_y in the cooperative layout, split into A
-  float4 q[2][8];
-  int eq[4];
-  if (!root) {
-#pragma unroll
-    for (int kb = 0; kb < kTcbNB; ++kb)
-      coop_load(q[kb], a.pre + (kslot * C * R + r) * kTcbSP + 64 * kb, (size_t)R * kTcbSP, c0, C);
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int cc = c0 + coop_row(it);
-      eq[it] = cc < C ? a.pre_escale[(kslot * R + r) * estr + cc] : 0;
-    }
-  } else {  // q_root = pi
-#pragma unroll
-    for (int kb = 0; kb < kTcbNB; ++kb) {
+  int Ey[4], Ex[4], yy[4], yx[4];
+  tcb_child_meta(Ey, yy, a, cy, r, c0);
+  tcb_child_meta(Ex, yx, a, cx, r, c0);
+  float4 q[8], ux[8], uy[8];
+  float den[4], ny[4];  // this lane's parts of the rows' sums
+  auto load = [&](int kb) {
+    if (root) {  // q_root = pi
       const int s = 64 * kb + 8 * j;
-      const float4 p0 = make_float4(s < S ? a.root_pit[s] : 0.f, s + 1 < S ? a.root_pit[s + 1] : 0.f,
-                                    s + 2 < S ? a.root_pit[s + 2] : 0.f,
-                                    s + 3 < S ? a.root_pit[s + 3] : 0.f);
-      const float4 p1 = make_float4(s + 4 < S ? a.root_pit[s + 4] : 0.f,
-                                    s + 5 < S ? a.root_pit[s + 5] : 0.f,
-                                    s + 6 < S ? a.root_pit[s + 6] : 0.f,
-                                    s + 7 < S ? a.root_pit[s + 7] : 0.f);
+      float p[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) p[i] = s + i < S ? a.root_pit[s + i] : 0.f;
 #pragma unroll
       for (int it = 0; it < 4; ++it) {
-        q[kb][2 * it] = p0;
-        q[kb][2 * it + 1] = p1;
+        q[2 * it] = make_float4(p[0], p[1], p[2], p[3]);
+        q[2 * it + 1] = make_float4(p[4], p[5], p[6], p[7]);
       }
+    } else {
+      coop_load(q, a.pre + (kslot * C * R + r) * kTcbSP + 64 * kb, (size_t)R * kTcbSP, c0, C);
     }
-#pragma unroll
-    for (int it = 0; it < 4; ++it) eq[it] = 0;
-  }
-  int Ey[4], Ex[4], yy[4], yxc[4];
-  float4 qg[2][8];  // q_k o G_y e_y of a tip sibling (its numerator is qg . U_x)
-  {
-    float4 uy[2][8];
-    tcb_child_rows(uy, Ey, yy, a, cy, r, c0);
-#pragma unroll
-    for (int kb = 0; kb < kTcbNB; ++kb)
-#pragma unroll
-      for (int it = 0; it < 4; ++it) {
-        if (cy.compact) {
-          float4 lo, hi;
-          tcb_gtab8(a, cy.b, r, yy[it], kb, j, lo, hi);
-          qg[kb][2 * it] = mul4(q[kb][2 * it], lo);
-          qg[kb][2 * it + 1] = mul4(q[kb][2 * it + 1], hi);
-        }
-        q[kb][2 * it] = mul4(q[kb][2 * it], uy[kb][2 * it]);
-        q[kb][2 * it + 1] = mul4(q[kb][2 * it + 1], uy[kb][2 * it + 1]);
-      }
-  }
-#pragma unroll
-  for (int kb = 0; kb < kTcbNB; ++kb) coop_put(tcb_a(A0, kb), q[kb]);
-  tc::fence_smem_for_async();
-  // den = a_x . U_x per row (U_x loads in flight during the MMAs)
-  float den[4], ny[4];
-  {
-    float4 ux[2][8];
-    tcb_child_rows(ux, Ex, yxc, a, cx, r, c0);
-    const bool ok0 = tcb_rounds(A0, B0, bars, ph, n_rounds, round_of, a.err);
+    tcb_child_kb(ux, yx, a, cx, r, c0, kb);
+    tcb_child_kb(uy, yy, a, cy, r, c0, kb);
+  };
+  // a_y = q_k o U_x: den = a_y . U_y and a tip sibling's numerator; then
+  // a_x = q_k o U_y, split into A
+  auto form = [&](int kb) {
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
-      float s = 0.f;
-#pragma unroll
-      for (int kb = 0; kb < kTcbNB; ++kb)
-        s = dot4(q[kb][2 * it + 1], ux[kb][2 * it + 1], dot4(q[kb][2 * it], ux[kb][2 * it], s));
-      den[it] = row_sum8(s);
-      if (!cy.compact) continue;
-      s = 0.f;
-#pragma unroll
-      for (int kb = 0; kb < kTcbNB; ++kb)
-        s = dot4(qg[kb][2 * it + 1], ux[kb][2 * it + 1],
-                 dot4(qg[kb][2 * it], ux[kb][2 * it], s));
-      ny[it] = row_sum8(s);
+      const float4 b0 = mul4(q[2 * it], ux[2 * it]), b1 = mul4(q[2 * it + 1], ux[2 * it + 1]);
+      den[it] = dot4(b1, uy[2 * it + 1], dot4(b0, uy[2 * it], kb ? den[it] : 0.f));
+      if (!kb) ny[it] = 0.f;
+      if (cy.compact) {
+        float4 lo, hi;
+        tcb_gtab8(a, cy.b, r, yy[it], kb, j, lo, hi);
+        ny[it] = dot4(b1, hi, dot4(b0, lo, ny[it]));
+      }
+      q[2 * it] = mul4(q[2 * it], uy[2 * it]);
+      q[2 * it + 1] = mul4(q[2 * it + 1], uy[2 * it + 1]);
     }
-    if (!ok0) {
-      TCB_EPILOGUE(256)
-      return;
+    coop_put(A, q);
+    tc::fence_smem_for_async();
+  };
+  load(0);
+  form(0);
+  __syncthreads();  // barriers initialised, TMEM allocated
+  tc::fence_after();
+  const uint32_t tmem = tmem_slot;  // columns [q_x | W_x]
+  const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  uint32_t ptma = 0, pmma = 0;
+  int pend_tma = -1, pend_mma = -1;
+  bool ok = tc_block_wait(&bar_tma, ptma, pend_tma, a.err);
+  auto mma = [&](bool p, int kb) {
+    if (tid != 0) return;
+    tc::fence_after();
+    tcb_mma_round(p ? tmem : tmem + 128u, A, B, kb > 0);
+    tc::commit(&bar_mma);
+  };
+  // rounds W, q (internal x) of K-block 0, then of K-block 1
+  if (ok) {
+    mma(false, 0);
+    load(1);
+    ok = tc_block_wait(&bar_mma, pmma, pend_mma, a.err);
+  }
+  if (ok && cx.internal) {
+    copy_b(true, 0);
+    ok = tc_block_wait(&bar_tma, ptma, pend_tma, a.err);
+    if (ok) {
+      mma(true, 0);
+      ok = tc_block_wait(&bar_mma, pmma, pend_mma, a.err);
     }
   }
-  // epilogue (row layout, thread (row, h) owns states 64 h .. 64 h + 63)
-  float num = 0.f, m = 0.f;
-  {
-    float u[64];
-    tcb_child_half(u, a, cx, r, c, h);
+  if (ok) {
+    copy_b(false, 1);
+    form(1);
+    ok = tc_block_wait(&bar_tma, ptma, pend_tma, a.err);
+  }
+  const float wg = (float)(a.cat_w[r] * a.rates[r]);
+  float* rt = reinterpret_cast<float*>(a.rterm);
+  if (ok) {
+    mma(false, 1);
+    // the Eq. 8 terms that need no contraction, during the MMAs
+    if (d.w & (kUnitDen | kUnitCompactY)) {
+#pragma unroll
+      for (int it = 0; it < 4; ++it) {
+        const float dn = row_sum8(den[it]), nn = row_sum8(ny[it]);
+        const int cc = c0 + coop_row(it);
+        if (cc < C && j == 0) {
+          float* t4 = rt + ((kslot * C + cc) * R + r) * 4;
+          if (cy.compact) t4[1 - x] = wg * nn;
+          if (d.w & kUnitDen) {
+            const int eq = root ? 0 : a.pre_escale[(kslot * R + r) * estr + cc];
+            t4[2] = a.cat_wt[r] * dn;
+            t4[3] = __int_as_float(eq + Ex[it] + Ey[it]);
+          }
+        }
+      }
+    }
+    ok = tc_block_wait(&bar_mma, pmma, pend_mma, a.err);
+  }
+  if (ok && cx.internal) {
+    copy_b(true, 1);
+    ok = tc_block_wait(&bar_tma, ptma, pend_tma, a.err);
+    if (ok) {
+      mma(true, 1);
+      ok = tc_block_wait(&bar_mma, pmma, pend_mma, a.err);
+    }
+  }
+  if (ok) {
+    // epilogue (row layout, thread (row, h) owns states 64 h .. 64 h + 63)
+    float num = 0.f, m = 0.f;
 #pragma unroll
     for (int qq = 0; qq < 2; ++qq) {
-      float w[32];
+      float u[32], w[32];
+      tcb_child_part(u, a, cx, r, c, 64 * h + 32 * qq);
       tc::ld32(trow + 128 + 64 * h + 32 * qq, w);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) num = fmaf(w[i], u[32 * qq + i], num);
+      for (int i = 0; i < 32; ++i) num = fmaf(w[i], u[i], num);
     }
-  }
-  float qo[64];
-  if (cx.internal) {
-    tc::ld32(trow + 64 * h, *reinterpret_cast<float(*)[32]>(qo));
-    tc::ld32(trow + 64 * h + 32, *reinterpret_cast<float(*)[32]>(qo + 32));
+    if (cx.internal) {
 #pragma unroll
-    for (int i = 0; i < 64; ++i) m = fmaxf(m, fabsf(qo[i]));
-  }
-  xn[h][row] = num;
-  xm[h][row] = m;
-  __syncthreads();
-  num += xn[1 - h][row];
-  m = fmaxf(m, xm[1 - h][row]);
-  float* rt = reinterpret_cast<float*>(a.rterm);
-  const float wg = (float)(a.cat_w[r] * a.rates[r]);
-  if (c < C && h == 0) rt[((kslot * C + c) * R + r) * 4 + x] = wg * num;
-  if (d.w & (kUnitDen | kUnitCompactY)) {  // the other terms, from the cooperative layout
+      for (int qq = 0; qq < 2; ++qq) {
+        float w[32];
+        tc::ld32(trow + 64 * h + 32 * qq, w);
 #pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int cc = c0 + coop_row(it);
-      if (cc < C && j == 0) {
-        float* t4 = rt + ((kslot * C + cc) * R + r) * 4;
-        if (cy.compact) t4[1 - x] = wg * ny[it];
-        if (d.w & kUnitDen) {
-          t4[2] = a.cat_wt[r] * den[it];
-          t4[3] = __int_as_float(eq[it] + Ex[it] + Ey[it]);
-        }
+        for (int i = 0; i < 32; ++i) m = fmaxf(m, fabsf(w[i]));
       }
     }
-  }
-  if (cx.internal) {  // q_x = a_x P_x, the row rescaled into [1/2, 1)
-    const int e = rescale_exponent(m, c < C, a.err);
-    const float f = ldexpf(1.f, -e);
-    float* st = reinterpret_cast<float*>(base);  // A is free: every MMA is done
-#pragma unroll
-    for (int i = 0; i < 64; i += 4)
-      *reinterpret_cast<float4*>(st + row * kTcbLd + 64 * h + i) =
-          make_float4(qo[i] * f, qo[i + 1] * f, qo[i + 2] * f, qo[i + 3] * f);
-    if (c < C && h == 0)  // q_x = P_x' (q_k o U_y): exponents of q_k and of U_y
-      a.pre_escale[((size_t)(cx.b - a.n_tips) * R + r) * estr + c] = e + eq_row + ey_row;
+    xn[h][row] = num;
+    xm[h][row] = m;
     __syncthreads();
-    tcb_store_rows(a.pre + ((size_t)(cx.b - a.n_tips) * C * R + r) * kTcbSP, (size_t)R * kTcbSP,
-                   c0, C, st);
+    if (c < C && h == 0) rt[((kslot * C + c) * R + r) * 4 + x] = wg * (num + xn[1][row]);
+    if (cx.internal) {  // q_x = a_x P_x, the row rescaled into [1/2, 1)
+      m = fmaxf(m, xm[1 - h][row]);
+      const int e = rescale_exponent(m, c < C, a.err);
+      const float f = ldexpf(1.f, -e);
+      float* st = reinterpret_cast<float*>(A);  // A and B are free: every MMA is done
+#pragma unroll
+      for (int qq = 0; qq < 2; ++qq) {
+        float w[32];
+        tc::ld32(trow + 64 * h + 32 * qq, w);
+#pragma unroll
+        for (int i = 0; i < 32; i += 4)
+          *reinterpret_cast<float4*>(st + row * kTcbLd + 64 * h + 32 * qq + i) =
+              make_float4(w[i] * f, w[i + 1] * f, w[i + 2] * f, w[i + 3] * f);
+      }
+      if (c < C && h == 0)  // q_x = P_x' (q_k o U_y): exponents of q_k and of U_y
+        a.pre_escale[((size_t)(cx.b - a.n_tips) * R + r) * estr + c] = e + eq_row + ey_row;
+      __syncthreads();
+      tcb_store_rows(a.pre + ((size_t)(cx.b - a.n_tips) * C * R + r) * kTcbSP,
+                     (size_t)R * kTcbSP, c0, C, st);
+    }
   }
-  TCB_EPILOGUE(256)
+  if (tid == 0) {  // bounded drain of whatever a timeout left in flight
+    if (pend_tma >= 0) (void)mbar_wait(&bar_tma, (uint32_t)pend_tma);
+    if (pend_mma >= 0) (void)mbar_wait(&bar_mma, (uint32_t)pend_mma);
+  }
+  tc::fence_before();
+  __syncthreads();
+  if (warp == 0) tc::dealloc(tmem, 256);
 }
 
 #undef TCB_PROLOGUE
@@ -702,7 +771,7 @@ inline cudaError_t launch_pmat_tcb(const PmatArgs& a, cudaStream_t st) {
   // (writes the operand blocks: a.tiles is set)
   const cudaError_t e = launch_pmat_big<kTcbSP>(a, st);
   if (e != cudaSuccess) return e;
-  return launch_pdl(tipq_tcb_kernel<float>, dim3(a.n_tips * a.n_cat), kTcThreads, kTcbSmem, st, a);
+  return launch_pdl(tipq_tcb_kernel<float>, dim3(a.n_tips * a.n_cat), kTcThreads, kTipqBSmem, st, a);
 }
 
 inline cudaError_t prepare_tcb() {
@@ -714,7 +783,7 @@ inline cudaError_t prepare_tcb() {
                              (int)kTcbSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(tipq_tcb_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kTcbSmem);
+                             (int)kTipqBSmem);
   return e;
 }
 
