@@ -560,7 +560,10 @@ __device__ __forceinline__ double tcd_scale(double x, int e) {
 
 // ---------------------------------------------------------------------------
 // Pre-order level (Eq. 4) with the per-category Eq. 8 terms: one CTA per
-// (tile, unit (pre_units), category).  rterm holds
+// (tile, node k, category r, child x); blockIdx.z = 2 r + x.  (The FP32 path's
+// units, which form a tip's numerator in its sibling's CTA, lost here: the
+// elementwise FP64 products bound a CTA, and the tips' are better on SMs of
+// their own: pre-order of 64 taxa x 570 patterns 0.46 -> 0.57 ms.)  rterm holds
 // {w_r num_i, w_r num_j, w_r den, exponent} per (node, pattern, category).
 // ---------------------------------------------------------------------------
 template <typename T>  // double only
@@ -574,10 +577,11 @@ __global__ void __launch_bounds__(kTcdThreads) pre_tcd_kernel(LevelArgs<T> a) {
   __shared__ int ecol[64], ecol_p[64];  // column exponents of Q and P_x
   const int tid = threadIdx.x, warp = tid >> 5, j = tid & 7;
   const int R = a.n_cat, C = a.n_patterns, S = a.n_states;
-  const int4 d = a.level_desc[blockIdx.z];  // a unit (pre_units)
-  const int k = d.x, r = (int)blockIdx.y, bx = d.y, by = d.z;
-  const int x = (d.w & kUnitSecond) ? 1 : 0;  // x's place among k's children
-  const bool cy = d.w & kUnitCompactY;
+  const int4 d = a.level_desc[blockIdx.y];
+  const int k = d.x, x = (int)(blockIdx.z & 1), r = (int)(blockIdx.z >> 1);
+  const int bx = x ? d.z : d.y, by = x ? d.y : d.z;
+  const bool cx = d.w & (x ? kDescFlagCompact1 : kDescFlagCompact0);
+  const bool cy = d.w & (x ? kDescFlagCompact0 : kDescFlagCompact1);
   const bool internal = bx >= a.n_tips;  // only these need contractions
   const size_t kslot = (size_t)(k - a.n_tips), xslot = (size_t)(bx - a.n_tips);
   const int c0 = blockIdx.x * 128, estr = a.escale_stride;
@@ -593,10 +597,11 @@ __global__ void __launch_bounds__(kTcdThreads) pre_tcd_kernel(LevelArgs<T> a) {
   if (internal && warp == 0) tc::alloc(&bars.tmem, 512);
   if (internal && tid < 64)
     ecol_p[tid] = reinterpret_cast<const int*>(tcd_unit(a, bx, r) + 2 * kTcdB)[tid];
-  double av[2][8], u[2][8], b[2][8];  // q_k, then a_x; U_x, then others; a_y = q_k o U_x
-  int y[2], ey[2] = {0, 0}, ex[2] = {0, 0}, eq[2];
+  double av[2][8], u[2][8];
+  int y[2], ey[2], ex[2], eq[2];
+  tcd_child(a, by, cy, r, c0, false, u, y, ey);
 #pragma unroll
-  for (int it = 0; it < 2; ++it) {
+  for (int it = 0; it < 2; ++it) {  // a_x = q_k o U_y
     const int c = c0 + tcd_row(it);
     eq[it] = 0;
     if (k == a.root) {
@@ -609,6 +614,8 @@ __global__ void __launch_bounds__(kTcdThreads) pre_tcd_kernel(LevelArgs<T> a) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) av[it][i] = 0.0;
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) av[it][i] *= u[it][i];
   }
   double* rt = static_cast<double*>(a.rterm);
   const double wr = a.cat_w[r];
@@ -616,36 +623,21 @@ __global__ void __launch_bounds__(kTcdThreads) pre_tcd_kernel(LevelArgs<T> a) {
   const int crow = c0 + tcd_row(0) + 64 * mit;
   const bool mine = (j >> 1) == 0 && crow < C;  // lanes j = 0, 1 write
   double* mine_t = rt + ((kslot * C + (mine ? crow : 0)) * R + r) * 4;
-  const bool den = d.w & kUnitDen;
-  if (den) {
-    tcd_child(a, bx, false, r, c0, false, u, y, ex);
-#pragma unroll
-    for (int it = 0; it < 2; ++it)
-#pragma unroll
-      for (int i = 0; i < 8; ++i) b[it][i] = av[it][i] * u[it][i];
-    if (cy) {  // num_y = a_y . (column of dP_y)
-      tcd_child(a, by, true, r, c0, true, u, y, ey);
-      const double s = tcd_row_sums(tcd_dot8(b[0], u[0]), tcd_dot8(b[1], u[1]));
-      if (mine) mine_t[1 - x] = wr * s;
+  if (x == 0 || !internal) {
+    if (x == 0) {  // den = a_x . U_x
+      tcd_child(a, bx, cx, r, c0, false, u, y, ex);
+      const double s = tcd_row_sums(tcd_dot8(av[0], u[0]), tcd_dot8(av[1], u[1]));
+      if (mine) {
+        mine_t[2] = wr * s;
+        mine_t[3] = (double)(mit ? eq[1] + ex[1] + ey[1] : eq[0] + ex[0] + ey[0]);
+      }
     }
-  }
-  tcd_child(a, by, cy, r, c0, false, u, y, ey);
-  if (den) {  // den = a_y . U_y
-    const double s = tcd_row_sums(tcd_dot8(b[0], u[0]), tcd_dot8(b[1], u[1]));
-    if (mine) {
-      mine_t[2] = wr * s;
-      mine_t[3] = (double)(mit ? eq[1] + ex[1] + ey[1] : eq[0] + ex[0] + ey[0]);
+    if (!internal) {  // num_x = a_x . (column of dP_x, or dP_x v)
+      tcd_child(a, bx, cx, r, c0, true, u, y, ex);
+      const double s = tcd_row_sums(tcd_dot8(av[0], u[0]), tcd_dot8(av[1], u[1]));
+      if (mine) mine_t[x] = wr * s;
+      return;  // block-uniform: no barrier, copy or TMEM is in use
     }
-  }
-#pragma unroll
-  for (int it = 0; it < 2; ++it)
-#pragma unroll
-    for (int i = 0; i < 8; ++i) av[it][i] *= u[it][i];  // a_x = q_k o U_y
-  if (!internal) {  // num_x = a_x . (column of dP_x, or dP_x v)
-    tcd_child(a, bx, false, r, c0, true, u, y, ex);
-    const double s = tcd_row_sums(tcd_dot8(av[0], u[0]), tcd_dot8(av[1], u[1]));
-    if (mine) mine_t[x] = wr * s;
-    return;  // block-uniform: no barrier, copy or TMEM is in use
   }
   // ---- internal child: [W_x; q_x] = a_x [Q; P_x], a_x normalised per row ----
   int ea[2];
@@ -737,50 +729,6 @@ __global__ void __launch_bounds__(kTcdThreads) pre_tcd_kernel(LevelArgs<T> a) {
   if (warp == 0) tc::dealloc(tmem, 512);
 }
 
-// Nodes whose children are both compact tips, after the last level: one block
-// per (tile, node, category).
-template <typename T>  // double only
-__global__ void __launch_bounds__(kTcdThreads) cherry_tcd_kernel(LevelArgs<T> a) {
-  pdl_wait_and_release();
-  const int R = a.n_cat, C = a.n_patterns, S = a.n_states, j = threadIdx.x & 7;
-  const int4 d = a.level_desc[blockIdx.z];
-  const int k = d.x, r = (int)blockIdx.y, c0 = blockIdx.x * 128;
-  const size_t kslot = (size_t)(k - a.n_tips);
-  double q[2][8], b[2][8], u[2][8], v[2][8];
-  int y[2], e[2], eq[2] = {0, 0};
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const int c = c0 + tcd_row(it);
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-      q[it][i] = k == a.root && 8 * j + i < S ? a.root_pi[8 * j + i] : 0.0;
-    if (k != a.root && c < C) {
-      tcd_load8(a.pre + ((kslot * C + c) * R + r) * 64 + 8 * j, q[it]);
-      eq[it] = a.pre_escale[(kslot * R + r) * a.escale_stride + c];
-    }
-  }
-  tcd_child(a, d.y, true, r, c0, false, u, y, e);
-  tcd_child(a, d.z, true, r, c0, false, v, y, e);
-#pragma unroll
-  for (int it = 0; it < 2; ++it)
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      b[it][i] = q[it][i] * u[it][i];  // a_j
-      q[it][i] *= v[it][i];            // a_i
-    }
-  const double den = tcd_row_sums(tcd_dot8(b[0], v[0]), tcd_dot8(b[1], v[1]));
-  tcd_child(a, d.y, true, r, c0, true, u, y, e);
-  const double ni = tcd_row_sums(tcd_dot8(q[0], u[0]), tcd_dot8(q[1], u[1]));
-  tcd_child(a, d.z, true, r, c0, true, u, y, e);
-  const double nj = tcd_row_sums(tcd_dot8(b[0], u[0]), tcd_dot8(b[1], u[1]));
-  const int c = c0 + tcd_row(0) + 64 * (j & 1);
-  if (j > 1 || c >= C) return;
-  double2* t = static_cast<double2*>(a.rterm) + ((kslot * C + c) * R + r) * 2;
-  const double wr = a.cat_w[r];
-  t[0] = make_double2(wr * ni, wr * nj);
-  t[1] = make_double2(wr * den, (double)(j ? eq[1] : eq[0]));
-}
-
 // Eq. 8 ratios and their per-tile sums (Eq. 7), from the per-category terms.
 template <typename T>  // double only
 __global__ void __launch_bounds__(128) ratio_tcd_kernel(LevelArgs<T> a) {
@@ -834,18 +782,13 @@ inline cudaError_t launch_tcd(const LevelArgs<double>& a, bool post, cudaStream_
   if (post)
     return launch_pdl(post_tcd_kernel<double>, dim3(a.n_tiles, a.n_level, a.n_cat), kTcdThreads,
                       kTcdSmem, st, a);
-  return launch_pdl(pre_tcd_kernel<double>, dim3(a.n_tiles, a.n_cat, a.n_level), kTcdThreads,
+  return launch_pdl(pre_tcd_kernel<double>, dim3(a.n_tiles, a.n_level, 2 * a.n_cat), kTcdThreads,
                     kTcdSmem, st, a);
 }
 
 template <typename T = double>
 inline cudaError_t launch_ratio_tcd(const LevelArgs<double>& a, cudaStream_t st) {
   if (a.n_tiles <= 0 || a.n_tips < 2) return cudaSuccess;
-  if (a.n_level > 0) {
-    const cudaError_t e = launch_pdl(cherry_tcd_kernel<double>,
-                                     dim3(a.n_tiles, a.n_cat, a.n_level), kTcdThreads, 0, st, a);
-    if (e != cudaSuccess) return e;
-  }
   return launch_pdl(ratio_tcd_kernel<double>, dim3(a.n_tiles, a.n_tips - 1), 128, 0, st, a);
 }
 

@@ -107,9 +107,9 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
   ok &= add_region(L, L.post_nodes, n_int * sizeof(int));
   ok &= add_region(L, L.pre_nodes, n_int * sizeof(int));
   ok &= add_region(L, L.post_desc, n_int * sizeof(int4));
-  // (units on the tensor-core paths: up to two per node)
+  // (units on the FP32 tensor-core paths: up to two per node)
   ok &= add_region(L, L.pre_desc,
-                   n_int * sizeof(int4) * (uses_tc_terms(L.SP, prec == PHYLO_FP64) ? 2 : 1));
+                   n_int * sizeof(int4) * (uses_units(L.SP, prec == PHYLO_FP64) ? 2 : 1));
   if (L.mode != kByLevel) {
     ok &= add_region(L, L.post_off, (n_int + 1) * sizeof(int));
     ok &= add_region(L, L.pre_off, (n_int + 1) * sizeof(int));
@@ -214,7 +214,7 @@ struct phylo_ctx {
   std::vector<int2> children;
   std::vector<int> post_nodes, post_off;  // level l: [post_off[l], post_off[l+1])
   std::vector<int> pre_nodes, pre_off;
-  std::vector<int> unit_off;  // tensor-core paths: the same offsets in pre-order
+  std::vector<int> unit_off;  // FP32 tensor-core paths: the same offsets in pre-order
                               // units, then the nodes with two compact tips
   int n_post_levels = 0, n_pre_levels = 0;    // the level schedule's length
   std::vector<char> post_cherry, pre_cherry;  // per level: a node has a fused cherry child
@@ -448,7 +448,7 @@ cudaError_t enqueue_phase(phylo_ctx* ctx, int phase, cudaStream_t st) {
     // (The tips' tables are built by a launch of their own in between.)
     bool after_pmat =
         post && !ctx->L.qn.bytes && !(ctx->L.tip_desc.bytes && a.tip_partials);
-    const bool units = !post && uses_tc_terms(ctx->L.SP, ctx->precision == PHYLO_FP64);
+    const bool units = !post && uses_units(ctx->L.SP, ctx->precision == PHYLO_FP64);
     for (size_t l = 0; l + 1 < off.size(); ++l) {
       NvtxRange range(post ? "phylo post-order level (Eq. 2)"
                            : "phylo pre-order level (Eqs. 4, 8)", (int)l);
@@ -644,7 +644,7 @@ int upload_descriptors(phylo_ctx* ctx) {
   for (int pass = 0; pass < 2; ++pass) {
     const std::vector<int>& nodes = pass == 0 ? ctx->post_nodes : ctx->pre_nodes;
     std::vector<int4> desc(nodes.size());
-    if (pass == 1 && uses_tc_terms(ctx->L.SP, ctx->precision == PHYLO_FP64)) {
+    if (pass == 1 && uses_units(ctx->L.SP, ctx->precision == PHYLO_FP64)) {
       desc.clear();
       ctx->unit_off.assign(1, 0);
       for (size_t l = 0; l + 1 < ctx->pre_off.size(); ++l) {

@@ -17,12 +17,13 @@ namespace phylo {
 constexpr int kDescFlagCompact0 = 1, kDescFlagCompact1 = 2;
 constexpr int kDescFlagCherry0 = 4, kDescFlagCherry1 = 8;
 
-// Pre-order units of the tensor-core paths: {k, child x, sibling y, flags}.
+// Pre-order units of the FP32 tensor-core paths: {k, child x, sibling y, flags}.
 // A unit contracts the a of a child that is internal or has partial vectors;
 // a compact tip's numerator is a table lookup in its sibling's unit.  A node
 // whose children are both compact tips has none: its terms are lookups only,
 // which nothing waits for, and follow after the last level, for all such nodes
 // in one launch.
+inline bool uses_units(int SP, bool fp64) { return (SP == 64 || SP == 128) && !fp64; }
 constexpr int kUnitCompactY = 1;  // y is a compact tip
 constexpr int kUnitSecond = 2;    // x is child 1 of k
 constexpr int kUnitDen = 4;       // writes the denominator
@@ -366,7 +367,7 @@ struct LevelArgs {
   const int2* children;        // [2N-1]; (-1,-1) for tips
   const int* level_nodes;      // internal nodes of this level
   const int4* level_desc;      // per level node: {k, child 0, child 1, flags}; the
-                               // pre-order pass of the tensor-core paths: units
+                               // pre-order pass of the FP32 tensor-core paths: units
   int n_level;                 // number of nodes (units) in the level
   int root_level;              // 1 if the level is the root alone
   int level_cherry;            // 1 if a node of the level has a fused cherry child
