@@ -849,9 +849,14 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
   const double cw = a.cat_w[r], rate = a.rates[r];  // used in the epilogue
   const float wr = a.cat_wt[r];
   if (a.mats_ready) issue_operands();
+  // So are the children's U: the post-order pass that wrote them ended with
+  // its root level, at least one launch back; only q_k comes from the launch
+  // before.  Every global load is issued before the first wait on a copy.
+  UFetch fx, fy;
+  coop_child_u_issue(fx, a, cx, r, c0);
+  coop_child_u_issue(fy, a, cy, r, c0);
   pdl_wait_and_release();  // before TMEM or any other global access
   if (!a.mats_ready) issue_operands();
-  // every global load is issued before the first wait
   float4 q[8];
   int eq[4];
   if (!root) {
@@ -877,9 +882,6 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
       eq[it] = 0;
     }
   }
-  UFetch fx, fy;
-  coop_child_u_issue(fx, a, cx, r, c0);
-  coop_child_u_issue(fy, a, cy, r, c0);
   if (warp == 0) tc::alloc(&tmem_slot, 128);
   __syncthreads();  // barriers initialised, TMEM allocated
   tc::fence_after();

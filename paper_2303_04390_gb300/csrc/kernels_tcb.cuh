@@ -563,6 +563,19 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_tcb_kernel(LevelArgs<T> a) 
              kOp128, &bar_tma);
   };
   copy_b(false, 0);
+  // The children's U and exponents are read before the wait: the post-order
+  // pass that wrote them ended with its root level, at least one launch back;
+  // only q_k comes from the launch before.
+  int Ey[4], Ex[4], yy[4], yx[4];
+  tcb_child_meta(Ey, yy, a, cy, r, c0);
+  tcb_child_meta(Ex, yx, a, cx, r, c0);
+  float4 q[8], ux[8], uy[8];
+  float den[4], ny[4];  // this lane's parts of the rows' sums
+  auto load_u = [&](int kb) {
+    tcb_child_kb(ux, yx, a, cx, r, c0, kb);
+    tcb_child_kb(uy, yy, a, cy, r, c0, kb);
+  };
+  load_u(0);
   pdl_wait_and_release();  // before TMEM or any other global access
   if (warp == 0) tc::alloc(&tmem_slot, 256);
   // row-layout values of this thread's row for the epilogue
@@ -571,12 +584,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_tcb_kernel(LevelArgs<T> a) 
     if (!root) eq_row = a.pre_escale[(kslot * R + r) * estr + c];
     if (cy.internal) ey_row = a.escale[((size_t)(cy.b - a.n_tips) * R + r) * estr + c];
   }
-  int Ey[4], Ex[4], yy[4], yx[4];
-  tcb_child_meta(Ey, yy, a, cy, r, c0);
-  tcb_child_meta(Ex, yx, a, cx, r, c0);
-  float4 q[8], ux[8], uy[8];
-  float den[4], ny[4];  // this lane's parts of the rows' sums
-  auto load = [&](int kb) {
+  auto load_q = [&](int kb) {
     if (root) {  // q_root = pi
       const int s = 64 * kb + 8 * j;
       float p[8];
@@ -590,8 +598,6 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_tcb_kernel(LevelArgs<T> a) 
     } else {
       coop_load(q, a.pre + (kslot * C * R + r) * kTcbSP + 64 * kb, (size_t)R * kTcbSP, c0, C);
     }
-    tcb_child_kb(ux, yx, a, cx, r, c0, kb);
-    tcb_child_kb(uy, yy, a, cy, r, c0, kb);
   };
   // a_y = q_k o U_x: den = a_y . U_y and a tip sibling's numerator; then
   // a_x = q_k o U_y, split into A
@@ -612,7 +618,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_tcb_kernel(LevelArgs<T> a) 
     coop_put(A, q);
     tc::fence_smem_for_async();
   };
-  load(0);
+  load_q(0);
   form(0);
   __syncthreads();  // barriers initialised, TMEM allocated
   tc::fence_after();
@@ -630,7 +636,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_tcb_kernel(LevelArgs<T> a) 
   // rounds W, q (internal x) of K-block 0, then of K-block 1
   if (ok) {
     mma(false, 0);
-    load(1);
+    load_q(1);
+    load_u(1);
     ok = tc_block_wait(&bar_mma, pmma, pend_mma, a.err);
   }
   if (ok && cx.internal) {

@@ -593,13 +593,16 @@ __global__ void __launch_bounds__(kTcdThreads) pre_tcd_kernel(LevelArgs<T> a) {
     }
     if (tid < 64) ecol[tid] = reinterpret_cast<const int*>(a.qt + kTcdB)[tid];
   }
-  pdl_wait_and_release();
-  if (internal && warp == 0) tc::alloc(&bars.tmem, 512);
+  // The matrices and the children's U are read before the wait: the matrix
+  // build and the post-order pass, which ended with its root level, are at
+  // least one launch back; only q_k comes from the launch before.
   if (internal && tid < 64)
     ecol_p[tid] = reinterpret_cast<const int*>(tcd_unit(a, bx, r) + 2 * kTcdB)[tid];
   double av[2][8], u[2][8];
   int y[2], ey[2], ex[2], eq[2];
   tcd_child(a, by, cy, r, c0, false, u, y, ey);
+  pdl_wait_and_release();
+  if (internal && warp == 0) tc::alloc(&bars.tmem, 512);
 #pragma unroll
   for (int it = 0; it < 2; ++it) {  // a_x = q_k o U_y
     const int c = c0 + tcd_row(it);
