@@ -116,27 +116,6 @@ __device__ __forceinline__ void matvec_t(const T* __restrict__ M,
 template <typename T, int SP>
 constexpr bool kTrSmall = std::is_same<T, float>::value && SP == 20;
 
-// Where the register kernels keep the partial vector of (slot, pattern c,
-// category r).  FP32 with 20 padded states: tile-blocked by the kernels'
-// block, [slot][tile][chunk][kSmallThreads][4] with tile = c / (threads /
-// RP) and lane (c % (threads / RP)) RP + r, so a warp's access to one
-// 16-byte chunk is 512 contiguous bytes (uses_p20_tiles); chunk stride
-// kSmallThreads float4.  Otherwise pattern-major [slot][c][r][SP].
-template <typename T, int SP, int RP>
-struct SmallVec {
-  static constexpr bool tiled = kTrSmall<T, SP>;
-  static constexpr int cs = tiled ? kSmallThreads : 1;  // chunk stride (vectors)
-  __device__ static size_t offset(size_t slot, int c, int r, int R, int C, int n_tiles) {
-    if constexpr (tiled) {
-      constexpr int CT = kSmallThreads / RP;
-      const size_t tile = slot * n_tiles + c / CT;
-      return tile * (size_t)(kSmallThreads * SP) + (size_t)((c % CT) * RP + r) * 4;
-    } else {
-      return ((slot * C + c) * R + r) * SP;
-    }
-  }
-};
-
 // out[j] = sum_i y[i] X[i][j], two outputs per packed FMA, i in order (the
 // same operations as matvec / matvec_t): X = M' gives M v, X = M gives M' a.
 template <int SP>
@@ -387,9 +366,7 @@ __device__ __forceinline__ void load_child(const LevelArgs<T>& a, int b,
     load_vec<T, SP>(a.tip_partials + ((size_t)b * C + c) * SP, in.v, active);
   } else {
     const size_t slot = (size_t)(b - a.n_tips);
-    using SV = SmallVec<T, SP, RP>;
-    load_vec<T, SP>(a.post + SV::offset(slot, c, r, a.n_cat, C, a.n_tiles), in.v, active,
-                    SV::cs);
+    load_vec<T, SP>(a.post + ((slot * C + c) * a.n_cat + r) * SP, in.v, active);
     if (want_e && active) in.e = a.escale[slot * a.escale_stride + c];
   }
 }
@@ -507,8 +484,7 @@ post_small_kernel(LevelArgs<T> a) {
     if (k != a.root) {
       const size_t slot = (size_t)(k - a.n_tips);
       if (active) {
-        using SV = SmallVec<T, SP, RP>;
-        store_vec<T, SP>(a.post + SV::offset(slot, c, r, R, C, a.n_tiles), ui, SV::cs);
+        store_vec<T, SP>(a.post + ((slot * C + c) * R + r) * SP, ui);
         if (r == 0) a.escale[slot * a.escale_stride + c] = e;
       }
       continue;
@@ -583,9 +559,7 @@ pre_small_kernel(LevelArgs<T> a) {
         for (int s = 0; s < SP; ++s)
           q[u][s] = (active && s < a.n_states) ? (T)a.root_pi[s] : T(0);
       } else {
-        using SV = SmallVec<T, SP, RP>;
-        load_vec<T, SP>(a.pre + SV::offset(k - a.n_tips, c, r, R, C, a.n_tiles), q[u], active,
-                        SV::cs);
+        load_vec<T, SP>(a.pre + (((size_t)(k - a.n_tips) * C + c) * R + r) * SP, q[u], active);
       }
       load_child<T, SP, RP>(a, d[u].y, d[u].w & kDescCompactX, c, r, active, false, in[u][0]);
       load_child<T, SP, RP>(a, d[u].z, d[u].w & kDescCompactY, c, r, active, false, in[u][1]);
@@ -641,8 +615,7 @@ pre_small_kernel(LevelArgs<T> a) {
       const T m = pattern_max<T, SP, RP>(out, active);
       rescale<T, SP>(out, m, valid_c, a.err);
       if (active) {
-        using SV = SmallVec<T, SP, RP>;
-        store_vec<T, SP>(a.pre + SV::offset(bi - a.n_tips, c, r, R, C, a.n_tiles), out, SV::cs);
+        store_vec<T, SP>(a.pre + (((size_t)(bi - a.n_tips) * C + c) * R + r) * SP, out);
       }
     }
     if (bj >= a.n_tips) {
@@ -653,8 +626,7 @@ pre_small_kernel(LevelArgs<T> a) {
       const T m = pattern_max<T, SP, RP>(out, active);
       rescale<T, SP>(out, m, valid_c, a.err);
       if (active) {
-        using SV = SmallVec<T, SP, RP>;
-        store_vec<T, SP>(a.pre + SV::offset(bj - a.n_tips, c, r, R, C, a.n_tiles), out, SV::cs);
+        store_vec<T, SP>(a.pre + (((size_t)(bj - a.n_tips) * C + c) * R + r) * SP, out);
       }
     }
     block_sum_acc<T, NT>(gi, gj, red, RP);
@@ -694,6 +666,38 @@ pre_small_kernel(LevelArgs<T> a) {
 // ---------------------------------------------------------------------------
 constexpr int kU20 = 20;
 
+// Vectors of 20 padded states, in tiles of 128 / RP patterns of 128 lanes.
+// QL = false: [slot][tile][chunk of 4 states][lane = (pattern, r)][4], so a
+// warp's 16-byte accesses are 512 contiguous bytes.  QL = true, on problems
+// whose wide levels run four patterns per thread (kernels_q20.cuh):
+// [slot][tile][state][lane = (pattern / 4, r)][pattern % 4]: 512 contiguous
+// bytes a state there, 128 here.
+template <int RP, bool QL>
+__device__ __forceinline__ size_t u20_offset(size_t slot, int c, int r, int n_tiles) {
+  constexpr int CT = kSmallThreads / RP;
+  const int pt = c % CT;
+  return (slot * n_tiles + c / CT) * (size_t)(kSmallThreads * kU20) +
+         (size_t)(QL ? ((pt >> 2) * RP + r) * 4 + (pt & 3) : (pt * RP + r) * 4);
+}
+template <bool QL>
+__device__ __forceinline__ void load20(const float* src, float (&v)[kU20], bool active) {
+  if constexpr (QL) {
+#pragma unroll
+    for (int s = 0; s < kU20; ++s) v[s] = active ? __ldg(src + s * kSmallThreads) : 0.f;
+  } else {
+    load_vec<float, kU20>(src, v, active, kSmallThreads);
+  }
+}
+template <bool QL>
+__device__ __forceinline__ void store20(float* dst, const float (&v)[kU20]) {
+  if constexpr (QL) {
+#pragma unroll
+    for (int s = 0; s < kU20; ++s) dst[s * kSmallThreads] = v[s];
+  } else {
+    store_vec<float, kU20>(dst, v, kSmallThreads);
+  }
+}
+
 // U slot of node x: internal nodes x - N, tips with partials N - 1 + x.
 __device__ __forceinline__ size_t u20_slot(const LevelArgs<float>& a, int x) {
   return x >= a.n_tips ? (size_t)(x - a.n_tips) : (size_t)(a.n_tips - 1 + x);
@@ -702,20 +706,17 @@ __device__ __forceinline__ size_t u20_slot(const LevelArgs<float>& a, int x) {
 // A child's U row for this thread's (pattern, category): stored (internal
 // child or tip with partials, with the child's exponent) or, for a compact
 // tip, its state (resolved by u20_resolve from the staged P').
-template <int RP>
+template <int RP, bool QL>
 __device__ __forceinline__ void load_u20(const LevelArgs<float>& a, int b, bool compact, int c,
                                          int r, bool active, bool want_e,
                                          ChildIn<float, kU20>& in) {
-  using SV = SmallVec<float, kU20, RP>;
   in.e = 0;
   if (compact) {
     in.y = active ? (int)a.tip_states[(size_t)b * a.state_stride + c] : 0;
     return;
   }
   in.y = -1;
-  load_vec<float, kU20>(
-      a.post + SV::offset(u20_slot(a, b), c, r, a.n_cat, a.n_patterns, a.n_tiles), in.v,
-      active, SV::cs);
+  load20<QL>(a.post + u20_offset<RP, QL>(u20_slot(a, b), c, r, a.n_tiles), in.v, active);
   if (want_e && active && b >= a.n_tips)
     in.e = a.escale[(size_t)(b - a.n_tips) * a.escale_stride + c];
 }
@@ -771,12 +772,11 @@ __device__ __forceinline__ void post_u20_stage(const LevelArgs<float>& a, const 
 
 // Post-order level: per node of the block, slots [P'_child0 | P'_child1 |
 // P'_node] (every category); on the tip level, P'_tip alone.
-template <int RP, int NPT>
+template <int RP, int NPT, bool QL>
 __global__ void __launch_bounds__(kSmallThreads, PHYLO_U20_POST_BLOCKS)
 post_u20_kernel(LevelArgs<float> a) {
   constexpr int SP = kU20, NT = kSmallThreads, CT = NT / RP;
   constexpr int MS = MatStride<float, SP>::v;
-  using SV = SmallVec<float, SP, RP>;
   extern __shared__ __align__(16) unsigned char smraw[];
   float* mats = reinterpret_cast<float*>(smraw);  // [NPT][3][RP][MS]
   __shared__ uint64_t bar;
@@ -808,8 +808,8 @@ post_u20_kernel(LevelArgs<float> a) {
       in[u][0].e = 0;
       load_vec<float, SP>(a.tip_partials + ((size_t)d[u].x * C + c) * SP, in[u][0].v, active);
     } else {
-      load_u20<RP>(a, d[u].y, d[u].w & kDescCompactX, c, r, active, true, in[u][0]);
-      load_u20<RP>(a, d[u].z, d[u].w & kDescCompactY, c, r, active, true, in[u][1]);
+      load_u20<RP, QL>(a, d[u].y, d[u].w & kDescCompactX, c, r, active, true, in[u][0]);
+      load_u20<RP, QL>(a, d[u].z, d[u].w & kDescCompactY, c, r, active, true, in[u][1]);
     }
   }
   if (!__syncthreads_and(mbar_wait(&bar, 0))) {
@@ -838,8 +838,7 @@ post_u20_kernel(LevelArgs<float> a) {
     if (k != a.root) {
       rowcomb2<SP>(Ptk, p, uk);  // U_k = P_k p_k
       if (active) {
-        store_vec<float, SP>(a.post + SV::offset(u20_slot(a, k), c, r, R, C, a.n_tiles), uk,
-                             SV::cs);
+        store20<QL>(a.post + u20_offset<RP, QL>(u20_slot(a, k), c, r, a.n_tiles), uk);
         if (!tip && r == 0) a.escale[(size_t)(k - a.n_tips) * a.escale_stride + c] = e;
       }
       continue;
@@ -894,13 +893,12 @@ __device__ __forceinline__ void pre_u20_stage(const LevelArgs<float>& a, const i
 
 // Pre-order level with the fused gradient: slots per node [P'_i | P'_j |
 // dP'_i | dP'_j | P_i | P_j] (every category), then Q (one matrix).
-template <int RP, int NPT>
+template <int RP, int NPT, bool QL>
 __global__ void __launch_bounds__(kSmallThreads, PHYLO_U20_PRE_BLOCKS)
 pre_u20_kernel(LevelArgs<float> a) {
   constexpr int SP = kU20, NT = kSmallThreads, CT = NT / RP;
   constexpr int MS = MatStride<float, SP>::v;
   constexpr int NS = 6;
-  using SV = SmallVec<float, SP, RP>;
   extern __shared__ __align__(16) unsigned char smraw[];
   float* mats = reinterpret_cast<float*>(smraw);  // [NPT][NS][RP][MS]
   float* Qm = mats + (size_t)NPT * NS * RP * MS;  // Q, row-major SP x SP
@@ -921,10 +919,18 @@ pre_u20_kernel(LevelArgs<float> a) {
   for (int u = 0; u < NPT; ++u)
     d[u] = u < nn ? a.level_desc[g0 + u] : make_int4(0, 0, 0, 0);
   if (a.mats_ready) pre_u20_stage<RP, NPT>(a, d, nn, mats, Qm, &bar);
+  // The children's U: the post-order pass that wrote them ended with its root
+  // level, at least one launch back; only q_k comes from the launch before.
+  ChildIn<float, SP> in[NPT][2];
+#pragma unroll
+  for (int u = 0; u < NPT; ++u) {
+    if (u >= nn) continue;
+    load_u20<RP, QL>(a, d[u].y, d[u].w & kDescCompactX, c, r, active, false, in[u][0]);
+    load_u20<RP, QL>(a, d[u].z, d[u].w & kDescCompactY, c, r, active, false, in[u][1]);
+  }
   pdl_wait_and_release();
   if (!a.mats_ready) pre_u20_stage<RP, NPT>(a, d, nn, mats, Qm, &bar);
   float q[NPT][SP];
-  ChildIn<float, SP> in[NPT][2];
 #pragma unroll
   for (int u = 0; u < NPT; ++u) {
     if (u >= nn) continue;
@@ -933,11 +939,8 @@ pre_u20_kernel(LevelArgs<float> a) {
 #pragma unroll
       for (int s = 0; s < SP; ++s) q[u][s] = (active && s < S) ? a.root_pit[s] : 0.f;
     } else {
-      load_vec<float, SP>(a.pre + SV::offset(k - a.n_tips, c, r, R, C, a.n_tiles), q[u], active,
-                          SV::cs);
+      load20<QL>(a.pre + u20_offset<RP, QL>(k - a.n_tips, c, r, a.n_tiles), q[u], active);
     }
-    load_u20<RP>(a, d[u].y, d[u].w & kDescCompactX, c, r, active, false, in[u][0]);
-    load_u20<RP>(a, d[u].z, d[u].w & kDescCompactY, c, r, active, false, in[u][1]);
   }
   const float w = active ? a.cat_wt[r] : 0.f;
   const float gam = active ? (float)a.rates[r] : 0.f;
@@ -1017,8 +1020,7 @@ pre_u20_kernel(LevelArgs<float> a) {
         const float m = pattern_max<float, SP, RP>(out, active);
         rescale<float, SP>(out, m, valid_c, a.err);
         if (active)
-          store_vec<float, SP>(a.pre + SV::offset(b[x] - a.n_tips, c, r, R, C, a.n_tiles), out,
-                               SV::cs);
+          store20<QL>(a.pre + u20_offset<RP, QL>(b[x] - a.n_tips, c, r, a.n_tiles), out);
       }
     }
     // sum over categories (Eq. 8) in FP32, then the ratio
@@ -1056,6 +1058,7 @@ constexpr size_t u20_smem(bool post) {
 
 #include "kernels_p4.cuh"
 #include "kernels_tree.cuh"
+#include "kernels_q20.cuh"
 #include "kernels_tc64.cuh"
 #include "kernels_tcd.cuh"
 #include "kernels_big.cuh"
@@ -1082,14 +1085,18 @@ template <typename T, int SP, int RP>
 cudaError_t launch_small(const LevelArgs<T>& a, bool post, cudaStream_t st) {
   constexpr int NPo = SmallNpt<T, SP>::post, NPr = SmallNpt<T, SP>::pre;
   if constexpr (kTrSmall<T, SP>) {  // FP32, 20 padded states: the U form
+    // four patterns per thread on the levels that fill the GPU that way (two
+    // blocks per SM), one elsewhere
+    if (a.quad && (long long)((a.n_tiles + 3) / 4) * a.n_level >= 2 * kSms)
+      return launch_q20<RP>(a, post, st);
     if (post) {
       dim3 grid(a.n_tiles, (a.n_level + NPo - 1) / NPo);
-      return launch_pdl(post_u20_kernel<RP, NPo>, grid, kSmallThreads, u20_smem<RP, NPo>(true),
-                        st, a);
+      return launch_pdl(a.quad ? post_u20_kernel<RP, NPo, true> : post_u20_kernel<RP, NPo, false>,
+                        grid, kSmallThreads, u20_smem<RP, NPo>(true), st, a);
     }
     dim3 grid(a.n_tiles, (a.n_level + NPr - 1) / NPr);
-    return launch_pdl(pre_u20_kernel<RP, NPr>, grid, kSmallThreads, u20_smem<RP, NPr>(false), st,
-                      a);
+    return launch_pdl(a.quad ? pre_u20_kernel<RP, NPr, true> : pre_u20_kernel<RP, NPr, false>,
+                      grid, kSmallThreads, u20_smem<RP, NPr>(false), st, a);
   }
   if (post) {
     dim3 grid(a.n_tiles, (a.n_level + NPo - 1) / NPo);
@@ -1105,13 +1112,16 @@ template <typename T, int SP, int RP>
 cudaError_t prepare_small() {
   constexpr int NPo = SmallNpt<T, SP>::post, NPr = SmallNpt<T, SP>::pre;
   if constexpr (kTrSmall<T, SP>) {
-    cudaError_t e = cudaFuncSetAttribute(post_u20_kernel<RP, NPo>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)u20_smem<RP, NPo>(true));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(pre_u20_kernel<RP, NPr>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)u20_smem<RP, NPr>(false));
+    cudaError_t e = prepare_q20<RP>();
+    for (auto k : {post_u20_kernel<RP, NPo, true>, post_u20_kernel<RP, NPo, false>})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)u20_smem<RP, NPo>(true));
+    for (auto k : {pre_u20_kernel<RP, NPr, true>, pre_u20_kernel<RP, NPr, false>})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)u20_smem<RP, NPr>(false));
+    return e;
   }
   cudaError_t e = cudaFuncSetAttribute(
       post_small_kernel<T, SP, RP, NPo>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -144,6 +144,16 @@ inline int walk_group(bool fp64, int n_tips, int C, int R, int RP) {
   const int resident = !fp64 && 2 * (smem(g) + 2048) <= 228 * 1024 ? 2 : 1;
   return blocks(g) <= kSms * resident ? g : -1;
 }
+// FP32 with 5..20 states: whether enough of a tree's levels fill the GPU with
+// four patterns per thread to lay the partials out for it (about a quarter of
+// the nodes sit in the widest level).  4 categories, before -> after: 256 taxa x
+// 5,000 patterns 0.99 -> 0.84 ms, 500 x 1,000 0.58 -> 0.55, 16 x 10,000 0.182 ->
+// 0.176; below the line it loses (500 x 300: 0.37 -> 0.38, 96 x 1,201 0.25 ->
+// 0.26).
+inline bool uses_quad(int SP, bool fp64, int n_tips, int n_tiles) {
+  return SP == 20 && !fp64 && n_tiles >= 32 &&
+         (long long)((n_tiles + 3) / 4) * n_tips >= 8 * kSms;
+}
 inline PassMode pass_mode(int SP, bool fp64, int n_tips, int C, int R, int RP) {
   if (SP != 4) return kByLevel;
   if (walk_group(fp64, n_tips, C, R, RP) >= 0) return kWalk;
@@ -408,6 +418,8 @@ struct LevelArgs {
   const unsigned char* qt;     // 21..128 states: Q' operand (FP64: kTcdModelBytes)
   const T* qmat;               // 4 and 20 padded states, U form: Q row-major [SP][SP]
   const double* rates;         // [R] category rates gamma_r
+  int quad;                    // FP32, 20 padded states: the partials' layout for four
+                               // patterns per thread (kernels.cuh, uses_quad)
   int tip_level;               // U-form paths: the level's nodes are tips with
                                // partials (their U = P p, before level 1)
   int mats_ready;              // 1 if P was complete before the previous launch
