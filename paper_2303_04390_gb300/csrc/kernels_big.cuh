@@ -519,7 +519,7 @@ cudaError_t prepare_big() {
 namespace phylo {
 
 // ---------------------------------------------------------------------------
-// Transition matrices for S_pad 128 and 256 on the FP32 path (Eq. 1):
+// Transition matrices for S_pad 256 on the FP32 path (Eq. 1):
 // P - I = V diag(e^{lambda gamma t} - 1) Vinv and dP = V diag(gamma lambda
 // e^{lambda gamma t}) Vinv in the double-float arithmetic of the 64-state
 // build (kernels_tc64.cuh: Dekker products, Knuth sums, ~48 bits), so that
@@ -527,9 +527,7 @@ namespace phylo {
 // cancellation in the sum over eigenvalues.  A CTA computes one 64 x 64
 // tile of P and dP of one (branch, category), streaming the double-float
 // eigenvector tables through shared memory kPmatBigChunk eigenvalues at a
-// time; each thread owns a 4 x 4 block.  With S_pad 128 (the tensor-core
-// path, whose pre-order step needs no dP) only P is built, written as the
-// split P and P' operand blocks.  For the symmetric decomposition
+// time; each thread owns a 4 x 4 block.  For the symmetric decomposition
 // of a reversible model (Vinv[m][t] = pi_t V[t][m]) P - I = K diag(pi) with
 // K = V diag(e) V' symmetric: only the tiles on and above the diagonal are
 // contracted, and an off-diagonal tile also writes its mirror.
@@ -539,7 +537,6 @@ constexpr int kPmatBigChunk = 32;
 template <int SP>
 __global__ void __launch_bounds__(256) pmat_big_df_kernel(PmatArgs a) {
   constexpr int T = SP / 64;
-  constexpr bool kD = SP != 128;  // dP wanted (the S_pad 256 CUDA-core path)
   __shared__ __align__(16) float sv_h[kPmatBigChunk][64], sv_l[kPmatBigChunk][64];
   __shared__ __align__(16) float sw_h[kPmatBigChunk][64], sw_l[kPmatBigChunk][64];
   __shared__ DF se[SP], sd[SP];
@@ -614,58 +611,15 @@ __global__ void __launch_bounds__(256) pmat_big_df_kernel(PmatArgs a) {
         const DF ve = df_mul(v[i], em);
 #pragma unroll
         for (int j = 0; j < 4; ++j) df_fma(accP[i][j], ve, w[j]);
-        if constexpr (kD) {
-          const DF vd = df_mul(v[i], dm);
+        const DF vd = df_mul(v[i], dm);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) df_fma(accD[i][j], vd, w[j]);
-        }
+        for (int j = 0; j < 4; ++j) df_fma(accD[i][j], vd, w[j]);
       }
     }
   }
   const int s0 = 64 * sb + ls, t0 = 64 * tb + lt;
   const float* pi_h = a.vsplit + 4 * sq;
   const float* pi_l = pi_h + SP;
-  if constexpr (SP == 128) {
-    // the tensor-core path's operand blocks instead of P: entry (s, t) goes
-    // to row s % 64, column t % 64 of block P (sb, tb), and to row t % 64,
-    // column s % 64 of block P' (tb, sb); the mirror entries (t, s) of a
-    // reversible model to the transposed places
-    unsigned char* U = static_cast<unsigned char*>(a.tiles) + (size_t)unit * kTcbUnitBytes;
-    float p[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int s = s0 + i, t = t0 + j;
-        DF kp = accP[i][j];
-        if (rev) kp = df_mul(kp, DF{pi_h[t], pi_l[t]});
-        p[i][j] = df_round(kp, s == t && s < S);
-      }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      put_split3_4(U + tcb_block(0, sb, tb), kTerm128, ls + i, lt,
-                   make_float4(p[i][0], p[i][1], p[i][2], p[i][3]));
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      put_split3_4(U + tcb_block(1, tb, sb), kTerm128, lt + j, ls,
-                   make_float4(p[0][j], p[1][j], p[2][j], p[3][j]));
-    if (rev && sb != tb) {  // mirror: P[t][s] = delta + K_st pi_s
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          p[i][j] = df_round(df_mul(accP[i][j], DF{pi_h[s0 + i], pi_l[s0 + i]}), false);
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        put_split3_4(U + tcb_block(0, tb, sb), kTerm128, lt + j, ls,
-                     make_float4(p[0][j], p[1][j], p[2][j], p[3][j]));
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        put_split3_4(U + tcb_block(1, sb, tb), kTerm128, ls + i, lt,
-                     make_float4(p[i][0], p[i][1], p[i][2], p[i][3]));
-    }
-    return;
-  }
   float* P = static_cast<float*>(a.P) + (size_t)unit * sq;
   float* D = static_cast<float*>(a.dP) + (size_t)unit * sq;
 #pragma unroll

@@ -774,9 +774,173 @@ inline cudaError_t launch_tcb(const LevelArgs<float>& a, bool post, cudaStream_t
   return launch_pdl(pre_tcb_kernel<float>, grid, kTcThreads, kTcbSmem, st, a);
 }
 
+// ---------------------------------------------------------------------------
+// Matrices (Eq. 1): P = I + V diag(expm1) Vinv by the exact digit contractions
+// of kernels_tcd.cuh (eight base-256 digits: the sum over eigenvalues, which
+// cancels in the small entries of short branches, carries no rounding), each
+// entry rounded to FP32 and written as the split operands.  One CTA per
+// (branch, category) and half of the columns (64 nh ..), K in two blocks of
+// 64 eigenvalues: the rows V diag(e) sliced here, Vinv's digits from the host.
+// It replaces the double-float contraction on the CUDA cores (12 FP32
+// operations a term; the step includes the tip tables): 254 branches x 4
+// categories, 122 states, 0.76 -> 0.40 ms.  A CTA is a serial chain (slice,
+// contract, slice, contract, split) that one CTA per SM (512 TMEM columns)
+// does not hide.
+// ---------------------------------------------------------------------------
+// Sum of the accumulators of one element in FP32 (K = 128: |D_d| <= 2^22 only
+// for d <= 2, < 2^24 after; the sum's magnitude below 2^8).
+__device__ __forceinline__ float tcb_digit_value(const float (&f)[8], int scale, bool one) {
+  constexpr unsigned K = 0x4b400000u;
+  unsigned n[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) n[d] = (unsigned)__float_as_int(f[d] + 12582912.f);
+  const int t01 = (int)(n[0] * 256u + n[1] - K * 257u);
+  const int t23 = (int)(n[2] * 256u + (unsigned)__float2int_rn(f[3]) - K * 256u);
+  const long long top = (long long)t01 * 65536 + t23;
+  long long low = (long long)__float2int_rn(f[4]) * 256 + __float2int_rn(f[5]);
+  low = low * 256 + __float2int_rn(f[6]);
+  low = low * 256 + __float2int_rn(f[7]);
+  long long V = (top << 19) + (low >> 13);  // in units of 2^(scale - 55)
+  if (one) {  // 1 + the sum (a small one shifted to units of 2^-61)
+    V >>= min(max(-6 - scale, 0), 63);
+    scale = max(scale, -6);
+    V += scale <= 55 ? 1ll << (55 - scale) : 0;
+  }
+  const unsigned long long m = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
+  const int lz = __clzll((long long)m);
+  const unsigned long long X = m << lz;
+  const int E = 127 + 63 + 7 - 62 - lz + scale;
+  if (m == 0 || E <= 0) return 0.f;
+  const unsigned bits = ((unsigned)(E - 1) << 23) + (unsigned)(X >> 40) +
+                        ((unsigned)(X >> 39) & 1u);
+  return __uint_as_float(bits | (V < 0 ? 0x80000000u : 0u));
+}
+
+template <typename T>  // float only
+__global__ void __launch_bounds__(kTcdThreads) pmat_tcb_kernel(PmatArgs a) {
+  static_assert(std::is_same<T, float>::value, "tensor-core path is FP32");
+  extern __shared__ unsigned char smraw[];
+  unsigned char* A = align1024(smraw);
+  unsigned char* B = A + kTcdA;
+  float* stage = reinterpret_cast<float*>(A);  // [128][kStageLd]
+  __shared__ TcdBars bars;
+  __shared__ TcdFactor ex[kTcbSP];
+  __shared__ int erow[kTcRows], ecol[64];
+  const int tid = threadIdx.x, warp = tid >> 5, j = tid & 7;
+  const int S = a.n_states, R = a.n_cat;
+  const int unit = blockIdx.x >> 1, nh = blockIdx.x & 1;
+  const int b = unit / R, r = unit % R;
+  const unsigned char* vd = static_cast<const unsigned char*>(a.vdigits);
+  auto copy_b = [&](int kb) {
+    if (tid == 0) tcd_copy_b(B, vd + (size_t)(2 * nh + kb) * kTcdB, &bars.tma);
+  };
+  if (tid == 0) {
+    mbar_init_fenced(&bars.tma, 1);
+    mbar_init_fenced(&bars.mma, 1);
+  }
+  copy_b(0);
+  if (tid < 64) ecol[tid] = reinterpret_cast<const int*>(vd + 4 * (size_t)kTcdB)[64 * nh + tid];
+  if (tid < kTcbSP) {
+    double e = 0.0;
+    if (tid < S) {
+      double t = a.t[b];
+      if (!(t >= 0.0) || !isfinite(t)) {
+        if (tid == 0 && r == 0 && nh == 0) atomicOr(a.err, ERR_BAD_LENGTH);
+        t = 0.0;
+      }
+      e = expm1(a.lambda[tid] * a.rates[r] * t);
+    }
+    ex[tcd_factor_at(tid)] = tcd_factor(e);
+  }
+  if (warp == 0) tc::alloc(&bars.tmem, 512);
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = bars.tmem;
+  uint32_t ptma = 0, pmma = 0;
+  int pend_tma = -1, pend_mma = -1;
+  // V diag(e) of both K-blocks; a row's digits share one scale
+  TcdFactor x[2][2][8];  // [kb][iteration]
+  int er[2];
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const int s = tcd_row(it);
+    int e[2];
+#pragma unroll
+    for (int kb = 0; kb < 2; ++kb) {
+      double v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int m = 64 * kb + 8 * j + i;
+        v[i] = s < S && m < S ? a.V[s * S + m] : 0.0;
+      }
+      e[kb] = tcd_products(v, ex + 64 * kb, j, x[kb][it]);
+    }
+    er[it] = max(e[0], e[1]);
+    if (j == 0) erow[s] = er[it];
+  }
+  bool ok = true;
+#pragma unroll
+  for (int kb = 0; kb < 2; ++kb) {
+    if (!ok) break;
+    if (kb) copy_b(1);
+#pragma unroll
+    for (int it = 0; it < 2; ++it) tcd_put(A, 128 * 128, tcd_row(it), j, x[kb][it], er[it]);
+    tc::fence_smem_for_async();
+    ok = tc_block_wait(&bars.tma, ptma, pend_tma, a.err);
+    if (!ok) break;
+    if (tid == 0) {
+      tc::fence_after();
+      tcd_mma(tmem, smem_addr(A), smem_addr(B), kb > 0);
+      tc::commit(&bars.mma);
+    }
+    ok = tc_block_wait(&bars.mma, pmma, pend_mma, a.err);
+  }
+  if (ok) {
+    const int s = tcd_acc_row();
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float acc[8][8];
+      const int t0 = tcd_acc_col() + 8 * q;
+      tcd_ld(tcd_acc_addr(tmem) + 8 * q, acc);
+      float v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float f[8] = {acc[0][i], acc[1][i], acc[2][i], acc[3][i],
+                            acc[4][i], acc[5][i], acc[6][i], acc[7][i]};
+        v[i] = tcb_digit_value(f, erow[s] + ecol[t0 + i], s == 64 * nh + t0 + i && s < S);
+      }
+      *reinterpret_cast<float4*>(stage + s * kStageLd + t0) = make_float4(v[0], v[1], v[2], v[3]);
+      *reinterpret_cast<float4*>(stage + s * kStageLd + t0 + 4) =
+          make_float4(v[4], v[5], v[6], v[7]);
+    }
+    __syncthreads();
+    // P: K-block nh of the operand, every row; P': row block nh of both K-blocks
+    unsigned char* U = static_cast<unsigned char*>(a.tiles) + (size_t)unit * kTcbUnitBytes;
+    for (int i = tid; i < 128 * 16; i += kTcdThreads) {
+      const int row = i >> 4, c4 = 4 * (i & 15);
+      put_split3_4(U + tcb_block(0, 0, nh), kTerm128, row, c4,
+                   *reinterpret_cast<const float4*>(stage + row * kStageLd + c4));
+    }
+    for (int i = tid; i < 64 * 32; i += kTcdThreads) {
+      // row t of P', states s4 ..: four lanes fill 32 bytes
+      const int s4 = 4 * (i & 3) + 16 * (i >> 8), t = i >> 2 & 63;
+      put_split3_4(U + tcb_block(1, nh, s4 >> 6), kTerm128, t, s4 & 63,
+                   make_float4(stage[s4 * kStageLd + t], stage[(s4 + 1) * kStageLd + t],
+                               stage[(s4 + 2) * kStageLd + t], stage[(s4 + 3) * kStageLd + t]));
+    }
+  }
+  if (tid == 0) {  // bounded drain of whatever a timeout left in flight
+    if (pend_tma >= 0) (void)mbar_wait(&bars.tma, (uint32_t)pend_tma);
+    if (pend_mma >= 0) (void)mbar_wait(&bars.mma, (uint32_t)pend_mma);
+  }
+  tc::fence_before();
+  __syncthreads();
+  if (warp == 0) tc::dealloc(tmem, 512);
+}
+
 inline cudaError_t launch_pmat_tcb(const PmatArgs& a, cudaStream_t st) {
-  // (writes the operand blocks: a.tiles is set)
-  const cudaError_t e = launch_pmat_big<kTcbSP>(a, st);
+  pmat_tcb_kernel<float><<<2 * a.n_branches * a.n_cat, kTcdThreads, kTcdSmem, st>>>(a);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_pdl(tipq_tcb_kernel<float>, dim3(a.n_tips * a.n_cat), kTcThreads, kTipqBSmem, st, a);
 }
@@ -791,6 +955,9 @@ inline cudaError_t prepare_tcb() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(tipq_tcb_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kTipqBSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(pmat_tcb_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kTcdSmem);
   return e;
 }
 

@@ -65,16 +65,16 @@ __device__ __forceinline__ unsigned long long tcd_fix(double x, int e) {
   return (hi < 0 ? 0ull - v : v) + 0x8080808080808080ull;
 }
 
-// Digit slices of 8 consecutive elements (chunk j of row `row`) of an operand
-// with `rows` rows per slice at `op` (128-byte rows, 128-byte swizzle).
-__device__ __forceinline__ void tcd_put(unsigned char* op, uint32_t slice, int row, int j,
-                                        const double (&x)[8], int e) {
+// Digit slices of 8 consecutive elements (chunk j of row `row`), given in
+// biased fixed point, of an operand at `op` with `slice` bytes per slice
+// (128-byte rows, 128-byte swizzle).
+__device__ __forceinline__ void tcd_put_fix(unsigned char* op, uint32_t slice, int row, int j,
+                                            const unsigned long long (&t)[8]) {
   uint32_t h[8], l[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const unsigned long long t = tcd_fix(x[i], e);
-    h[i] = (uint32_t)(t >> 32);
-    l[i] = (uint32_t)t;
+    h[i] = (uint32_t)(t[i] >> 32);
+    l[i] = (uint32_t)t[i];
   }
   const uint32_t off = tc::b16_chunk(row, j);
   const __half2 bias = __floats2half2_rn(-1152.f, -1152.f);
@@ -93,6 +93,62 @@ __device__ __forceinline__ void tcd_put(unsigned char* op, uint32_t slice, int r
     }
     *reinterpret_cast<uint4*>(op + s * slice + off) = make_uint4(w[0], w[1], w[2], w[3]);
   }
+}
+
+__device__ __forceinline__ void tcd_put(unsigned char* op, uint32_t slice, int row, int j,
+                                        const double (&x)[8], int e) {
+  unsigned long long t[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) t[i] = tcd_fix(x[i], e);
+  tcd_put_fix(op, slice, row, j, t);
+}
+
+// The products V(s, m) e_m in fixed point without the FP64 pipe (a product
+// there takes 64 clocks per warp; the 122-state matrix build 439 -> 406 us):
+// x = m 2^(k - 63) with the sign apart, m in [2^63, 2^64) or zero.
+struct __align__(16) TcdFactor {
+  unsigned long long m;
+  int k, neg;
+};
+constexpr int kTcdZero = -(1 << 20);  // exponent of a zero
+__device__ __forceinline__ TcdFactor tcd_factor(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const int E = (hi >> 20) & 0x7ff;
+  if (E == 0) return TcdFactor{0, kTcdZero, 0};  // (below 2^-1022: as zero)
+  return TcdFactor{(unsigned long long)((hi & 0xfffffu) | 0x100000u) << 43 |
+                       (unsigned long long)lo << 11,
+                   E - 1023, (int)(hi >> 31)};
+}
+// Place of eigenvalue m's factor: the 8 lanes of a row read m = 8 j + i.
+__device__ __forceinline__ int tcd_factor_at(int m) {
+  return (m & ~63) | (m & 7) << 3 | (m >> 3 & 7);
+}
+// Exponent e >= -900 with |v_i f_i| < 2^e over the row's 8 lanes; 0 for zeros.
+__device__ __forceinline__ int tcd_products(const double (&v)[8], const TcdFactor* f, int j,
+                                            TcdFactor (&p)[8]) {
+  int k = kTcdZero;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const TcdFactor a = tcd_factor(v[i]), b = f[8 * i + j];
+    p[i] = TcdFactor{__umul64hi(a.m, b.m), a.k + b.k, a.neg ^ b.neg};
+    k = max(k, p[i].k);
+  }
+  k = max(k, __shfl_xor_sync(kFull, k, 1));
+  k = max(k, __shfl_xor_sync(kFull, k, 2));
+  k = max(k, __shfl_xor_sync(kFull, k, 4));
+  return k < -4096 ? 0 : max(k + 2, -900);
+}
+__device__ __forceinline__ void tcd_put(unsigned char* op, uint32_t slice, int row, int j,
+                                        const TcdFactor (&p)[8], int e) {
+  unsigned long long t[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {  // |x| = m 2^(k - 62), times 2^(62 - e)
+    unsigned long long v;
+    asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(p[i].m), "r"(e - p[i].k));  // >= 2
+    t[i] = (p[i].neg ? 0ull - v : v) + 0x8080808080808080ull;
+  }
+  tcd_put_fix(op, slice, row, j, t);
 }
 
 // D_d accumulators of one element -> sum_d D_d 2^(-12 - 8 d + scale), rounded
@@ -127,9 +183,10 @@ __host__ __device__ constexpr uint32_t tcd_idesc(int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((128u >> 4) << 24);
 }
 
-// Every digit product with i + j <= 7 into the 512 columns at `tmem`.  One
-// thread issues.
-__device__ __forceinline__ void tcd_mma(uint32_t tmem, uint32_t A, uint32_t B) {
+// Every digit product with i + j <= 7 into (or added to) the 512 columns at
+// `tmem`.  One thread issues.
+__device__ __forceinline__ void tcd_mma(uint32_t tmem, uint32_t A, uint32_t B,
+                                        bool accumulate = false) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
 #pragma unroll
@@ -138,7 +195,8 @@ __device__ __forceinline__ void tcd_mma(uint32_t tmem, uint32_t A, uint32_t B) {
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
         tc::mma_bf16(tmem + 64 * i + n0, tc::desc(A + i * 128 * 128 + kk * 32),
-                     tc::desc(B + n0 * 128 + kk * 32), tcd_idesc(N), (i | kk) ? 1 : 0);
+                     tc::desc(B + n0 * 128 + kk * 32), tcd_idesc(N),
+                     (accumulate || (i | kk)) ? 1 : 0);
     }
   }
 }
@@ -297,7 +355,7 @@ __global__ void __launch_bounds__(kTcdThreads) pmat_tcd_kernel(PmatArgs a) {
   unsigned char* B = A + kTcdA;
   double* stage = reinterpret_cast<double*>(A);
   __shared__ TcdBars bars;
-  __shared__ double ex[2][64], dx[2][64];
+  __shared__ TcdFactor ex[2][64], dx[2][64];
   __shared__ int erow[128], ecol[64];
   const int tid = threadIdx.x, warp = tid >> 5, j = tid & 7;
   const int S = a.n_states, R = a.n_cat, units = a.n_branches * R;
@@ -323,8 +381,8 @@ __global__ void __launch_bounds__(kTcdThreads) pmat_tcd_kernel(PmatArgs a) {
       e = expm1(x);
       if (unit / R < a.n_tips) de = g * a.lambda[m] * exp(x);
     }
-    ex[h][m] = e;
-    dx[h][m] = de;
+    ex[h][tcd_factor_at(m)] = tcd_factor(e);
+    dx[h][tcd_factor_at(m)] = tcd_factor(de);
   }
   if (warp == 0) tc::alloc(&bars.tmem, 512);
   __syncthreads();
@@ -338,13 +396,14 @@ __global__ void __launch_bounds__(kTcdThreads) pmat_tcd_kernel(PmatArgs a) {
 #pragma unroll
     for (int it = 0; it < 2; ++it) {
       const int row = tcd_row(it), h = row >> 6, s = row & 63;
-      double x[8];
+      double v[8];
+      TcdFactor x[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int m = 8 * j + i;
-        x[i] = s < S && m < S ? a.V[s * S + m] * (d ? dx : ex)[h][m] : 0.0;
+        v[i] = s < S && m < S ? a.V[s * S + m] : 0.0;
       }
-      const int e = tcd_row_exp(x, false, a.err);
+      const int e = tcd_products(v, (d ? dx : ex)[h], j, x);
       if (j == 0) erow[row] = e;
       tcd_put(A, 128 * 128, row, j, x, e);
     }

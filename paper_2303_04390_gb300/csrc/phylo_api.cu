@@ -49,7 +49,7 @@ struct Layout {
   Region tc_tiles;  // 65..128 states, FP32: pre-split matrix blocks
   Region qt;        // 21..128 states, FP32, and 21..64, FP64: Q' as a tensor-core operand
   Region qn;        // 21..128 states, FP32: Q as a tensor-core operand
-  Region vdigits;   // 21..64 states, FP64: the digits of Vinv'
+  Region vdigits;   // 21..64 states, FP64, and 65..128, FP32: the digits of Vinv'
   Region qmat;      // 4 and 20 padded states, FP32: Q row-major
   Region tip_desc;  // U-form paths with tip partials: descriptors of the tips
                     // whose U = P p the first post-order launch forms
@@ -139,9 +139,10 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
     ok &= add_region(L, L.qn, qt_bytes(L.SP));
   }
   if (tcd) {
-    ok &= add_region(L, L.qt, kTcdModelBytes);
-    ok &= add_region(L, L.vdigits, kTcdModelBytes);
+    ok &= add_region(L, L.qt, digit_bytes(L.SP));
   }
+  if (tcd || uses_tc_big(L.SP, prec == PHYLO_FP64))
+    ok &= add_region(L, L.vdigits, digit_bytes(L.SP));
   if (uses_tr_layout(L.SP, prec == PHYLO_FP64))  // the U form's Q (row-major)
     ok &= add_region(L, L.qmat, (size_t)L.SP * L.SP * L.elem);
   if (C > (1 << 30)) return "n_patterns too large";
@@ -1091,6 +1092,14 @@ int phylo_set_eigen(phylo_ctx* ctx, const double* V, const double* Vinv,
       if (!std::isfinite(acc) || std::fabs(acc - want) > 1e-8)
         return fail(ctx, PHYLO_EINVAL, "V * Vinv differs from I at (%d,%d)", i, j);
     }
+  std::vector<double> bV, bW;
+  if (ctx->L.vdigits.bytes) {  // the same decomposition, scaled for fixed point
+    bV.assign(V, V + (size_t)S * S);
+    bW.assign(Vinv, Vinv + (size_t)S * S);
+    balance_eigen(S, bV.data(), bW.data());
+    V = bV.data();
+    Vinv = bW.data();
+  }
   int rc;
   if ((rc = upload(ctx, ctx->L.V, V, (size_t)S * S, "upload V"))) return rc;
   if ((rc = upload(ctx, ctx->L.Vinv, Vinv, (size_t)S * S, "upload Vinv"))) return rc;
@@ -1107,14 +1116,17 @@ int phylo_set_eigen(phylo_ctx* ctx, const double* V, const double* Vinv,
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
   }
   if (ctx->L.vdigits.bytes) {
+    std::vector<unsigned char> tile(digit_bytes(ctx->L.SP));
+    build_digits(S, ctx->L.SP, [&](int n, int k) { return Vinv[(size_t)k * S + n]; }, tile.data());
+    if ((rc = upload(ctx, ctx->L.vdigits, tile.data(), tile.size(), "upload V operand"))) return rc;
+    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+  }
+  if (uses_tcd(ctx->L.SP, ctx->precision == PHYLO_FP64)) {
     std::vector<double> q((size_t)S * S);  // Q, row-major
     build_q_matrix(S, S, V, Vinv, lambda, q.data());
-    std::vector<unsigned char> tile(kTcdModelBytes);
-    build_digits(S, [&](int n, int k) { return q[(size_t)k * S + n]; }, tile.data());
+    std::vector<unsigned char> tile(digit_bytes(ctx->L.SP));
+    build_digits(S, ctx->L.SP, [&](int n, int k) { return q[(size_t)k * S + n]; }, tile.data());
     if ((rc = upload(ctx, ctx->L.qt, tile.data(), tile.size(), "upload Q operand"))) return rc;
-    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
-    build_digits(S, [&](int n, int k) { return Vinv[(size_t)k * S + n]; }, tile.data());
-    if ((rc = upload(ctx, ctx->L.vdigits, tile.data(), tile.size(), "upload V operand"))) return rc;
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
   } else if (ctx->L.qt.bytes) {
     std::vector<unsigned char> qt(qt_bytes(ctx->L.SP));

@@ -6,6 +6,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <cstring>
+#include <vector>
 
 #include <cuda_runtime.h>
 
@@ -177,22 +178,28 @@ constexpr size_t kTcQtBytes = 3 * 64 * 128;
 inline bool uses_tcd(int SP, bool fp64) { return SP == 64 && fp64; }
 constexpr uint32_t kTcdDigits = 8 * 64 * 128;           // one 64 x 64 operand
 constexpr size_t kTcdUnitBytes = 2 * (size_t)kTcdDigits + 64 * sizeof(int);
-constexpr size_t kTcdModelBytes = kTcdDigits + 64 * sizeof(int);
 
-// The digits of a 64 x 64 operand with rows M(n, k), n, k < S (zero beyond),
-// row n scaled by 2^-e_n to magnitudes below 1: digit i of element (n, k) of
+// The digits of an operand with rows M(n, k), n, k < S (zero beyond) in blocks
+// of 64 x 64 (block of rows n >> 6, columns k >> 6; columns fastest), row n
+// scaled by 2^-e_n to magnitudes below 1: digit i of element (n, k) of
 // round(M 2^(62 - e_n)) = sum_i a_i 256^(7 - i) as an FP16 integer in slice i
-// (8 KB), K-major 128-byte swizzle; then e_n as 64 ints.  out: kTcdModelBytes.
+// (8 KB) of its block, K-major 128-byte swizzle; then e_n as ints.  SP: 64 or
+// 128 padded states.  out: digit_bytes(SP).
+inline size_t digit_bytes(int SP) {
+  return (size_t)(SP / 64) * (SP / 64) * kTcdDigits + SP * sizeof(int);
+}
 template <typename F>
-inline void build_digits(int S, F M, unsigned char* out) {
-  std::memset(out, 0, kTcdModelBytes);
+inline void build_digits(int S, int SP, F M, unsigned char* out) {
+  const int NB = SP / 64;
+  std::memset(out, 0, digit_bytes(SP));
   for (int n = 0; n < S; ++n) {
     double mx = 0.0;
     for (int k = 0; k < S; ++k) mx = std::fmax(mx, std::fabs(M(n, k)));
     int e = 0;
     (void)std::frexp(mx, &e);
-    std::memcpy(out + kTcdDigits + n * sizeof(int), &e, sizeof(int));
+    std::memcpy(out + (size_t)NB * NB * kTcdDigits + n * sizeof(int), &e, sizeof(int));
     for (int k = 0; k < S; ++k) {
+      unsigned char* blk = out + (size_t)((n >> 6) * NB + (k >> 6)) * kTcdDigits;
       const long long v = std::llrint(std::ldexp(M(n, k), 62 - e));
       const uint64_t t = (uint64_t)v + 0x8080808080808080ull;
       for (int i = 0; i < 8; ++i) {
@@ -203,10 +210,47 @@ inline void build_digits(int S, F M, unsigned char* out) {
           const double f = std::frexp(std::fabs((double)digit), &ex);
           h = (uint16_t)((digit < 0 ? 0x8000 : 0) + ((ex + 13) << 10) + (int)(f * 2048.0));
         }
-        const size_t off = (size_t)n * 128 + ((size_t)((k >> 3) ^ (n & 7)) << 4) + (k & 7) * 2;
-        std::memcpy(out + (size_t)i * 64 * 128 + off, &h, 2);
+        const size_t off = (size_t)(n & 63) * 128 +
+                           ((size_t)(((k & 63) >> 3) ^ (n & 7)) << 4) + (k & 7) * 2;
+        std::memcpy(blk + (size_t)i * 64 * 128 + off, &h, 2);
       }
     }
+  }
+}
+
+// Eigenvectors for the digit contractions: fixed point keeps what each term
+// V(s, m) Vinv(m, t) adds to an entry only while no term needs a row's or a
+// column's scale to itself, so the free factor of every eigenvector pair is
+// chosen to give column m of V and row m of Vinv the same size relative to
+// the rows of V and the columns of Vinv.  Powers of two (exact); pairs within
+// a factor of 16, as an orthonormal or a symmetrised basis has, stay as given.
+inline void balance_eigen(int S, double* V, double* W) {
+  std::vector<double> r(S), c(S);
+  for (int pass = 0; pass < 32; ++pass) {
+    bool changed = false;
+    for (int s = 0; s < S; ++s) {
+      r[s] = c[s] = 0.0;
+      for (int m = 0; m < S; ++m) {
+        r[s] = std::fmax(r[s], std::fabs(V[(size_t)s * S + m]));
+        c[s] = std::fmax(c[s], std::fabs(W[(size_t)m * S + s]));
+      }
+    }
+    for (int m = 0; m < S; ++m) {
+      double a = 0.0, b = 0.0;
+      for (int s = 0; s < S; ++s) {
+        if (r[s] > 0.0) a = std::fmax(a, std::fabs(V[(size_t)s * S + m]) / r[s]);
+        if (c[s] > 0.0) b = std::fmax(b, std::fabs(W[(size_t)m * S + s]) / c[s]);
+      }
+      if (!(a > 0.0 && b > 0.0)) continue;
+      const int k = (std::ilogb(b) - std::ilogb(a)) / 2;
+      if (k >= -2 && k <= 2) continue;
+      changed = true;
+      for (int s = 0; s < S; ++s) {
+        V[(size_t)s * S + m] = std::ldexp(V[(size_t)s * S + m], k);
+        W[(size_t)m * S + s] = std::ldexp(W[(size_t)m * S + s], -k);
+      }
+    }
+    if (!changed) break;
   }
 }
 
@@ -310,8 +354,8 @@ inline bool uses_tc_terms(int SP, bool fp64) {
 // Returns whether the decomposition is the symmetric one of a reversible
 // model, Vinv[m][t] = pi_t V[t][m] (then P(t) = I + V diag(e) V' diag(pi)
 // and P_st pi_s = P_ts pi_t, which the kernel exploits).
-// The same tables for S_pad = 128 and 256 (FP32 matrix build of
-// kernels_big.cuh): each SP x SP, then pi, SP each.
+// The same tables for the other padded sizes (S_pad = 256: the FP32 matrix
+// build of kernels_big.cuh): each SP x SP, then pi, SP each.
 inline size_t eigen_split_floats(int SP) { return 4 * (size_t)SP * SP + 2 * (size_t)SP; }
 constexpr size_t kEigenSplitFloats = 4 * 64 * 64 + 2 * 64;
 inline bool build_eigen_split(int S, int SP, const double* V, const double* Vinv,
@@ -339,8 +383,9 @@ inline bool build_eigen_split(int S, int SP, const double* V, const double* Vinv
   }
   return reversible;
 }
-// FP32 paths build their matrices from the double-float tables.
-inline bool uses_eigen_split(int SP, bool fp64) { return !fp64; }
+// FP32 paths build their matrices from the double-float tables, except those
+// of 65..128 states (digits of the eigenvectors).
+inline bool uses_eigen_split(int SP, bool fp64) { return !fp64 && SP != 128; }
 
 // Exponent planes per node: R on the tensor-core path, else 1 (one
 // exponent per (node, pattern) shared by all categories).
@@ -415,7 +460,7 @@ struct LevelArgs {
   int* err;                    // numeric flags
   const unsigned char* tc_tiles;  // 65..128 states, FP32: the pre-split matrix
                                   // blocks [2N-2][R][kTcbUnitBytes] (else null)
-  const unsigned char* qt;     // 21..128 states: Q' operand (FP64: kTcdModelBytes)
+  const unsigned char* qt;     // 21..128 states: Q' operand (FP64: its digits)
   const T* qmat;               // 4 and 20 padded states, U form: Q row-major [SP][SP]
   const double* rates;         // [R] category rates gamma_r
   int quad;                    // FP32, 20 padded states: the partials' layout for four
@@ -457,7 +502,8 @@ struct PmatArgs {
   const unsigned char* qn;  // 21..128 states, FP32: Q as an operand (its rows), for the
                             // tables Q P of compact tips
   const int* tip_has;    // [N] or nullptr: tips with partial vectors (no table)
-  const void* vdigits;   // FP64, 21..64 states: the digits of Vinv' (build_digits)
+  const void* vdigits;   // 21..64 states FP64, 65..128 FP32: the digits of Vinv'
+                         // (build_digits)
   int n_tips;
   int reversible;        // tensor-core path: the table's decomposition is symmetric
   const double* V;       // [S][S]
