@@ -247,6 +247,24 @@ __device__ __forceinline__ int tcd_row_exp(const double (&x)[8], bool valid, int
   return E ? max(E - 1022, -900) : 0;  // (rows below 2^-900 vanish)
 }
 
+// Exponent of a row of P, whose products are read with tcd_value<0>: 0 where
+// the row's absolute sum is at most about 1, as in every stochastic matrix
+// (P sums to one), else enough to bring the sum below 1.
+__device__ __forceinline__ int tcd_sum_exp(const double (&x)[8], int* err) {
+  const int e = tcd_row_exp(x, false, err);
+  unsigned sum = 0;  // in units of 2^-24 (entries above 1 decide by e)
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int hi = __double2hiint(x[i]), k = 1023 - ((hi >> 20) & 0x7ff);
+    const unsigned m = ((unsigned)hi & 0xfffffu) | 0x100000u;  // 2^20 at x = 1
+    sum += k < 0 ? 1u << 25 : k > 20 ? 0u : m << 4 >> k;
+  }
+  sum += __shfl_xor_sync(kFull, sum, 1);
+  sum += __shfl_xor_sync(kFull, sum, 2);
+  sum += __shfl_xor_sync(kFull, sum, 4);
+  return sum <= (1u << 24) + (1u << 8) ? 0 : max(e, 0) + 6;
+}
+
 // Row sums over the 8 lanes of both iterations' rows: 3 additions for two.
 // Lane j even returns iteration 0's sum, odd iteration 1's.
 __device__ __forceinline__ double tcd_row_sums(double s0, double s1) {
@@ -459,10 +477,14 @@ __global__ void __launch_bounds__(kTcdThreads) pmat_tcd_kernel(PmatArgs a) {
           x[i] = st[r8 * kTcdLd + 8 * j + i];
           y[i] = st[(8 * j + i) * kTcdLd + r8];
         }
-        tcd_put(out, 64 * 128, r8, j, x, 0);
+        const int ep = tcd_sum_exp(x, a.err);
+        tcd_put(out, 64 * 128, r8, j, x, ep);
         const int e = tcd_row_exp(y, false, a.err);
         tcd_put(out + kTcdB, 64 * 128, r8, j, y, e);
-        if (j == 0) reinterpret_cast<int*>(out + 2 * kTcdB)[r8] = e;
+        if (j == 0) {
+          reinterpret_cast<int*>(out + 2 * kTcdB)[r8] = e;
+          reinterpret_cast<int*>(out + 2 * kTcdB)[64 + r8] = ep;
+        }
       }
     }
     __syncthreads();  // the staging is the next contraction's operand
@@ -486,6 +508,7 @@ __global__ void __launch_bounds__(kTcdThreads) post_tcd_kernel(LevelArgs<T> a) {
   unsigned char* B = A + kTcdA;
   double* stage = reinterpret_cast<double*>(A);
   __shared__ TcdBars bars;
+  __shared__ int erow[64];  // exponents of P_k's rows
   const int tid = threadIdx.x, warp = tid >> 5, j = tid & 7;
   const int R = a.n_cat, C = a.n_patterns;
   const int4 d = a.level_desc[blockIdx.y];
@@ -500,6 +523,7 @@ __global__ void __launch_bounds__(kTcdThreads) post_tcd_kernel(LevelArgs<T> a) {
   if (a.mats_ready) issue();
   pdl_wait_and_release();
   if (!a.mats_ready) issue();
+  if (tid < 64) erow[tid] = reinterpret_cast<const int*>(tcd_unit(a, k, r) + 2 * kTcdB)[64 + tid];
   if (warp == 0) tc::alloc(&bars.tmem, 512);
   double p[2][8], u[2][8];
   int y[2], e[2], e1[2];
@@ -541,7 +565,9 @@ __global__ void __launch_bounds__(kTcdThreads) post_tcd_kernel(LevelArgs<T> a) {
                             acc[4][i], acc[5][i], acc[6][i], acc[7][i]};
         const float g[8] = {acc[0][i + 1], acc[1][i + 1], acc[2][i + 1], acc[3][i + 1],
                             acc[4][i + 1], acc[5][i + 1], acc[6][i + 1], acc[7][i + 1]};
-        *reinterpret_cast<double2*>(st + i) = make_double2(tcd_value<0>(f, 0), tcd_value<0>(g, 0));
+        *reinterpret_cast<double2*>(st + i) = make_double2(
+            tcd_value<0>(f, erow[tcd_acc_col() + 8 * q + i]),
+            tcd_value<0>(g, erow[tcd_acc_col() + 8 * q + i + 1]));
       }
     }
     __syncthreads();

@@ -54,7 +54,7 @@ def test_free_factors_of_the_eigenvectors(S, precision):
     ctx.close()
 
 
-@pytest.mark.parametrize("S,precision", [(122, "fp32")])
+@pytest.mark.parametrize("S,precision", [(122, "fp32"), (61, "fp64"), (21, "fp64")])
 def test_entries_above_one(S, precision):
     """A decomposition whose exponentials are positive but not stochastic:
     D Q D^-1, with entries and row sums far above 1 off the diagonal."""
