@@ -213,32 +213,21 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
       yb[1] = a.tip_states[(size_t)gj2.y * a.state_stride + c];
     }
   }
-  // The children's vectors.  The pre-order pass reads them before the wait as
-  // well: the post-order pass that wrote them ended with its root level, at
-  // least one launch back, and only q_k comes from the launch before.
-  auto load_children = [&] {
-#pragma unroll
-    for (int r = 0; r < RM; ++r) {
-      const bool on = valid && r < R;
-      vi[r] = zero4; vj[r] = zero4;
-      if (on && !ci && !hi_)
-        vi[r] = bi < a.n_tips ? __ldg(reinterpret_cast<const float4*>(a.tip_partials) + (size_t)bi * C + c)
-                              : __ldg(reinterpret_cast<const float4*>(a.post) +
-                                      p4_index(bi - a.n_tips, c, r, R, a.n_tiles));
-      if (on && !cj && !hj_)
-        vj[r] = bj < a.n_tips ? __ldg(reinterpret_cast<const float4*>(a.tip_partials) + (size_t)bj * C + c)
-                              : __ldg(reinterpret_cast<const float4*>(a.post) +
-                                      p4_index(bj - a.n_tips, c, r, R, a.n_tiles));
-    }
-  };
-  if (PRE) load_children();
   pdl_wait_and_release();
   if (!a.mats_ready) issue_copies();
-  if (!PRE) load_children();
 #pragma unroll
   for (int r = 0; r < RM; ++r) {
-    q[r] = zero4;
-    if (PRE && valid && r < R && k != a.root)
+    const bool on = valid && r < R;
+    vi[r] = zero4; vj[r] = zero4; q[r] = zero4;
+    if (on && !ci && !hi_)
+      vi[r] = bi < a.n_tips ? __ldg(reinterpret_cast<const float4*>(a.tip_partials) + (size_t)bi * C + c)
+                            : __ldg(reinterpret_cast<const float4*>(a.post) +
+                                    p4_index(bi - a.n_tips, c, r, R, a.n_tiles));
+    if (on && !cj && !hj_)
+      vj[r] = bj < a.n_tips ? __ldg(reinterpret_cast<const float4*>(a.tip_partials) + (size_t)bj * C + c)
+                            : __ldg(reinterpret_cast<const float4*>(a.post) +
+                                    p4_index(bj - a.n_tips, c, r, R, a.n_tiles));
+    if (PRE && on && k != a.root)
       q[r] = __ldg(reinterpret_cast<const float4*>(a.pre) +
                    p4_index(k - a.n_tips, c, r, R, a.n_tiles));
   }
