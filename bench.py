@@ -576,11 +576,12 @@ def rooflines(w, precision, phase_ms, level_counts, peaks, n_sm, workload):
                "pre": "pre-order level kernel (fused gradient)",
                "reduce": "reduce_kernel"}
     if precision == "fp32" and 20 < w.n_states <= 64:
-        kernels = {"pmat": "pmat_tc_kernel", "post": "post_u_kernel + root_u_kernel",
+        kernels = {"pmat": "pmat_tc_kernel + tipq_tc_kernel",
+                   "post": "post_u_kernel + root_u_kernel",
                    "pre": "pre_u_kernel + ratio_tc_kernel",
                    "reduce": "reduce_kernel"}
     if precision == "fp32" and 64 < w.n_states <= 128:
-        kernels = {"pmat": "pmat_big_df_kernel (writes the split operand blocks)",
+        kernels = {"pmat": "pmat_tcb_kernel + tipq_tcb_kernel",
                    "post": "post_tcb_kernel + root_tcb_kernel",
                    "pre": "pre_tcb_kernel + ratio_tc_kernel",
                    "reduce": "reduce_kernel"}
