@@ -898,20 +898,15 @@ __global__ void __launch_bounds__(kTcdThreads) pmat_tcb_kernel(PmatArgs a) {
   if (ok) {
     const int s = tcd_acc_row();
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      float acc[8][8];
-      const int t0 = tcd_acc_col() + 8 * q;
-      tcd_ld(tcd_acc_addr(tmem) + 8 * q, acc);
-      float v[8];
+    for (int q = 0; q < 4; ++q) {
+      float f[4][8];
+      const int t0 = tcd_acc_col() + 4 * q;
+      tcd_ld(tcd_acc_addr(tmem) + 4 * q, f);
+      float v[4];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float f[8] = {acc[0][i], acc[1][i], acc[2][i], acc[3][i],
-                            acc[4][i], acc[5][i], acc[6][i], acc[7][i]};
-        v[i] = tcb_digit_value(f, erow[s] + ecol[t0 + i], s == 64 * nh + t0 + i && s < S);
-      }
+      for (int i = 0; i < 4; ++i)
+        v[i] = tcb_digit_value(f[i], erow[s] + ecol[t0 + i], s == 64 * nh + t0 + i && s < S);
       *reinterpret_cast<float4*>(stage + s * kStageLd + t0) = make_float4(v[0], v[1], v[2], v[3]);
-      *reinterpret_cast<float4*>(stage + s * kStageLd + t0 + 4) =
-          make_float4(v[4], v[5], v[6], v[7]);
     }
     __syncthreads();
     // P: K-block nh of the operand, every row; P': row block nh of both K-blocks

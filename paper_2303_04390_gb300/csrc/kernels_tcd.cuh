@@ -16,13 +16,24 @@
 //   without any rounding.  The epilogue adds them in integer arithmetic,
 //   sum_d D_d 256^(7 - d), and rounds once to FP64.
 //
-// What is dropped (digits past the 62nd bit, products with i + j > 7, the last
-// bits of a sum that may reach 64) is below 2^-56 of the product of the row's
-// and the column's largest entries.  The matrices carry a larger absolute
-// error from the eigenvector route (about 2^-53), so the results are as far
-// from exact as with FP64 products: gradient (2-norm) 1.4e-14 to 2.7e-13 over
-// 8 to 64 taxa, mean branch lengths 0.002 to 0.1, 1 and 4 categories, within
-// 3% of what the FP64 products gave on the same inputs.
+// What is dropped (digits past the 62nd bit, products with i + j > 7) is about
+// 2^-59 of the product of the row's and the column's largest entries: an
+// absolute error.  On a short branch P has entries of the order t, t^2 and t^3
+// beside a diagonal near 1, and where the two sides of an internal branch
+// disagree the site likelihood is one of those.  So the contractions take
+// E = P - I = V diag(expm1) Vinv, whose rows and columns have scales of their
+// own (of the order t), and the identity's part stays in FP64:
+//   U = p + E p,   q_x = a_x + E' a_x.
+// The error is then 2^-59 of E's entries times p, while the eigenvector route
+// leaves one of about 2^-56 t in those entries themselves.  The matrix build
+// and a_x Q, whose sums may be far below the largest product, are rounded at
+// the 53rd bit of the sum instead of at a fixed place.  Measured: codons that
+// differ by 1, 2 and 3 nucleotides across internal branches of 1e-8 to 2e-3 are
+// as far from exact as FP64 products on the same eigenvectors are (with P in
+// place of E: up to 1e8 times as far); simulated alignments, 20 to 61 taxa,
+// mean branch lengths 0.002 to 0.1: gradient (2-norm) 1.2e-14 to 1.2e-13, 0.98
+// to 1.01 times what FP64 products leave.  It costs 6% (61 taxa x 601 patterns
+// x 4 categories 0.72 -> 0.76 ms): one FP64 addition per entry.
 //
 // The digits of slice i of the 128-row operand multiply the digits 0..7 - i
 // of the 64-row operand, whose accumulators are adjacent TMEM columns: one
@@ -32,9 +43,9 @@
 // Structure as in kernels_tc64.cuh (U form, per-category exponents, one CTA
 // per 128-pattern tile, node and category), with FP64 vectors: the elementwise
 // products, the dot products of Eq. 8 and the sums stay on the FP64 pipe.
-//   post:  p_k = U_i o U_j, normalised per row,  U_k = p_k P_k'
+//   post:  p_k = U_i o U_j, normalised per row,  U_k = p_k + p_k E_k'
 //   pre:   a_x = q_k o U_y, den = a_x . U_x, num_x = gamma_r (a_x Q) . U_x,
-//          q_x = a_x P_x  (a normalised per row)
+//          q_x = a_x + a_x E_x  (a normalised per row)
 //   a tip: U_x is column y of P_x and num_x = a_x . (column y of dP_x), from
 //          FP64 tables; a tip with a partial vector multiplies them out.
 #pragma once
@@ -51,15 +62,15 @@ static_assert(128 * kTcdLd * 8 <= kTcdA, "staging fits in the operand buffer");
 constexpr size_t kTcdSmem = 1024 + kTcdA + kTcdB;
 constexpr uint32_t kTcdTab = 64 * 64 * 8;  // one FP64 table
 
-// The digits' fixed point of x / 2^e, |x| < 2^e (or x = 2^e), towards zero:
-// x 2^(62 - e), plus the bias that makes every byte a digit + 128.  e >= -900.
-__device__ __forceinline__ unsigned long long tcd_fix(double x, int e) {
+// The digits' fixed point of x, |x| <= 1, towards zero: x 2^62, plus the bias
+// that makes every byte a digit + 128.
+__device__ __forceinline__ unsigned long long tcd_fix(double x, int s) {
   const int hi = __double2hiint(x);
   const unsigned lo = (unsigned)__double2loint(x);
   // 2^62 <= m < 2^63; a zero or subnormal x is shifted out (k > 63)
   const unsigned long long m =
       ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32 | lo) << 10;
-  const int k = 1023 + e - ((hi >> 20) & 0x7ff);
+  const int k = 1023 + s - ((hi >> 20) & 0x7ff);
   unsigned long long v;
   asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(k));  // (shifts past 63 give 0)
   return (hi < 0 ? 0ull - v : v) + 0x8080808080808080ull;
@@ -96,10 +107,10 @@ __device__ __forceinline__ void tcd_put_fix(unsigned char* op, uint32_t slice, i
 }
 
 __device__ __forceinline__ void tcd_put(unsigned char* op, uint32_t slice, int row, int j,
-                                        const double (&x)[8], int e) {
+                                        const double (&x)[8], int s = 0) {
   unsigned long long t[8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) t[i] = tcd_fix(x[i], e);
+  for (int i = 0; i < 8; ++i) t[i] = tcd_fix(x[i], s);
   tcd_put_fix(op, slice, row, j, t);
 }
 
@@ -124,7 +135,7 @@ __device__ __forceinline__ TcdFactor tcd_factor(double x) {
 __device__ __forceinline__ int tcd_factor_at(int m) {
   return (m & ~63) | (m & 7) << 3 | (m >> 3 & 7);
 }
-// Exponent e >= -900 with |v_i f_i| < 2^e over the row's 8 lanes; 0 for zeros.
+// Exponent e with |v_i f_i| < 2^e over the row's 8 lanes; 0 for zeros.
 __device__ __forceinline__ int tcd_products(const double (&v)[8], const TcdFactor* f, int j,
                                             TcdFactor (&p)[8]) {
   int k = kTcdZero;
@@ -137,7 +148,7 @@ __device__ __forceinline__ int tcd_products(const double (&v)[8], const TcdFacto
   k = max(k, __shfl_xor_sync(kFull, k, 1));
   k = max(k, __shfl_xor_sync(kFull, k, 2));
   k = max(k, __shfl_xor_sync(kFull, k, 4));
-  return k < -4096 ? 0 : max(k + 2, -900);
+  return k < -4096 ? 0 : k + 2;
 }
 __device__ __forceinline__ void tcd_put(unsigned char* op, uint32_t slice, int row, int j,
                                         const TcdFactor (&p)[8], int e) {
@@ -151,11 +162,24 @@ __device__ __forceinline__ void tcd_put(unsigned char* op, uint32_t slice, int r
   tcd_put_fix(op, slice, row, j, t);
 }
 
-// D_d accumulators of one element -> sum_d D_d 2^(-12 - 8 d + scale), rounded
-// once at the 53rd bit or 2^(BITS - 62), whichever is coarser; the sum's
-// magnitude is below 2^(BITS + 1).  |D_d| <= 2^22 for d <= 4 (read from the
-// float's bits), < 2^23 after.
-template <int BITS>
+// 64-bit shifts that give 0 past 63.
+__device__ __forceinline__ unsigned long long tcd_shl(unsigned long long x, int k) {
+  unsigned long long y;
+  asm("shl.b64 %0, %1, %2;" : "=l"(y) : "l"(x), "r"(k));
+  return y;
+}
+__device__ __forceinline__ unsigned long long tcd_shr(unsigned long long x, int k) {
+  unsigned long long y;
+  asm("shr.u64 %0, %1, %2;" : "=l"(y) : "l"(x), "r"(k));
+  return y;
+}
+
+// D_d accumulators of one element -> sum_d D_d 2^(-12 - 8 d + scale).
+// |D_d| <= 2^22 for d <= 4 (read from the float's bits), < 2^23 after.
+// UNIT: the sum's magnitude is at most about 1 (tcd_sum_shift), and it is
+// rounded once, at the 53rd bit or 2^-62, whichever is coarser; else it may
+// reach 64 and is rounded at its 53rd bit.  A result below 2^-1022 is 0.
+template <bool UNIT>
 __device__ __forceinline__ double tcd_value(const float (&f)[8], int scale) {
   constexpr unsigned K = 0x4b400000u;  // bits of 1.5 2^23: D + K - K
   unsigned n[8];
@@ -165,16 +189,37 @@ __device__ __forceinline__ double tcd_value(const float (&f)[8], int scale) {
   for (int d = 5; d < 8; ++d) n[d] = (unsigned)__float2int_rn(f[d]);
   const int t01 = (int)(n[0] * 256u + n[1] - K * 257u), t23 = (int)(n[2] * 256u + n[3] - K * 257u);
   const int t45 = (int)(n[4] * 256u + n[5] - K * 256u), t67 = (int)(n[6] * 256u + n[7]);
+  // the sum is top 2^32 + low in units of 2^-68
   const long long top = (long long)t01 * 65536 + t23, low = (long long)t45 * 65536 + t67;
-  // in units of 2^(BITS - 62): top 2^32 + low in units of 2^-68
-  const long long V = (top << (26 - BITS)) + (low >> (6 + BITS));
-  const unsigned long long m = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
-  const int lz = __clzll((long long)m);
-  const unsigned long long X = m << lz;  // the sum is X 2^(-lz + BITS - 62)
-  const int E = 1023 + 63 + BITS - 62 - lz + scale;
-  if (m == 0 || E <= 0) return 0.0;
+  bool neg;
+  unsigned long long X;  // the magnitude is X 2^-z, X in [2^63, 2^64) unless 0
+  int z;
+  if constexpr (UNIT) {
+    const long long V = (top << 26) + (low >> 6);
+    neg = V < 0;
+    const unsigned long long m = neg ? 0ull - (unsigned long long)V : (unsigned long long)V;
+    const int lz = __clzll((long long)m);
+    X = m << (lz & 63);
+    z = 62 + lz;
+  } else {
+    const long long t = top + (low >> 32);
+    neg = t < 0;  // (the complement is one unit short of the magnitude)
+    unsigned long long h = (unsigned long long)(neg ? ~t : t);
+    unsigned long long l = (unsigned long long)(neg ? ~(unsigned)low : (unsigned)low) << 32;
+    z = 36;
+    if (h == 0) {  // less than 2^-36
+      h = l;
+      l = 0;
+      z = 100;
+    }
+    const int lz = __clzll((long long)h);
+    X = tcd_shl(h, lz) | tcd_shr(l, 64 - lz);  // (lz > 0 where l != 0)
+    z += lz;
+  }
+  const int E = 1023 + 63 - z + scale;
+  if (X == 0 || E <= 0) return 0.0;
   unsigned long long bits = (X >> 11) + ((X >> 10) & 1u);  // (carries into the exponent)
-  bits += (unsigned long long)((unsigned)(E - 1) | (V < 0 ? 0x800u : 0u)) << 52;
+  bits += (unsigned long long)((unsigned)(E - 1) | (neg ? 0x800u : 0u)) << 52;
   return __longlong_as_double((long long)bits);
 }
 
@@ -201,21 +246,19 @@ __device__ __forceinline__ void tcd_mma(uint32_t tmem, uint32_t A, uint32_t B,
   }
 }
 
-// 8 accumulator columns of this thread's row from each of the eight sums.
-__device__ __forceinline__ void tcd_ld(uint32_t taddr, float (&v)[8][8]) {
-  uint32_t r[8][8];
+// 4 accumulator columns of this thread's row from each of the eight sums.
+__device__ __forceinline__ void tcd_ld(uint32_t taddr, float (&v)[4][8]) {
+  uint32_t r[8][4];
 #pragma unroll
   for (int d = 0; d < 8; ++d)
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=r"(r[d][0]), "=r"(r[d][1]), "=r"(r[d][2]), "=r"(r[d][3]), "=r"(r[d][4]),
-          "=r"(r[d][5]), "=r"(r[d][6]), "=r"(r[d][7])
-        : "r"(taddr + 64 * d));
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[d][0]), "=r"(r[d][1]), "=r"(r[d][2]), "=r"(r[d][3])
+                 : "r"(taddr + 64 * d));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int d = 0; d < 8; ++d)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[d][i] = __uint_as_float(r[d][i]);
+    for (int i = 0; i < 4; ++i) v[i][d] = __uint_as_float(r[d][i]);
 }
 
 // Cooperative layout: in iteration it (0, 1) lane l of warp w handles row
@@ -233,36 +276,52 @@ __device__ __forceinline__ void tcd_load8(const double* src, double (&v)[8]) {
   }
 }
 
-// Exponent e >= -900 with max |x| of the row's 8 lanes below 2^e; 0 for a zero
-// row.  A NaN or infinity raises ERR_ZERO_PARTIAL.
-__device__ __forceinline__ int tcd_row_exp(const double (&x)[8], bool valid, int* err) {
+// Divides a row (8 lanes) by the power of two that brings its largest
+// magnitude into [1/2, 1); returns the exponent, 0 for a zero row.  Only
+// entries below 2^-64 of the largest can be flushed.  A NaN or infinity raises
+// ERR_ZERO_PARTIAL.  FP64 products are kept out of it: exponent fields.
+__device__ __forceinline__ int tcd_row_max(const double (&x)[8]) {
   int m = 0;
 #pragma unroll
   for (int i = 0; i < 8; ++i) m = max(m, tree_abs_bits(x[i]));
   m = max(m, __shfl_xor_sync(kFull, m, 1));
   m = max(m, __shfl_xor_sync(kFull, m, 2));
-  m = max(m, __shfl_xor_sync(kFull, m, 4));
-  const int E = m >> 20;
+  return max(m, __shfl_xor_sync(kFull, m, 4)) >> 20;
+}
+__device__ __forceinline__ int tcd_normalise(double (&x)[8], bool valid, int* err) {
+  int E = tcd_row_max(x), shift = 0;
+  if (__any_sync(kFull, valid && E < 64)) {  // close to or among the subnormals
+    if (valid && E < 64) {
+      shift = -128;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] *= 0x1p128;
+    }
+    E = tcd_row_max(x);
+  }
   if (valid && E == 0x7ff) atomicOr(err, ERR_ZERO_PARTIAL);
-  return E ? max(E - 1022, -900) : 0;  // (rows below 2^-900 vanish)
+  if (E == 0) return 0;
+  const int e = E - 1022;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int hi = __double2hiint(x[i]), field = (hi >> 20) & 0x7ff;
+    const bool keep = field > max(e, 0);
+    x[i] = __hiloint2double(keep ? hi - (e << 20) : 0, keep ? __double2loint(x[i]) : 0);
+  }
+  return e + shift;
 }
 
-// Exponent of a row of P, whose products are read with tcd_value<0>: 0 where
-// the row's absolute sum is at most about 1, as in every stochastic matrix
-// (P sums to one), else enough to bring the sum below 1.
-__device__ __forceinline__ int tcd_sum_exp(const double (&x)[8], int* err) {
-  const int e = tcd_row_exp(x, false, err);
-  unsigned sum = 0;  // in units of 2^-24 (entries above 1 decide by e)
+// s with sum |x| <= 2^s (about) over a normalised row.
+__device__ __forceinline__ int tcd_sum_shift(const double (&x)[8]) {
+  unsigned sum = 0;  // in units of 2^-20
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int hi = __double2hiint(x[i]), k = 1023 - ((hi >> 20) & 0x7ff);
-    const unsigned m = ((unsigned)hi & 0xfffffu) | 0x100000u;  // 2^20 at x = 1
-    sum += k < 0 ? 1u << 25 : k > 20 ? 0u : m << 4 >> k;
+    sum += k > 20 ? 0u : (((unsigned)hi & 0xfffffu) | 0x100000u) >> k;
   }
   sum += __shfl_xor_sync(kFull, sum, 1);
   sum += __shfl_xor_sync(kFull, sum, 2);
   sum += __shfl_xor_sync(kFull, sum, 4);
-  return sum <= (1u << 24) + (1u << 8) ? 0 : max(e, 0) + 6;
+  return sum <= 1u << 20 ? 0 : 12 - __clz(sum - 1);
 }
 
 // Row sums over the 8 lanes of both iterations' rows: 3 additions for two.
@@ -329,15 +388,11 @@ __device__ __forceinline__ void tcd_child(const LevelArgs<double>& a, int b, boo
   }
 }
 
-// Staged rows [128][kTcdLd] -> global rows, coalesced.
-__device__ __forceinline__ void tcd_store(const double* st, double* base, size_t stride, int c0,
-                                          int C) {
-  const int lane = threadIdx.x & 31;
-  for (int row = threadIdx.x >> 5; row < 128; row += kTcdThreads / 32) {
-    if (c0 + row >= C) return;
-    reinterpret_cast<double2*>(base + (size_t)(c0 + row) * stride)[lane] =
-        reinterpret_cast<const double2*>(st + row * kTcdLd)[lane];
-  }
+// Staging rows [128][kTcdLd], pairs of doubles: place of pair c of a row (of
+// 32), so that the eight lanes of a row write their own pairs without conflict.
+__device__ __forceinline__ int tcd_pair(int c) { return c ^ (c >> 3 & 3); }
+__device__ __forceinline__ double2* tcd_at(double* st, int row, int c) {
+  return reinterpret_cast<double2*>(st + row * kTcdLd) + tcd_pair(c);
 }
 
 struct TcdBars {
@@ -360,11 +415,47 @@ __device__ __forceinline__ uint32_t tcd_acc_addr(uint32_t tmem) {
   return tmem + ((uint32_t)(32 * ((threadIdx.x >> 5) & 3)) << 16) + tcd_acc_col();
 }
 
+// x + x E' -> global rows, from the rows x in the cooperative layout and the
+// accumulators of x E' (column exponents ecol), by way of the staging rows.
+// (Adding x on the way from there to the rows, straight from its registers,
+// saves a pass over the staging but not the stores' coalescing: 0.79 ms
+// against 0.76 for 61 taxa x 601 patterns.)
+__device__ __forceinline__ void tcd_store_sum(double* st, const double (&x)[2][8], uint32_t tmem,
+                                              const int* ecol, double* base, size_t stride, int c0,
+                                              int C) {
+  const int lane = threadIdx.x & 31, j = threadIdx.x & 7, col = tcd_acc_col();
+#pragma unroll
+  for (int it = 0; it < 2; ++it)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      *tcd_at(st, tcd_row(it), 4 * j + i) = make_double2(x[it][2 * i], x[it][2 * i + 1]);
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float f[4][8];
+    tcd_ld(tcd_acc_addr(tmem) + 4 * q, f);
+#pragma unroll
+    for (int i = 0; i < 4; i += 2) {
+      const int c = col + 4 * q + i;
+      double2* p = tcd_at(st, tcd_acc_row(), c >> 1);
+      const double2 v = *p;
+      *p = make_double2(v.x + tcd_value<true>(f[i], ecol[c]),
+                        v.y + tcd_value<true>(f[i + 1], ecol[c + 1]));
+    }
+  }
+  __syncthreads();
+  for (int row = threadIdx.x >> 5; row < 128; row += kTcdThreads / 32) {
+    if (c0 + row >= C) return;
+    reinterpret_cast<double2*>(base + (size_t)(c0 + row) * stride)[lane] = *tcd_at(st, row, lane);
+  }
+}
+
 // ---------------------------------------------------------------------------
-// Matrices (Eq. 1): P = I + V diag(expm1) Vinv of two (branch, category) units
-// per CTA (64 rows each), the rows V diag(e) sliced here, Vinv's digits from
-// the host.  Internal branches get the digits of P and of P', tips the FP64
-// tables P' and dP' (a second contraction with gamma lambda e^x).
+// Matrices (Eq. 1): E = P - I = V diag(expm1) Vinv of two (branch, category)
+// units per CTA (64 rows each), the rows V diag(e) sliced here, Vinv's digits
+// from the host.  Internal branches get the digits of E and of E', every row
+// with its own exponent, tips the FP64 tables P' and dP' (a second contraction
+// with gamma lambda e^x).
 // ---------------------------------------------------------------------------
 template <typename T>  // double only
 __global__ void __launch_bounds__(kTcdThreads) pmat_tcd_kernel(PmatArgs a) {
@@ -437,21 +528,20 @@ __global__ void __launch_bounds__(kTcdThreads) pmat_tcd_kernel(PmatArgs a) {
     ok = tc_block_wait(&bars.mma, pmma, pend_mma, a.err);
     if (!ok) break;
     const int row = tcd_acc_row(), s = row & 63;
+    const bool one = d == 0 && (u0 + (row >> 6)) / R < a.n_tips;  // a tip's P, not E
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      float acc[8][8];
-      const int t0 = tcd_acc_col() + 8 * q;
-      tcd_ld(tcd_acc_addr(tmem) + 8 * q, acc);
-      double v[8];
+    for (int q = 0; q < 4; ++q) {
+      float f[4][8];
+      const int t0 = tcd_acc_col() + 4 * q;
+      tcd_ld(tcd_acc_addr(tmem) + 4 * q, f);
+      double v[4];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float f[8] = {acc[0][i], acc[1][i], acc[2][i], acc[3][i],
-                            acc[4][i], acc[5][i], acc[6][i], acc[7][i]};
-        v[i] = tcd_value<6>(f, erow[row] + ecol[t0 + i]);
-        if (d == 0 && s == t0 + i && s < S) v[i] += 1.0;
+      for (int i = 0; i < 4; ++i) {
+        v[i] = tcd_value<false>(f[i], erow[row] + ecol[t0 + i]);
+        if (one && s == t0 + i && s < S) v[i] += 1.0;
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 2; ++i)
         *reinterpret_cast<double2*>(stage + row * kTcdLd + t0 + 2 * i) =
             make_double2(v[2 * i], v[2 * i + 1]);
     }
@@ -469,7 +559,7 @@ __global__ void __launch_bounds__(kTcdThreads) pmat_tcd_kernel(PmatArgs a) {
         for (int i = tid; i < 64 * 64; i += kTcdThreads)
           tab[i] = st[(i & 63) * kTcdLd + (i >> 6)];
       } else if (d == 0) {
-        // one 8-element chunk of P and one of P' per thread
+        // one 8-element chunk of E and one of E' per thread
         const int r8 = tid >> 3;
         double x[8], y[8];
 #pragma unroll
@@ -477,13 +567,15 @@ __global__ void __launch_bounds__(kTcdThreads) pmat_tcd_kernel(PmatArgs a) {
           x[i] = st[r8 * kTcdLd + 8 * j + i];
           y[i] = st[(8 * j + i) * kTcdLd + r8];
         }
-        const int ep = tcd_sum_exp(x, a.err);
-        tcd_put(out, 64 * 128, r8, j, x, ep);
-        const int e = tcd_row_exp(y, false, a.err);
-        tcd_put(out + kTcdB, 64 * 128, r8, j, y, e);
+        const int ep = tcd_normalise(x, r8 < S, a.err);
+        const int sp = tcd_sum_shift(x);
+        tcd_put(out, 64 * 128, r8, j, x, sp);
+        const int e = tcd_normalise(y, r8 < S, a.err);
+        const int sy = tcd_sum_shift(y);
+        tcd_put(out + kTcdB, 64 * 128, r8, j, y, sy);
         if (j == 0) {
-          reinterpret_cast<int*>(out + 2 * kTcdB)[r8] = e;
-          reinterpret_cast<int*>(out + 2 * kTcdB)[64 + r8] = ep;
+          reinterpret_cast<int*>(out + 2 * kTcdB)[r8] = e + sy;
+          reinterpret_cast<int*>(out + 2 * kTcdB)[64 + r8] = ep + sp;
         }
       }
     }
@@ -508,7 +600,7 @@ __global__ void __launch_bounds__(kTcdThreads) post_tcd_kernel(LevelArgs<T> a) {
   unsigned char* B = A + kTcdA;
   double* stage = reinterpret_cast<double*>(A);
   __shared__ TcdBars bars;
-  __shared__ int erow[64];  // exponents of P_k's rows
+  __shared__ int erow[64];  // exponents of E_k's rows
   const int tid = threadIdx.x, warp = tid >> 5, j = tid & 7;
   const int R = a.n_cat, C = a.n_patterns;
   const int4 d = a.level_desc[blockIdx.y];
@@ -518,7 +610,7 @@ __global__ void __launch_bounds__(kTcdThreads) post_tcd_kernel(LevelArgs<T> a) {
     if (tid != 0) return;
     mbar_init_fenced(&bars.tma, 1);
     mbar_init_fenced(&bars.mma, 1);
-    tcd_copy_b(B, tcd_unit(a, k, r), &bars.tma);  // digits of P_k
+    tcd_copy_b(B, tcd_unit(a, k, r), &bars.tma);  // digits of E_k
   };
   if (a.mats_ready) issue();
   pdl_wait_and_release();
@@ -534,8 +626,8 @@ __global__ void __launch_bounds__(kTcdThreads) post_tcd_kernel(LevelArgs<T> a) {
     const int row = tcd_row(it), c = c0 + row;
 #pragma unroll
     for (int i = 0; i < 8; ++i) p[it][i] *= u[it][i];
-    const int er = tcd_row_exp(p[it], c < C, a.err);
-    tcd_put(A, 128 * 128, row, j, p[it], er);
+    const int er = tcd_normalise(p[it], c < C, a.err);
+    tcd_put(A, 128 * 128, row, j, p[it]);
     if (j == 0 && c < C) a.escale[(slot * R + r) * a.escale_stride + c] = e[it] + e1[it] + er;
   }
   tc::fence_smem_for_async();
@@ -553,25 +645,8 @@ __global__ void __launch_bounds__(kTcdThreads) post_tcd_kernel(LevelArgs<T> a) {
     }
     ok = tc_block_wait(&bars.mma, pmma, pend_mma, a.err);
   }
-  if (ok) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      float acc[8][8];
-      tcd_ld(tcd_acc_addr(tmem) + 8 * q, acc);
-      double* st = stage + tcd_acc_row() * kTcdLd + tcd_acc_col() + 8 * q;
-#pragma unroll
-      for (int i = 0; i < 8; i += 2) {
-        const float f[8] = {acc[0][i], acc[1][i], acc[2][i], acc[3][i],
-                            acc[4][i], acc[5][i], acc[6][i], acc[7][i]};
-        const float g[8] = {acc[0][i + 1], acc[1][i + 1], acc[2][i + 1], acc[3][i + 1],
-                            acc[4][i + 1], acc[5][i + 1], acc[6][i + 1], acc[7][i + 1]};
-        *reinterpret_cast<double2*>(st + i) = make_double2(
-            tcd_value<0>(f, erow[tcd_acc_col() + 8 * q + i]),
-            tcd_value<0>(g, erow[tcd_acc_col() + 8 * q + i + 1]));
-      }
-    }
-    __syncthreads();
-    tcd_store(stage, a.post + (slot * C * R + r) * 64, (size_t)R * 64, c0, C);
+  if (ok) {  // U_k = p_k + E_k p_k
+    tcd_store_sum(stage, p, tmem, erow, a.post + (slot * C * R + r) * 64, (size_t)R * 64, c0, C);
   }
   if (tid == 0) {
     if (pend_tma >= 0) (void)mbar_wait(&bars.tma, (uint32_t)pend_tma);
@@ -659,7 +734,7 @@ __global__ void __launch_bounds__(kTcdThreads) pre_tcd_kernel(LevelArgs<T> a) {
   double* stage = reinterpret_cast<double*>(A);
   __shared__ TcdBars bars;
   __shared__ double nums[4][128];
-  __shared__ int ecol[64], ecol_p[64];  // column exponents of Q and P_x
+  __shared__ int ecol[64], ecol_p[64];  // column exponents of Q and E_x
   const int tid = threadIdx.x, warp = tid >> 5, j = tid & 7;
   const int R = a.n_cat, C = a.n_patterns, S = a.n_states;
   const int4 d = a.level_desc[blockIdx.y];
@@ -727,13 +802,13 @@ __global__ void __launch_bounds__(kTcdThreads) pre_tcd_kernel(LevelArgs<T> a) {
       return;  // block-uniform: no barrier, copy or TMEM is in use
     }
   }
-  // ---- internal child: [W_x; q_x] = a_x [Q; P_x], a_x normalised per row ----
+  // ---- internal child: W_x = a_x Q, q_x = a_x + a_x E_x, a_x normalised per row ----
   int ea[2];
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
     const int row = tcd_row(it), c = c0 + row;
-    ea[it] = tcd_row_exp(av[it], c < C, a.err);
-    tcd_put(A, 128 * 128, row, j, av[it], ea[it]);
+    ea[it] = tcd_normalise(av[it], c < C, a.err);
+    tcd_put(A, 128 * 128, row, j, av[it]);
     if (j == 0 && c < C)
       a.pre_escale[(xslot * R + r) * estr + c] = ea[it] + eq[it] + ey[it];
   }
@@ -754,23 +829,21 @@ __global__ void __launch_bounds__(kTcdThreads) pre_tcd_kernel(LevelArgs<T> a) {
   }
   const int arow = tcd_acc_row(), acol = tcd_acc_col();
   if (ok) {
-    // Q's digits have been read: P_x' takes their place
+    // Q's digits have been read: E_x' takes their place
     if (tid == 0) tcd_copy_b(B, tcd_unit(a, bx, r) + kTcdB, &bars.tma);
     const int c = c0 + arow;
     const double* ux = a.post + ((xslot * C + (c < C ? c : 0)) * R + r) * 64 + acol;
     double num = 0.0;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      double uu[8];
-      tcd_load8(ux + 8 * q, uu);
-      float acc[8][8];
-      tcd_ld(tcd_acc_addr(tmem) + 8 * q, acc);
+    for (int q = 0; q < 4; ++q) {
+      const double2 u0 = reinterpret_cast<const double2*>(ux)[2 * q],
+                    u1 = reinterpret_cast<const double2*>(ux)[2 * q + 1];
+      const double uu[4] = {u0.x, u0.y, u1.x, u1.y};
+      float f[4][8];
+      tcd_ld(tcd_acc_addr(tmem) + 4 * q, f);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float f[8] = {acc[0][i], acc[1][i], acc[2][i], acc[3][i],
-                            acc[4][i], acc[5][i], acc[6][i], acc[7][i]};
-        num = fma(tcd_value<6>(f, ecol[acol + 8 * q + i]), uu[i], num);
-      }
+      for (int i = 0; i < 4; ++i)
+        num = fma(tcd_value<false>(f[i], ecol[acol + 4 * q + i]), uu[i], num);
     }
     nums[acol >> 4][arow] = num;
     tc::fence_before();
@@ -790,23 +863,8 @@ __global__ void __launch_bounds__(kTcdThreads) pre_tcd_kernel(LevelArgs<T> a) {
     ok = tc_block_wait(&bars.mma, pmma, pend_mma, a.err);
   }
   if (ok) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      float acc[8][8];
-      tcd_ld(tcd_acc_addr(tmem) + 8 * q, acc);
-      double* st = stage + arow * kTcdLd + acol + 8 * q;
-#pragma unroll
-      for (int i = 0; i < 8; i += 2) {
-        const float f[8] = {acc[0][i], acc[1][i], acc[2][i], acc[3][i],
-                            acc[4][i], acc[5][i], acc[6][i], acc[7][i]};
-        const float g[8] = {acc[0][i + 1], acc[1][i + 1], acc[2][i + 1], acc[3][i + 1],
-                            acc[4][i + 1], acc[5][i + 1], acc[6][i + 1], acc[7][i + 1]};
-        *reinterpret_cast<double2*>(st + i) = make_double2(tcd_value<6>(f, ecol_p[acol + 8 * q + i]),
-                         tcd_value<6>(g, ecol_p[acol + 8 * q + i + 1]));
-      }
-    }
-    __syncthreads();
-    tcd_store(stage, a.pre + (xslot * C * R + r) * 64, (size_t)R * 64, c0, C);
+    tcd_store_sum(stage, av, tmem, ecol_p, a.pre + (xslot * C * R + r) * 64, (size_t)R * 64, c0,
+                  C);
   }
   if (tid == 0) {
     if (pend_tma >= 0) (void)mbar_wait(&bars.tma, (uint32_t)pend_tma);

@@ -173,8 +173,8 @@ constexpr size_t kTcQtBytes = 3 * 64 * 128;
 
 // FP64 with 21..64 states runs on the tensor cores as well, in exact integer
 // arithmetic on base-256 digits (kernels_tcd.cuh): per (branch, category) an
-// internal branch's P and P' as eight-digit operands, the exponents of their
-// rows (P' first), a tip's P' and dP' in FP64.
+// internal branch's E = P - I and E' as eight-digit operands, the exponents of
+// their rows (E' first), a tip's P' and dP' in FP64.
 inline bool uses_tcd(int SP, bool fp64) { return SP == 64 && fp64; }
 constexpr uint32_t kTcdDigits = 8 * 64 * 128;           // one 64 x 64 operand
 constexpr size_t kTcdUnitBytes = 2 * (size_t)kTcdDigits + 128 * sizeof(int);
