@@ -21,6 +21,7 @@
 // sum_r w_r den; sum_c W_c g_{i,c} is reduced per tile in FP64.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 

@@ -1,6 +1,6 @@
 // Whole-pass kernels for 4 padded states (nucleotide models): one launch
-// walks every level of a pass, in FP64 at any size and in FP32 for problems
-// too small to fill the GPU level by level.
+// walks every level of a pass, or a run of levels, in FP64 at any size and in
+// FP32 for problems too small to fill the GPU level by level.
 //
 // Site patterns never mix before the final sums, so a tile of patterns can
 // climb (post-order) or descend (pre-order) the whole tree on its own: only
@@ -199,14 +199,14 @@ __device__ __forceinline__ void tree_put_q(T* Qs, const LevelArgs<T>& a) {
 
 template <typename T, int RP>
 __global__ void __launch_bounds__(kTreeThreads)
-tree4_post_kernel(LevelArgs<T> a, TreeSched s) {
+tree4_post_kernel(LevelArgs<T> a, TreeSched s, int first, int last) {
   const TreeLane<RP> t(a.n_patterns, a.n_cat);
   const int C = a.n_patterns, R = a.n_cat, S = a.n_states;
   pdl_wait_and_release();
-  int lo = s.off[0];
-  for (int l = 0; l < s.n_levels; ++l) {
+  int lo = s.off[first];
+  for (int l = first; l < last; ++l) {
     const int hi = s.off[l + 1];
-    for (int i = lo + t.warp; i < hi; i += kTreeWarps) {
+    for (int i = lo + blockIdx.y * kTreeWarps + t.warp; i < hi; i += gridDim.y * kTreeWarps) {
       const int4 d = s.desc[i];
       const int k = d.x;
       T p[4], uj[4];
@@ -303,7 +303,7 @@ __device__ __forceinline__ void tree_tile_sum(const LevelArgs<T>& a, int tile, i
 
 template <typename T, int RP>
 __global__ void __launch_bounds__(kTreeThreads)
-tree4_pre_kernel(LevelArgs<T> a, TreeSched s) {
+tree4_pre_kernel(LevelArgs<T> a, TreeSched s, int first, int last) {
   __shared__ __align__(16) T Qs[RP * 16];
   const TreeLane<RP> t(a.n_patterns, a.n_cat);
   const int C = a.n_patterns, R = a.n_cat, S = a.n_states;
@@ -313,10 +313,10 @@ tree4_pre_kernel(LevelArgs<T> a, TreeSched s) {
   const T W = t.valid ? a.pattern_wt[t.c] : T(0);
   __syncthreads();
   pdl_wait_and_release();
-  int lo = s.off[0];
-  for (int l = 0; l < s.n_levels; ++l) {
+  int lo = s.off[first];
+  for (int l = first; l < last; ++l) {
     const int hi = s.off[l + 1];
-    for (int i = lo + t.warp; i < hi; i += kTreeWarps) {
+    for (int i = lo + blockIdx.y * kTreeWarps + t.warp; i < hi; i += gridDim.y * kTreeWarps) {
       const int4 d = s.desc[i];
       const int k = d.x, b[2] = {d.y, d.z};
       T q[4], u[2][4];
@@ -641,15 +641,66 @@ cudaError_t prepare_walk4() {
   return e;
 }
 
+// The launches of a kByTile pass.  A block per tile leaves most of the GPU idle
+// where there are few tiles, and a wide level then waits for the FP64 pipes of
+// a few SMs.  So with room for two blocks per SM, a level of more than `wide`
+// nodes is a launch of its own, its nodes split over them, eight nodes or more
+// a block; the levels between two of those stay in one launch.  4 categories,
+// one launch a pass -> with the split (one launch per level): 1,024 taxa x 100
+// patterns 1103 -> 320 us (726), 4,096 x 1 4117 -> 333 (913), 1,024 x 640 1702
+// -> 791 (1472), 100 x 100 184 -> 164 (386).  `wide`: a pre-order step has
+// three times the FP64 instructions of a post-order one, and a launch costs
+// about what 8 of its nodes take a block; 16 (and 48 for post-order) was slower
+// with few tiles (64 x 100: 124 us against 112).
+template <typename F>
+cudaError_t tree_launches(const TreeSched& s, int n_tiles, int wide, F launch) {
+  const int most = 2 * kSms / n_tiles;  // blocks per tile
+  int first = 0;
+  for (int l = 0; l <= s.n_levels; ++l) {
+    const int w = l < s.n_levels ? s.host_off[l + 1] - s.host_off[l] : 0;
+    const bool own = most > 1 && w > wide;
+    if ((own || l == s.n_levels) && first < l) {
+      const cudaError_t e = launch(first, l, 1);
+      if (e != cudaSuccess) return e;
+    }
+    if (own) {
+      const cudaError_t e =
+          launch(l, l + 1, std::min(most, (w + kTreeWarps - 1) / kTreeWarps));
+      if (e != cudaSuccess) return e;
+      first = l + 1;
+    }
+  }
+  return cudaSuccess;
+}
+
+// A block that starts early is placed while its predecessor's blocks hold
+// their SMs, and stays where it is: with tiles on more than a quarter of the
+// SMs some SMs then hold two long blocks and others none.  Those launches start
+// in turn (128 taxa x 1,000 patterns 252 -> 195 us, 256 x 500 271 -> 248);
+// below, the early start saves its microseconds (1,024 x 8: 256 -> 244).
+template <typename K, typename... Args>
+cudaError_t tree_launch(bool early, K kern, dim3 grid, cudaStream_t st, Args... args) {
+  if (early) return launch_pdl(kern, grid, kTreeThreads, 0, st, args...);
+  kern<<<grid, kTreeThreads, 0, st>>>(args...);
+  return cudaGetLastError();
+}
+
 template <typename T, int RP>
 cudaError_t launch_tree_rp(const LevelArgs<T>& a, const TreePass& p, cudaStream_t st) {
   if (p.walk) return launch_walk4<T, RP>(a, p, st);
   if constexpr (sizeof(T) == 8) {  // kByTile: FP64 only
-    const dim3 grid((unsigned)a.n_tiles), block(kTreeThreads);
+    const bool early = 4 * a.n_tiles <= kSms;
     cudaError_t e = cudaSuccess;
-    if (p.do_post) e = launch_pdl(tree4_post_kernel<T, RP>, grid, block, 0, st, a, p.post);
+    if (p.do_post)
+      e = tree_launches(p.post, a.n_tiles, 24, [&](int first, int last, int split) {
+        return tree_launch(early, tree4_post_kernel<T, RP>, dim3(a.n_tiles, split), st, a, p.post,
+                           first, last);
+      });
     if (p.do_pre && e == cudaSuccess)
-      e = launch_pdl(tree4_pre_kernel<T, RP>, grid, block, 0, st, a, p.pre);
+      e = tree_launches(p.pre, a.n_tiles, 8, [&](int first, int last, int split) {
+        return tree_launch(early, tree4_pre_kernel<T, RP>, dim3(a.n_tiles, split), st, a, p.pre,
+                           first, last);
+      });
     return e;
   }
   return cudaErrorInvalidValue;

@@ -384,6 +384,7 @@ cudaError_t enqueue_tree(phylo_ctx* ctx, bool do_post, bool do_pre, cudaStream_t
     TreeSched& s = post ? p.post : p.pre;
     s.desc = ctx->dev<int4>(post ? ctx->L.post_desc : ctx->L.pre_desc);
     s.off = ctx->dev<int>(post ? ctx->L.post_off : ctx->L.pre_off);
+    s.host_off = (post ? ctx->post_off : ctx->pre_off).data();
     s.n_levels = (int)(post ? ctx->post_off : ctx->pre_off).size() - 1;
   }
   p.do_post = do_post;

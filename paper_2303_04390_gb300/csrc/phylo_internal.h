@@ -488,6 +488,7 @@ struct ReduceArgs {
 struct TreeSched {
   const int4* desc;
   const int* off;
+  const int* host_off;  // the same offsets on the host
   int n_levels;
 };
 struct TreePass {
