@@ -124,14 +124,19 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
 // B = B0 + B1 + B2 split into BF16 terms of decreasing magnitude (each
 // about 2^-8 of the previous one): the six products of order up to 2^-16,
 // A0B0 + A0B1 + A1B0 + A0B2 + A1B1 + A2B0, give FP32 accuracy; the dropped
-// ones are below 2^-24 relative.  a[t], b[t] are the shared addresses of
-// the term tiles (A: 128 rows, B: N rows).  One thread issues.
+// ones are below 2^-24 relative.  The tensor core cuts off what an addition
+// shifts below its accumulator's last bits, so the products are summed
+// smallest first: 4 instead of 24 additions to a sum of full size, and the
+// gradient of the 61- and 122-state paths is 2 to 3 times as close to FP64
+// (37 taxa x 389 codon patterns: 1.20e-6 -> 4.7e-7, 2-norm).  a[t], b[t] are
+// the shared addresses of the term tiles (A: 128 rows, B: N rows).  One thread
+// issues.
 template <int N>
 __device__ __forceinline__ void mma_split_bf16x3(uint32_t d_tmem, const uint32_t (&a)[3],
                                                  const uint32_t (&b)[3]) {
   constexpr uint32_t id = idesc_bf16(128, N);
-  constexpr int pa[6] = {0, 0, 1, 0, 1, 2};
-  constexpr int pb[6] = {0, 1, 0, 2, 1, 0};
+  constexpr int pa[6] = {2, 1, 0, 1, 0, 0};
+  constexpr int pb[6] = {0, 1, 2, 0, 1, 0};
 #pragma unroll
   for (int p = 0; p < 6; ++p)
 #pragma unroll
@@ -146,8 +151,8 @@ template <int N>
 __device__ __forceinline__ void mma_split_bf16x3_acc(uint32_t d_tmem, const uint32_t (&a)[3],
                                                      const uint32_t (&b)[3], bool accumulate) {
   constexpr uint32_t id = idesc_bf16(128, N);
-  constexpr int pa[6] = {0, 0, 1, 0, 1, 2};
-  constexpr int pb[6] = {0, 1, 0, 2, 1, 0};
+  constexpr int pa[6] = {2, 1, 0, 1, 0, 0};
+  constexpr int pb[6] = {0, 1, 2, 0, 1, 0};
 #pragma unroll
   for (int p = 0; p < 6; ++p)
 #pragma unroll
