@@ -789,26 +789,32 @@ __global__ void __launch_bounds__(kTcRows) root_u_kernel(LevelArgs<T> a) {
 // ---------------------------------------------------------------------------
 // Pre-order level (Eq. 4) with the per-category Eq. 8 terms: one CTA per
 // (tile, unit, category).  A unit (pre_units) is a node k with a child x to
-// contract; a compact tip's numerator needs no contraction, a_y . (G_y e) with
-// a_y = q_k o U_x, so it is formed in its sibling's unit from the rows loaded
-// there.  Against one CTA per child, with a contraction W_x = a_x Q for tips
-// too, that is half as many CTAs.
+// contract.
+//   TAB: a compact tip's numerator needs no contraction, a_y . (G_y e) with
+//   a_y = q_k o U_x, so it is formed in its sibling's unit from the rows loaded
+//   there.  Against one CTA per child, with a contraction W_x = a_x Q for tips
+//   too, that is half as many CTAs.
+//   Otherwise (small problems, where the CTAs have SMs to spare and a level
+//   takes one CTA's latency) a tip has its own unit, which keeps the lookup of
+//   G out of its sibling's.
 // ---------------------------------------------------------------------------
-template <typename T>  // float only
+template <typename T, bool TAB>  // T: float only
 __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
   static_assert(std::is_same<T, float>::value, "tensor-core path is FP32");
   static_assert(kStageBytes <= kOp128 && kStageBytes <= 2 * kOp64, "staging fits");
   static_assert(2 * kPt32Bytes <= kOp128, "the sibling's tables fit in the operand buffer");
+  static_assert(kPt32Bytes <= kOp64, "a lookup table fits in the P' buffer");
   extern __shared__ unsigned char smraw[];
   unsigned char* base = align1024(smraw);
   unsigned char* A = base;                     // a_x as three BF16 terms
-  // [P_x' | Q'] as one 128-row operand (rows = columns of P_x, then of Q): one
-  // chain of N = 128 MMAs where two of N = 64 took as many clocks each
+  // TAB: [P_x' | Q'] as one 128-row operand (rows = columns of P_x, then of Q),
+  // one chain of N = 128 MMAs where two of N = 64 took as many clocks each;
+  // otherwise P_x' (a tip: its FP32 P' for lookups), then Q', 64 rows each
   unsigned char* B = base + kOp128;
   float* stW = reinterpret_cast<float*>(A);    // W_x rows, after the MMAs
   float* stQ = reinterpret_cast<float*>(B);    // q_x rows, after the MMAs
-  // a compact sibling's tables (columns of P and of G = Q P, FP32) in A until
-  // the split
+  // a compact sibling's tables (columns of P and, with TAB, of G = Q P, FP32) in
+  // A until the split
   const float* pt32y = reinterpret_cast<const float*>(A);
   const float* gy = reinterpret_cast<const float*>(A + kPt32Bytes);
   __shared__ uint64_t bar_tma, bar_mma;
@@ -820,7 +826,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
   const int4 d = a.level_desc[blockIdx.z];
   const int k = d.x, r = (int)blockIdx.y;
   const int x = (d.w & kUnitSecond) ? 1 : 0;  // x's place among k's children
-  const TcChild cx = tc_child(a.n_tips, d.y, false);
+  const TcChild cx = tc_child(a.n_tips, d.y, !TAB && (d.w & kUnitCompactX));
   const TcChild cy = tc_child(a.n_tips, d.z, d.w & kUnitCompactY);
   const bool root = k == a.root;
   const size_t kslot = (size_t)(k - a.n_tips);
@@ -833,6 +839,15 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
     if (tid != 0) return;
     mbar_init_fenced(&bar_tma, 1);
     mbar_init_fenced(&bar_mma, 1);
+    if constexpr (!TAB) {
+      mbar_expect_tx(&bar_tma, kOp64 + (cx.internal ? kOp64 : 0) +
+                                   (cx.compact ? kPt32Bytes : 0) + (cy.compact ? kPt32Bytes : 0));
+      bulk_g2s(B + kOp64, a.qt, kOp64, &bar_tma);
+      if (cx.internal) bulk_g2s(B, unit_tiles(a, cx.b, r) + kUnitPt, kOp64, &bar_tma);
+      if (cx.compact) bulk_g2s(B, unit_tiles(a, cx.b, r) + kUnitPt32, kPt32Bytes, &bar_tma);
+      if (cy.compact) bulk_g2s(A, unit_tiles(a, cy.b, r) + kUnitPt32, kPt32Bytes, &bar_tma);
+      return;
+    }
     mbar_expect_tx(&bar_tma, kOp64 + (cx.internal ? kOp64 : 0) +
                                  (cy.compact ? 2 * kPt32Bytes : 0));
     for (int t = 0; t < 3; ++t) {
@@ -894,9 +909,18 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
   float* rt = reinterpret_cast<float*>(a.rterm);
   float den[4], ny[4];  // this lane's parts of the rows' sums
   if (ok) {
+    if constexpr (!TAB)
+      coop_child_u_finish(fx, cx.compact, reinterpret_cast<const float*>(B), S);
     coop_child_u_finish(fy, cy.compact, pt32y, S);
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
+      if constexpr (!TAB) {  // a_x = q_k o U_y (into q), den = a_x . U_x
+        q[2 * it] = mul4(q[2 * it], fy.v[2 * it]);
+        q[2 * it + 1] = mul4(q[2 * it + 1], fy.v[2 * it + 1]);
+        den[it] =
+            row_sum8(dot4(q[2 * it + 1], fx.v[2 * it + 1], dot4(q[2 * it], fx.v[2 * it], 0.f)));
+        continue;
+      }
       // a_y = q_k o U_x: den = a_y . U_y and a tip sibling's numerator;
       // then a_x = q_k o U_y (into q)
       const float4 b0 = mul4(q[2 * it], fx.v[2 * it]), b1 = mul4(q[2 * it + 1], fx.v[2 * it + 1]);
@@ -918,7 +942,14 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
       tc::fence_after();
       uint32_t ta[3], tb[3];
       term_addrs(A, kTerm128, ta);
-      if (cx.internal) {
+      if constexpr (!TAB) {
+        term_addrs(B + kOp64, kTerm64, tb);
+        tc::mma_split_bf16x3<64>(tmem + 64, ta, tb);
+        if (cx.internal) {
+          term_addrs(B, kTerm64, tb);
+          tc::mma_split_bf16x3<64>(tmem, ta, tb);
+        }
+      } else if (cx.internal) {
         term_addrs(B, kTerm128, tb);
         tc::mma_split_bf16x3<128>(tmem, ta, tb);
       } else {
@@ -928,7 +959,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
       tc::commit(&bar_mma);
     }
     // the Eq. 8 terms that need no contraction, during the MMAs
-    if (d.w & (kUnitDen | kUnitCompactY)) {
+    if (TAB && (d.w & (kUnitDen | kUnitNumY))) {
 #pragma unroll
       for (int it = 0; it < 4; ++it) {
         const float dn = row_sum8(den[it]), nn = row_sum8(ny[it]);
@@ -978,9 +1009,15 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_u_kernel(LevelArgs<T> a) {
       const int rr = coop_row(it), c = c0 + rr;
       const float4 w0 = *reinterpret_cast<const float4*>(stW + rr * kStageLd + 8 * j);
       const float4 w1 = *reinterpret_cast<const float4*>(stW + rr * kStageLd + 8 * j + 4);
-      const float num = row_sum8(dot4(w1, fx.v[2 * it + 1], dot4(w0, fx.v[2 * it], 0.f)));
+      float num = row_sum8(dot4(w1, fx.v[2 * it + 1], dot4(w0, fx.v[2 * it], 0.f)));
+      if (!TAB && cx.compact && fx.y[it] >= S) num = 0.f;  // d/dt of the all-ones vector is 0
       if (c < C && j == 0) {
-        rt[((kslot * C + c) * R + r) * 4 + x] = wg * num;
+        float* t4 = rt + ((kslot * C + c) * R + r) * 4;
+        t4[x] = wg * num;
+        if (!TAB && (d.w & kUnitDen)) {
+          t4[2] = wr * den[it];
+          t4[3] = __int_as_float(eq[it] + fx.E[it] + fy.E[it]);
+        }
         if (cx.internal)  // q_x = P_x' (q_k o U_y): exponents of q_k and of U_y
           a.pre_escale[((size_t)(cx.b - a.n_tips) * R + r) * estr + c] =
               eexp[rr] + eq[it] + fy.E[it];
@@ -1135,8 +1172,8 @@ inline cudaError_t launch_tc64(const LevelArgs<float>& a, bool post, cudaStream_
   if (post)
     return launch_pdl(post_u_kernel<float>, dim3(a.n_tiles, a.n_level, a.n_cat), kTcThreads,
                       kPostUSmem, st, a);
-  return launch_pdl(pre_u_kernel<float>, dim3(a.n_tiles, a.n_cat, a.n_level), kTcThreads,
-                    kPreUSmem, st, a);
+  return launch_pdl(a.tip_tables ? pre_u_kernel<float, true> : pre_u_kernel<float, false>,
+                    dim3(a.n_tiles, a.n_cat, a.n_level), kTcThreads, kPreUSmem, st, a);
 }
 
 template <typename T = float>
@@ -1146,7 +1183,7 @@ inline cudaError_t launch_pmat_tc64(const PmatArgs& a, cudaStream_t st) {
   // the reversible form has 136 blocks of (s, t) per unit: 5 warps
   pmat_tc_kernel<float><<<units, a.reversible ? 160 : kPmatTcThreads, kPmatTcSmem, st>>>(a);
   const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || !a.qn) return e;
   return launch_pdl(tipq_tc_kernel<float>, dim3((a.n_tips * a.n_cat + 1) / 2), kTcThreads,
                     kTipqSmem, st, a);
 }
@@ -1156,9 +1193,9 @@ inline cudaError_t prepare_tc64() {
   cudaError_t e = cudaFuncSetAttribute(post_u_kernel<float>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kPostUSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(pre_u_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kPreUSmem);
+  for (auto k : {pre_u_kernel<float, true>, pre_u_kernel<float, false>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPreUSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(tipq_tc_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kTipqSmem);

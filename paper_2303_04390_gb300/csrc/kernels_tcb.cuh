@@ -658,7 +658,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) pre_tcb_kernel(LevelArgs<T> a) 
   if (ok) {
     mma(false, 1);
     // the Eq. 8 terms that need no contraction, during the MMAs
-    if (d.w & (kUnitDen | kUnitCompactY)) {
+    if (d.w & (kUnitDen | kUnitNumY)) {
 #pragma unroll
       for (int it = 0; it < 4; ++it) {
         const float dn = row_sum8(den[it]), nn = row_sum8(ny[it]);

@@ -48,7 +48,7 @@ struct Layout {
   Region vsplit;  // tensor-core path: eigenvectors as double-float tables
   Region tc_tiles;  // 65..128 states, FP32: pre-split matrix blocks
   Region qt;        // 21..128 states, FP32, and 21..64, FP64: Q' as a tensor-core operand
-  Region qn;        // 21..128 states, FP32: Q as a tensor-core operand
+  Region qn;        // uses_tip_tables: Q as a tensor-core operand
   Region vdigits;   // 21..64 states, FP64, and 65..128, FP32: the digits of Vinv'
   Region qmat;      // 4 and 20 padded states, FP32: Q row-major
   Region tip_desc;  // U-form paths with tip partials: descriptors of the tips
@@ -136,8 +136,9 @@ const char* compute_layout(int N, int C, int S, int R, int prec, int flags,
   ok &= add_region(L, L.pre, L.mode == kWalk ? 0 : part);
   if (tc || uses_tc_big(L.SP, prec == PHYLO_FP64)) {
     ok &= add_region(L, L.qt, qt_bytes(L.SP));
-    ok &= add_region(L, L.qn, qt_bytes(L.SP));
   }
+  if (uses_tip_tables(L.SP, prec == PHYLO_FP64, N, L.n_tiles, R))
+    ok &= add_region(L, L.qn, qt_bytes(L.SP));
   if (tcd) {
     ok &= add_region(L, L.qt, digit_bytes(L.SP));
   }
@@ -329,6 +330,7 @@ LevelArgs<T> level_args(const phylo_ctx* ctx) {
   a.qmat = ctx->L.qmat.bytes ? ctx->dev<T>(ctx->L.qmat) : nullptr;
   a.rates = ctx->dev<double>(ctx->L.rates);
   a.quad = uses_quad(ctx->L.SP, ctx->precision == PHYLO_FP64, ctx->N, ctx->L.n_tiles);
+  a.tip_tables = ctx->L.qn.bytes != 0;
   a.tip_level = 0;
   return a;
 }
@@ -648,6 +650,7 @@ int upload_descriptors(phylo_ctx* ctx) {
     const std::vector<int>& nodes = pass == 0 ? ctx->post_nodes : ctx->pre_nodes;
     std::vector<int4> desc(nodes.size());
     if (pass == 1 && uses_units(ctx->L.SP, ctx->precision == PHYLO_FP64)) {
+      const bool tables = ctx->L.qn.bytes != 0;
       desc.clear();
       ctx->unit_off.assign(1, 0);
       for (size_t l = 0; l + 1 < ctx->pre_off.size(); ++l) {
@@ -655,13 +658,14 @@ int upload_descriptors(phylo_ctx* ctx) {
           const int2 ch = ctx->children[nodes[i]];
           int4 u[2];
           const int n = pre_units(nodes[i], ch.x, ch.y, ch.x < ctx->N && !ctx->tip_has[ch.x],
-                                  ch.y < ctx->N && !ctx->tip_has[ch.y], u);
+                                  ch.y < ctx->N && !ctx->tip_has[ch.y], tables, u);
           desc.insert(desc.end(), u, u + n);
         }
         ctx->unit_off.push_back((int)desc.size());
       }
-      // then the nodes whose children are both compact tips
+      // then, with tables, the nodes whose children are both compact tips
       for (int k : nodes) {
+        if (!tables) break;
         const int2 ch = ctx->children[k];
         if (ch.x < ctx->N && ch.y < ctx->N && !ctx->tip_has[ch.x] && !ctx->tip_has[ch.y])
           desc.push_back(make_int4(k, ch.x, ch.y, 0));
@@ -1134,9 +1138,11 @@ int phylo_set_eigen(phylo_ctx* ctx, const double* V, const double* Vinv,
     build_qt_tile(S, ctx->L.SP, V, Vinv, lambda, qt.data());
     if ((rc = upload(ctx, ctx->L.qt, qt.data(), qt.size(), "upload Q operand"))) return rc;
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
-    build_qt_tile(S, ctx->L.SP, V, Vinv, lambda, qt.data(), true);
-    if ((rc = upload(ctx, ctx->L.qn, qt.data(), qt.size(), "upload Q operand"))) return rc;
-    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+    if (ctx->L.qn.bytes) {
+      build_qt_tile(S, ctx->L.SP, V, Vinv, lambda, qt.data(), true);
+      if ((rc = upload(ctx, ctx->L.qn, qt.data(), qt.size(), "upload Q operand"))) return rc;
+      CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+    }
   }
   if ((rc = upload(ctx, ctx->L.lambda, lambda, (size_t)S, "upload lambda"))) return rc;
   if ((rc = upload(ctx, ctx->L.pi, pi, (size_t)S, "upload pi"))) return rc;

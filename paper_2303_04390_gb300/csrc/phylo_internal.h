@@ -18,29 +18,45 @@ namespace phylo {
 constexpr int kDescFlagCompact0 = 1, kDescFlagCompact1 = 2;
 constexpr int kDescFlagCherry0 = 4, kDescFlagCherry1 = 8;
 
-// Pre-order units of the FP32 tensor-core paths: {k, child x, sibling y, flags}.
-// A unit contracts the a of a child that is internal or has partial vectors;
-// a compact tip's numerator is a table lookup in its sibling's unit.  A node
-// whose children are both compact tips has none: its terms are lookups only,
-// which nothing waits for, and follow after the last level, for all such nodes
-// in one launch.
+// Pre-order units of the FP32 tensor-core paths: {k, child x, sibling y, flags};
+// a unit contracts the a of child x.  With tip tables (uses_tip_tables) only
+// children that are internal or have partial vectors have one: a compact tip's
+// numerator is a table lookup in its sibling's unit, and a node whose children
+// are both compact tips has none (its terms are lookups only, which nothing
+// waits for, and follow after the last level, for all such nodes in one
+// launch).  Without, every child has one.
 inline bool uses_units(int SP, bool fp64) { return (SP == 64 || SP == 128) && !fp64; }
 constexpr int kUnitCompactY = 1;  // y is a compact tip
 constexpr int kUnitSecond = 2;    // x is child 1 of k
 constexpr int kUnitDen = 4;       // writes the denominator
+constexpr int kUnitCompactX = 8;  // x is a compact tip
+constexpr int kUnitNumY = 16;     // writes y's numerator, from y's table
+// The tables (a launch after the matrix build) and the lookups of the nodes
+// with two tips (a launch after the last level) halve the CTAs of a level,
+// which pays once levels fill the GPU.  21..64 states, without -> with, by the
+// product below: 64 taxa x 100 patterns x 4 categories (256) 205 -> 224 us,
+// 64 x 1,100 x 1 (576) 185 -> 200, 128 x 200 x 4 (1,024) 275 -> 283,
+// 64 x 600 x 4 (1,280) 268 -> 276, 40 x 1,500 x 4 (1,920) 280 -> 270,
+// 30 x 3,000 x 4 (2,880) 310 -> 288.  65..128 states: with tables from the
+// smallest (8 x 50).
+inline bool uses_tip_tables(int SP, bool fp64, int n_tips, int n_tiles, int R) {
+  return uses_units(SP, fp64) && (SP == 128 || (long long)n_tips * n_tiles * R >= 1536);
+}
 // The units of node k with children (i, j); returns their number (0 to 2).
-inline int pre_units(int k, int i, int j, bool compact_i, bool compact_j, int4 (&out)[2]) {
-  if (compact_i && compact_j) return 0;
-  if (compact_j) {
-    out[0] = make_int4(k, i, j, kUnitCompactY | kUnitDen);
+inline int pre_units(int k, int i, int j, bool compact_i, bool compact_j, bool tables,
+                     int4 (&out)[2]) {
+  const int ci = compact_i ? 1 : 0, cj = compact_j ? 1 : 0;
+  if (tables && ci && cj) return 0;
+  if (tables && cj) {
+    out[0] = make_int4(k, i, j, kUnitCompactY | kUnitNumY | kUnitDen);
     return 1;
   }
-  if (compact_i) {
-    out[0] = make_int4(k, j, i, kUnitCompactY | kUnitSecond | kUnitDen);
+  if (tables && ci) {
+    out[0] = make_int4(k, j, i, kUnitCompactY | kUnitNumY | kUnitSecond | kUnitDen);
     return 1;
   }
-  out[0] = make_int4(k, i, j, kUnitDen);
-  out[1] = make_int4(k, j, i, kUnitSecond);
+  out[0] = make_int4(k, i, j, kUnitDen | ci * kUnitCompactX | cj * kUnitCompactY);
+  out[1] = make_int4(k, j, i, kUnitSecond | cj * kUnitCompactX | ci * kUnitCompactY);
   return 2;
 }
 
@@ -465,6 +481,7 @@ struct LevelArgs {
   const double* rates;         // [R] category rates gamma_r
   int quad;                    // FP32, 20 padded states: the partials' layout for four
                                // patterns per thread (kernels.cuh, uses_quad)
+  int tip_tables;              // uses_tip_tables
   int tip_level;               // U-form paths: the level's nodes are tips with
                                // partials (their U = P p, before level 1)
   int mats_ready;              // 1 if P was complete before the previous launch
@@ -500,8 +517,8 @@ struct TreePass {
 
 struct PmatArgs {
   const float* vsplit;   // tensor-core path: build_eigen_split's table
-  const unsigned char* qn;  // 21..128 states, FP32: Q as an operand (its rows), for the
-                            // tables Q P of compact tips
+  const unsigned char* qn;  // uses_tip_tables: Q as an operand (its rows), for the tables
+                            // Q P of compact tips (else null)
   const int* tip_has;    // [N] or nullptr: tips with partial vectors (no table)
   const void* vdigits;   // 21..64 states FP64, 65..128 FP32: the digits of Vinv'
                          // (build_digits)

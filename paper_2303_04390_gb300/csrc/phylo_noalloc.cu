@@ -127,7 +127,7 @@ void na_layout(int N, int C, int S, int R, NaLayout* Lp) {
   if (tc) {
     const size_t total = L.total;
     na_add(L, L.units, 2 * n_int * sizeof(int4));
-    na_add(L, L.qn, kTcQtBytes);
+    if (uses_tip_tables(L.SP, false, N, L.n_tiles, R)) na_add(L, L.qn, kTcQtBytes);
     L.total = total;
   }
   *Lp = L;
@@ -326,13 +326,14 @@ int phylo_evaluate_noalloc(int N, int C, int S, int R, const int32_t* parent,
         for (int i = l ? unit_end : 0; i < end; ++i) {
           const int2 c2 = ch[pre_nodes[i]];
           int4 u[2];
-          const int m = pre_units(pre_nodes[i], c2.x, c2.y, c2.x < N, c2.y < N, u);
+          const int m =
+              pre_units(pre_nodes[i], c2.x, c2.y, c2.x < N, c2.y < N, L.qn.bytes != 0, u);
           for (int v = 0; v < m; ++v) units[n_units++] = u[v];
         }
         unit_end = end;
         pre_off[l + 1] = n_units;
       }
-      for (int i = 0; i < N - 1; ++i) {  // then the nodes with two tips
+      for (int i = 0; i < N - 1 && L.qn.bytes; ++i) {  // then the nodes with two tips
         const int2 c2 = ch[pre_nodes[i]];
         if (c2.x < N && c2.y < N) units[n_units++] = make_int4(pre_nodes[i], c2.x, c2.y, 0);
       }
@@ -364,9 +365,11 @@ int phylo_evaluate_noalloc(int N, int C, int S, int R, const int32_t* parent,
   static thread_local unsigned char qt[2][kTcQtBytes];
   if (L.qt.bytes) {
     build_qt_tile(S, L.SP, V, Vinv, lambda, qt[0]);
-    build_qt_tile(S, L.SP, V, Vinv, lambda, qt[1], true);
     NA_TRY(up(L.qt, qt[0], kTcQtBytes), "upload Q operand");
-    NA_TRY(up(L.qn, qt[1], kTcQtBytes), "upload Q operand");
+    if (L.qn.bytes) {
+      build_qt_tile(S, L.SP, V, Vinv, lambda, qt[1], true);
+      NA_TRY(up(L.qn, qt[1], kTcQtBytes), "upload Q operand");
+    }
   }
   NA_TRY(up(L.lambda, lambda, (size_t)S * 8), "upload lambda");
   NA_TRY(up(L.pi, root_freqs, (size_t)S * 8), "upload pi");
@@ -435,6 +438,7 @@ int phylo_evaluate_noalloc(int N, int C, int S, int R, const int32_t* parent,
   a.n_tiles = L.n_tiles;
   a.err = flag;
   a.qt = L.qt.bytes ? reinterpret_cast<const unsigned char*>(ws + L.qt.off) : nullptr;
+  a.tip_tables = L.qn.bytes != 0;
   a.qmat = L.qmat.bytes ? reinterpret_cast<const float*>(ws + L.qmat.off) : nullptr;
   a.rates = reinterpret_cast<const double*>(ws + L.rates.off);
   a.tip_level = 0;
