@@ -1088,15 +1088,19 @@ cudaError_t launch_small(const LevelArgs<T>& a, bool post, cudaStream_t st) {
   if constexpr (kTrSmall<T, SP>) {  // FP32, 20 padded states: the U form
     // four patterns per thread on the levels that fill the GPU that way (two
     // blocks per SM), one elsewhere
-    if (a.quad && (long long)((a.n_tiles + 3) / 4) * a.n_level >= 2 * kSms)
-      return launch_q20<RP>(a, post, st);
+    constexpr bool Q = RP >= 4;  // (uses_quad: 3 categories or more)
+    if constexpr (Q) {
+      if (a.quad && (long long)((a.n_tiles + 3) / 4) * a.n_level >= 2 * kSms)
+        return launch_q20<RP>(a, post, st);
+    }
+    const bool ql = Q && a.quad;
     if (post) {
       dim3 grid(a.n_tiles, (a.n_level + NPo - 1) / NPo);
-      return launch_pdl(a.quad ? post_u20_kernel<RP, NPo, true> : post_u20_kernel<RP, NPo, false>,
+      return launch_pdl(ql ? post_u20_kernel<RP, NPo, Q> : post_u20_kernel<RP, NPo, false>,
                         grid, kSmallThreads, u20_smem<RP, NPo>(true), st, a);
     }
     dim3 grid(a.n_tiles, (a.n_level + NPr - 1) / NPr);
-    return launch_pdl(a.quad ? pre_u20_kernel<RP, NPr, true> : pre_u20_kernel<RP, NPr, false>,
+    return launch_pdl(ql ? pre_u20_kernel<RP, NPr, Q> : pre_u20_kernel<RP, NPr, false>,
                       grid, kSmallThreads, u20_smem<RP, NPr>(false), st, a);
   }
   if (post) {
@@ -1113,12 +1117,14 @@ template <typename T, int SP, int RP>
 cudaError_t prepare_small() {
   constexpr int NPo = SmallNpt<T, SP>::post, NPr = SmallNpt<T, SP>::pre;
   if constexpr (kTrSmall<T, SP>) {
-    cudaError_t e = prepare_q20<RP>();
-    for (auto k : {post_u20_kernel<RP, NPo, true>, post_u20_kernel<RP, NPo, false>})
+    constexpr bool Q = RP >= 4;
+    cudaError_t e = cudaSuccess;
+    if constexpr (Q) e = prepare_q20<RP>();
+    for (auto k : {post_u20_kernel<RP, NPo, Q>, post_u20_kernel<RP, NPo, false>})
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)u20_smem<RP, NPo>(true));
-    for (auto k : {pre_u20_kernel<RP, NPr, true>, pre_u20_kernel<RP, NPr, false>})
+    for (auto k : {pre_u20_kernel<RP, NPr, Q>, pre_u20_kernel<RP, NPr, false>})
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)u20_smem<RP, NPr>(false));

@@ -297,21 +297,17 @@ post_q20_kernel(LevelArgs<float> a) {
   if (t.lane == 0) a.lpart[t.tile] = term;
 }
 
-// Sums over a quad's RP lanes: afterwards a lane holds the sums of its own
-// patterns, i = r, r + min(RP, 4), ... in v[0], v[1], ... (RP = 8: lanes r < 4).
+// Sums over a quad's RP lanes: afterwards lane r < 4 holds the sum of its own
+// pattern, r, in v[0].
 template <int RP>
 __device__ __forceinline__ void q20_sum(float (&v)[4], int r) {
-  if constexpr (RP >= 2) {
-    const bool b = r & 1;
+  static_assert(RP >= 4, "a lane per pattern of the quad");
+  const bool odd = r & 1, two = r & 2;
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-      v[i] = (b ? v[2 * i + 1] : v[2 * i]) +
-             __shfl_xor_sync(kFull, b ? v[2 * i] : v[2 * i + 1], 1);
-  }
-  if constexpr (RP >= 4) {
-    const bool b = r & 2;
-    v[0] = (b ? v[1] : v[0]) + __shfl_xor_sync(kFull, b ? v[0] : v[1], 2);
-  }
+  for (int i = 0; i < 2; ++i)
+    v[i] = (odd ? v[2 * i + 1] : v[2 * i]) +
+           __shfl_xor_sync(kFull, odd ? v[2 * i] : v[2 * i + 1], 1);
+  v[0] = (two ? v[1] : v[0]) + __shfl_xor_sync(kFull, two ? v[0] : v[1], 2);
   if constexpr (RP == 8) v[0] += __shfl_xor_sync(kFull, v[0], 4);
 }
 
@@ -512,18 +508,15 @@ pre_q20_kernel(LevelArgs<float> a) {
   q20_sum<RP>(num[1], t.r);
   using A = Acc<float>;
   F2 g[2] = {A::zero(), A::zero()};
-  constexpr int ML = RP < 4 ? RP : 4;  // lanes that hold a quad's sums
-#pragma unroll
-  for (int i = 0; i < 4 / ML; ++i) {
-    const int c = t.c + t.r + ML * i;
-    if (t.r >= ML || c >= a.n_patterns) continue;
-    if (!(den[i] > 0.f) || !isfinite(den[i])) {
+  const int c = t.c + t.r;
+  if (t.r < 4 && c < a.n_patterns) {  // (lane r: pattern r of the quad)
+    if (!(den[0] > 0.f) || !isfinite(den[0])) {
       atomicOr(a.err, ERR_BAD_RATIO);
-      continue;
+    } else {
+      const float W = a.pattern_wt[c];
+      g[0] = A::prod(W, num[0][0] / den[0]);
+      g[1] = A::prod(W, num[1][0] / den[0]);
     }
-    const float W = a.pattern_wt[c];
-    g[0] = A::add(g[0], A::prod(W, num[0][i] / den[i]));
-    g[1] = A::add(g[1], A::prod(W, num[1][i] / den[i]));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {

@@ -329,7 +329,7 @@ LevelArgs<T> level_args(const phylo_ctx* ctx) {
   a.qt = ctx->L.qt.bytes ? ctx->dev<unsigned char>(ctx->L.qt) : nullptr;
   a.qmat = ctx->L.qmat.bytes ? ctx->dev<T>(ctx->L.qmat) : nullptr;
   a.rates = ctx->dev<double>(ctx->L.rates);
-  a.quad = uses_quad(ctx->L.SP, ctx->precision == PHYLO_FP64, ctx->N, ctx->L.n_tiles);
+  a.quad = uses_quad(ctx->L.SP, ctx->precision == PHYLO_FP64, ctx->N, ctx->L.n_tiles, ctx->R);
   a.tip_tables = ctx->L.qn.bytes != 0;
   a.tip_level = 0;
   return a;

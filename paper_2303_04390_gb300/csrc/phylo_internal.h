@@ -166,9 +166,11 @@ inline int walk_group(bool fp64, int n_tips, int C, int R, int RP) {
 // the nodes sit in the widest level).  4 categories, before -> after: 256 taxa x
 // 5,000 patterns 0.99 -> 0.84 ms, 500 x 1,000 0.58 -> 0.55, 16 x 10,000 0.182 ->
 // 0.176; below the line it loses (500 x 300: 0.37 -> 0.38, 96 x 1,201 0.25 ->
-// 0.26).
-inline bool uses_quad(int SP, bool fp64, int n_tips, int n_tiles) {
-  return SP == 20 && !fp64 && n_tiles >= 32 &&
+// 0.26).  With 3 categories or more a warp's matrix reads hit that many rows
+// and are what it saves; with 1 or 2 it loses (256 x 5,000: 1 category 293 ->
+// 306 us, 2 462 -> 490, 3 986 -> 909, 8 2,601 -> 1,984).
+inline bool uses_quad(int SP, bool fp64, int n_tips, int n_tiles, int R) {
+  return SP == 20 && !fp64 && R > 2 && n_tiles >= 32 &&
          (long long)((n_tiles + 3) / 4) * n_tips >= 8 * kSms;
 }
 inline PassMode pass_mode(int SP, bool fp64, int n_tips, int C, int R, int RP) {
