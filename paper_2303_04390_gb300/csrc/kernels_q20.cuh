@@ -538,10 +538,19 @@ constexpr size_t q20_smem(bool post) {
 }
 
 template <int RP>
-cudaError_t launch_q20(const LevelArgs<float>& a, bool post, cudaStream_t st) {
-  const dim3 grid((a.n_tiles + kQ20Threads / 32 - 1) / (kQ20Threads / 32), a.n_level);
-  if (post) return launch_pdl(post_q20_kernel<RP>, grid, kQ20Threads, q20_smem<RP>(true), st, a);
-  return launch_pdl(pre_q20_kernel<RP>, grid, kQ20Threads, q20_smem<RP>(false), st, a);
+cudaError_t launch_q20(LevelArgs<float> a, bool post, cudaStream_t st) {
+  // One node per grid row: 65,536 tips with partial vectors take two launches
+  // (each waits for the one before it, so the level after them sees both).
+  constexpr int kRows = 65535;
+  cudaError_t e = cudaSuccess;
+  for (int left = a.n_level; left > 0 && e == cudaSuccess; left -= kRows, a.level_desc += kRows) {
+    a.n_level = std::min(left, kRows);
+    const dim3 grid((a.n_tiles + kQ20Threads / 32 - 1) / (kQ20Threads / 32), a.n_level);
+    e = post ? launch_pdl(post_q20_kernel<RP>, grid, kQ20Threads, q20_smem<RP>(true), st, a)
+             : launch_pdl(pre_q20_kernel<RP>, grid, kQ20Threads, q20_smem<RP>(false), st, a);
+    a.mats_ready = 0;
+  }
+  return e;
 }
 
 template <int RP>
