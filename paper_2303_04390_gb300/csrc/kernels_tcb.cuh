@@ -787,7 +787,7 @@ inline cudaError_t launch_tcb(const LevelArgs<float>& a, bool post, cudaStream_t
 // contract, slice, contract, split) that one CTA per SM (512 TMEM columns)
 // does not hide.
 // ---------------------------------------------------------------------------
-// Sum of the accumulators of one element in FP32 (K = 128: |D_d| <= 2^22 only
+// Sum of the accumulators of one element in FP32, infinite past its range (K = 128: |D_d| <= 2^22 only
 // for d <= 2, < 2^24 after; the sum's magnitude below 2^8).
 __device__ __forceinline__ float tcb_digit_value(const float (&f)[8], int scale, bool one) {
   constexpr unsigned K = 0x4b400000u;
@@ -811,6 +811,7 @@ __device__ __forceinline__ float tcb_digit_value(const float (&f)[8], int scale,
   const unsigned long long X = m << lz;
   const int E = 127 + 63 + 7 - 62 - lz + scale;
   if (m == 0 || E <= 0) return 0.f;
+  if (E > 254) return V < 0 ? -INFINITY : INFINITY;
   const unsigned bits = ((unsigned)(E - 1) << 23) + (unsigned)(X >> 40) +
                         ((unsigned)(X >> 39) & 1u);
   return __uint_as_float(bits | (V < 0 ? 0x80000000u : 0u));

@@ -62,8 +62,8 @@ static_assert(128 * kTcdLd * 8 <= kTcdA, "staging fits in the operand buffer");
 constexpr size_t kTcdSmem = 1024 + kTcdA + kTcdB;
 constexpr uint32_t kTcdTab = 64 * 64 * 8;  // one FP64 table
 
-// The digits' fixed point of x, |x| <= 1, towards zero: x 2^62, plus the bias
-// that makes every byte a digit + 128.
+// The digits' fixed point of x / 2^s, |x| <= 2^s, towards zero: x 2^(62 - s),
+// plus the bias that makes every byte a digit + 128.
 __device__ __forceinline__ unsigned long long tcd_fix(double x, int s) {
   const int hi = __double2hiint(x);
   const unsigned lo = (unsigned)__double2loint(x);
