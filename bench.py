@@ -561,7 +561,7 @@ def fp64_path(pg, w, stream, K, barrier):
             "hbm_gbs_all_phases": sum(by64.values()) / (ms / K / 1e3) / 1e9}
 
 
-def rooflines(w, precision, phase_ms, level_counts, peaks, n_sm, workload):
+def rooflines(w, precision, phase_ms, phase_launches, peaks, n_sm, workload):
     """The dominant phase against its bound: HBM for 4 and 20 states (with
     the FP32 ALU rate beside it at 20 states), the tensor pipe for the
     tensor-core path (21-64 states, FP32; the HBM figure is the main
@@ -590,9 +590,7 @@ def rooflines(w, precision, phase_ms, level_counts, peaks, n_sm, workload):
         phases[n_] = {"ms": ms_, "algorithmic_bytes": by[n_],
                       "achieved_gbs": by[n_] / (ms_ / 1e3) / 1e9 if ms_ > 0 else None}
     dom = max(names, key=lambda n_: phases[n_]["ms"])
-    n_launch_dom = {"pmat": 1, "reduce": 1}.get(dom)
-    if n_launch_dom is None:
-        n_launch_dom = level_counts[0 if dom == "post" else 1]
+    n_launch_dom = phase_launches[names.index(dom)]
     achieved = phases[dom]["achieved_gbs"]
     tr = _traffic_record(dom, workload, precision)
     traffic = tr[0] if tr is not None else None
@@ -705,8 +703,7 @@ def run_ours(args):
     ms, per_step = m.steps(K, W, barrier)
     ms = max_over_ranks(ms)
     value = world * K / (ms / 1e3)
-    launches = m.ctx.launches_per_evaluation()
-    level_counts = m.ctx.level_counts()
+    launches, phase_launches = m.ctx.kernel_launches()
     # -- per-phase device times (four graph launches, events between) -----
     phase_ms = m.phases(min(max(K, 20), 200), barrier)
     # -- end to end through the C ABI with host buffers -------------------
@@ -737,7 +734,7 @@ def run_ours(args):
         pass
     n_sm = torch.cuda.get_device_properties(local).multi_processor_count
     roofline, tensor, phases, bytes_all = rooflines(
-        w, precision, phase_ms, level_counts, peaks, n_sm, args.workload)
+        w, precision, phase_ms, phase_launches, peaks, n_sm, args.workload)
 
     # -- the plain FP64 path on the same workload (>= 20 steps) -----------
     fp64 = None
@@ -756,7 +753,7 @@ def run_ours(args):
                 msx, perx = mx.steps(max(K, 20), max(W, 3), barrier)
                 kx = max(K, 20)
                 phx = mx.phases(min(max(K, 20), 200), barrier)
-                lcx = mx.ctx.level_counts()
+                lcx = mx.ctx.kernel_launches()[1]
             finally:
                 mx.close()
             rx, tx, phsx, _ = rooflines(wx, prec, phx, lcx, peaks, n_sm, name)

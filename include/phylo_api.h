@@ -215,21 +215,29 @@ int phylo_gradient_branch_sum(phylo_ctx* ctx, const int32_t* branches, const dou
  * the last check (PHYLO_ENUMERIC) or PHYLO_OK. */
 int phylo_check(phylo_ctx* ctx);
 
-/* Number of steps of one evaluation (the level schedule's length plus the
- * matrix build and the final reduction); 0 before the tree is set.  Each step
- * is one kernel launch, except that with up to 4 states the FP64 path, and
- * the FP32 path on problems of one wave of blocks, walk all the levels of a
- * pass in one launch. */
+/* Number of steps of one evaluation: the length of the level schedule
+ * (phylo_level_counts), the matrix build, the final reduction and, with 21 to
+ * 128 states, the steps between them (tables of the compact tips, Eq. 8
+ * ratios); 0 before the tree is set.  What is launched for them differs by
+ * path: phylo_kernel_launches counts it. */
 int phylo_launches_per_evaluation(const phylo_ctx* ctx);
 
 /* Length of the level schedule: the number of post-order steps (tree
  * height, less the heights left empty by fused cherries on the FP32
- * 4-state path; plus one for Eq. 3 at the root on the FP32 path for 65-128
- * states) and of pre-order steps (distinct depths of internal nodes;
- * twice that on the FP32 path for 65-128 states, which runs two kernels per
- * level).  Both 0 before the tree is set. */
+ * 4-state path; plus one for the tips with partial vectors on the FP32 paths
+ * for 5 to 128 states) and of pre-order steps (distinct depths of internal
+ * nodes).  Both 0 before the tree is set. */
 int phylo_level_counts(const phylo_ctx* ctx, int* n_post_levels,
                        int* n_pre_levels);
+
+/* Kernel launches of one evaluation, and of each of its four phases run apart
+ * (phases[4], as phylo_evaluate_device_timed runs them: matrices, post-order
+ * pass, pre-order pass, final reduction), counted in the captured sequences.
+ * Every input has to be set.  With up to 4 states the FP64 path, and the FP32
+ * path on problems of one wave of blocks, walk many or all levels of a pass, or
+ * both passes, in one launch; with 21 to 128 states a pre-order step without a
+ * contraction is not launched, and the nodes with two tips may take one more. */
+int phylo_kernel_launches(phylo_ctx* ctx, int* evaluation, int* phases);
 
 /* Self-test of the bounded device waits (no counterpart in the paper; the
  * kernels' asynchronous copies and MMAs complete on mbarriers, and every

@@ -60,6 +60,8 @@ SIGNATURES = {
     "phylo_launches_per_evaluation": (_c_int, [_vp]),
     "phylo_level_counts": (_c_int, [_vp, ctypes.POINTER(_c_int),
                                     ctypes.POINTER(_c_int)]),
+    "phylo_kernel_launches": (_c_int, [_vp, ctypes.POINTER(_c_int),
+                                       ctypes.POINTER(_c_int)]),
     "phylo_selftest_bounded_wait": (_c_int, [_c_int, _vp]),
     "phylo_last_error": (ctypes.c_char_p, [_vp]),
     "phylo_destroy": (_c_int, [_vp]),

@@ -284,14 +284,22 @@ class PhyloContext:
         self._check(self._lib.phylo_check(self._ctx))
 
     def launches_per_evaluation(self) -> int:
+        """Steps of one evaluation; `kernel_launches` counts the launches."""
         return int(self._lib.phylo_launches_per_evaluation(self._ctx))
 
     def level_counts(self):
-        """(post-order launches, pre-order launches) of one evaluation."""
+        """(post-order steps, pre-order steps) of the level schedule."""
         a, b = ctypes.c_int(0), ctypes.c_int(0)
         self._check(self._lib.phylo_level_counts(self._ctx, ctypes.byref(a),
                                                  ctypes.byref(b)))
         return int(a.value), int(b.value)
+
+    def kernel_launches(self):
+        """Kernel launches of one evaluation, and of its four phases run apart
+        (matrices, post-order, pre-order, reduction)."""
+        n, ph = ctypes.c_int(0), (ctypes.c_int * 4)()
+        self._check(self._lib.phylo_kernel_launches(self._ctx, ctypes.byref(n), ph))
+        return int(n.value), tuple(ph)
 
     def close(self):
         if getattr(self, "_ctx", None):

@@ -536,8 +536,24 @@ int ensure_host_out(phylo_ctx* ctx) {
   return PHYLO_OK;
 }
 
-// Capture a sequence of phases into an executable graph.
-int capture(phylo_ctx* ctx, unsigned seq, cudaGraphExec_t* exec) {
+// Kernel launches in a captured graph.
+cudaError_t count_kernels(cudaGraph_t g, int* kernels) {
+  size_t n = 0;
+  cudaError_t e = cudaGraphGetNodes(g, nullptr, &n);
+  std::vector<cudaGraphNode_t> nodes(n);
+  if (e == cudaSuccess && n) e = cudaGraphGetNodes(g, nodes.data(), &n);
+  *kernels = 0;
+  for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
+    cudaGraphNodeType type;
+    e = cudaGraphNodeGetType(nodes[i], &type);
+    *kernels += type == cudaGraphNodeTypeKernel;
+  }
+  return e;
+}
+
+// Capture a sequence of phases into an executable graph (exec may be null: the
+// launches are only counted).
+int capture(phylo_ctx* ctx, unsigned seq, cudaGraphExec_t* exec, int* kernels = nullptr) {
   int rc = ensure_capture_stream(ctx);
   if (rc) return rc;
   CUDA_TRY(ctx, cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal),
@@ -550,7 +566,12 @@ int capture(phylo_ctx* ctx, unsigned seq, cudaGraphExec_t* exec) {
     return cuda_fail(ctx, le, "kernel launch during capture");
   }
   if (ce != cudaSuccess) return cuda_fail(ctx, ce, "cudaStreamEndCapture");
-  cudaError_t ie = cudaGraphInstantiate(exec, g, 0);
+  cudaError_t ie = kernels ? count_kernels(g, kernels) : cudaSuccess;
+  if (ie != cudaSuccess) {
+    cudaGraphDestroy(g);
+    return cuda_fail(ctx, ie, "cudaGraphGetNodes");
+  }
+  if (exec) ie = cudaGraphInstantiate(exec, g, 0);
   cudaGraphDestroy(g);
   if (ie != cudaSuccess) {
     *exec = nullptr;
@@ -1508,6 +1529,18 @@ int phylo_launches_per_evaluation(const phylo_ctx* ctx) {
     if (has_tip_level(ctx)) ++n;                // U of the tips with partials
   }
   return n;
+}
+
+int phylo_kernel_launches(phylo_ctx* ctx, int* evaluation, int* phases) {
+  if (!ctx) return PHYLO_EINVAL;
+  if (!evaluation || !phases) return fail(ctx, PHYLO_EINVAL, "NULL argument");
+  int rc = check_ready(ctx);
+  if (rc) return rc;
+  rc = ensure_cuda_objects(ctx);
+  if (!rc && (ctx->graph_dirty || ctx->phase_dirty)) rc = upload_descriptors(ctx);
+  if (!rc) rc = capture(ctx, kSeqEvaluate, nullptr, evaluation);
+  for (int ph = 0; ph < kPhases && !rc; ++ph) rc = capture(ctx, 1u << ph, nullptr, phases + ph);
+  return rc;
 }
 
 int phylo_level_counts(const phylo_ctx* ctx, int* n_post_levels,
