@@ -94,13 +94,36 @@ def algorithmic_flops(w, precision="fp32"):
     P p, dP p and P' a.  The tensor-core form for 21..128 states (FP32)
     stores U = P p in the post-order pass and writes Eq. 8's numerator
     through dP = gamma Q P, so its pre-order pass needs P' a of every
-    internal child and Q' a of every child, tips included."""
+    internal child and Q' a of every child, tips included.  What the kernels
+    perform is less (contraction_flops): compact tips have tables."""
     N, C, S, R = w.n_tips, w.n_patterns, w.n_states, w.n_categories
     node = 2 * S * S * R * C
     if precision == "fp32" and 20 < S <= 128:
         return {"pmat": 0, "post": node * (N - 2),
                 "pre": node * ((N - 2) + (2 * N - 2)), "reduce": 0}
     return {"pmat": 0, "post": node * (N - 2), "pre": 3 * node * (N - 2), "reduce": 0}
+
+
+def contraction_flops(w, precision="fp32"):
+    """The dense contractions that are performed (2 S^2 flops per matrix-vector
+    product): P p of every internal non-root node in the post-order pass; in
+    the pre-order pass P' a and a' Q of every internal child where the
+    post-order pass stores U = P p (FP32 up to 128 states, FP64 up to 4 and
+    with 21 to 64), else P p, dP p and P' a.  A compact tip's products are
+    column lookups; its table of Q P (FP32, 65 to 128 states, and 21 to 64 on
+    all but small problems) counts with the matrices, and on small problems
+    its a' Q with the pre-order pass."""
+    N, C, S, R = w.n_tips, w.n_patterns, w.n_states, w.n_categories
+    node = 2 * S * S * R * C
+    u_form = S <= 4 or 20 < S <= 64 or (precision == "fp32" and S <= 128)
+    pre = (2 if u_form else 3) * node * (N - 2)
+    pmat = 0
+    if precision == "fp32" and 20 < S <= 128:
+        if S > 64 or N * -(-C // 128) * R >= 1536:
+            pmat = 2 * S ** 3 * N * R
+        else:
+            pre += node * N
+    return {"pmat": pmat, "post": node * (N - 2), "pre": pre, "reduce": 0}
 
 
 # ---------------------------------------------------------------------------
@@ -570,7 +593,7 @@ def rooflines(w, precision, phase_ms, phase_launches, peaks, n_sm, workload):
     peak_kind = "measured" if hbm_peak else "fallback"
     hbm_peak = hbm_peak or 6800.0
     by = algorithmic_bytes(w, precision)
-    fl = algorithmic_flops(w, precision)
+    fl = contraction_flops(w, precision)
     names = ["pmat", "post", "pre", "reduce"]
     kernels = {"pmat": "pmat_kernel", "post": "post-order level kernel",
                "pre": "pre-order level kernel (fused gradient)",
