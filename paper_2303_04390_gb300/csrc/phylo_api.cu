@@ -1110,14 +1110,16 @@ int phylo_set_eigen(phylo_ctx* ctx, const double* V, const double* Vinv,
   }
   if (std::fabs(psum - 1.0) > 1e-10)
     return fail(ctx, PHYLO_EINVAL, "root frequencies sum to %.17g, not 1", psum);
-  for (int i = 0; i < S; ++i)
+  const std::vector<double> ones(S, 1.0);
+  double row[kMaxStates];
+  for (int i = 0; i < S; ++i) {
+    q_row(S, V, Vinv, ones.data(), i, row);  // (V 1) Vinv: the same products
     for (int j = 0; j < S; ++j) {
-      double acc = 0.0;
-      for (int m = 0; m < S; ++m) acc += V[i * S + m] * Vinv[m * S + j];
-      const double want = i == j ? 1.0 : 0.0;
+      const double acc = row[j], want = i == j ? 1.0 : 0.0;
       if (!std::isfinite(acc) || std::fabs(acc - want) > 1e-8)
         return fail(ctx, PHYLO_EINVAL, "V * Vinv differs from I at (%d,%d)", i, j);
     }
+  }
   std::vector<double> bV, bW;
   if (ctx->L.vdigits.bytes) {  // the same decomposition, scaled for fixed point
     bV.assign(V, V + (size_t)S * S);

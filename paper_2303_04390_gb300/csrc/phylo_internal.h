@@ -206,8 +206,20 @@ constexpr size_t kTcdUnitBytes = 2 * (size_t)kTcdDigits + 128 * sizeof(int);
 inline size_t digit_bytes(int SP) {
   return (size_t)(SP / 64) * (SP / 64) * kTcdDigits + SP * sizeof(int);
 }
+// FP16 of the integers -128 .. 127 (index + 128).
+struct DigitHalves {
+  uint16_t h[256];
+  DigitHalves() {
+    for (int d = -128; d < 128; ++d) {
+      int ex;
+      const double f = std::frexp(std::fabs((double)d), &ex);
+      h[d + 128] = d ? (uint16_t)((d < 0 ? 0x8000 : 0) + ((ex + 13) << 10) + (int)(f * 2048.0)) : 0;
+    }
+  }
+};
 template <typename F>
 inline void build_digits(int S, int SP, F M, unsigned char* out) {
+  static const DigitHalves halves;
   const int NB = SP / 64;
   std::memset(out, 0, digit_bytes(SP));
   for (int n = 0; n < S; ++n) {
@@ -221,16 +233,9 @@ inline void build_digits(int S, int SP, F M, unsigned char* out) {
       const long long v = std::llrint(std::ldexp(M(n, k), 62 - e));
       const uint64_t t = (uint64_t)v + 0x8080808080808080ull;
       for (int i = 0; i < 8; ++i) {
-        const int digit = (int)(t >> (56 - 8 * i) & 0xff) - 128;
-        uint16_t h = 0;  // FP16 of an integer below 2^11
-        if (digit) {
-          int ex;
-          const double f = std::frexp(std::fabs((double)digit), &ex);
-          h = (uint16_t)((digit < 0 ? 0x8000 : 0) + ((ex + 13) << 10) + (int)(f * 2048.0));
-        }
         const size_t off = (size_t)(n & 63) * 128 +
                            ((size_t)(((k & 63) >> 3) ^ (n & 7)) << 4) + (k & 7) * 2;
-        std::memcpy(blk + (size_t)i * 64 * 128 + off, &h, 2);
+        std::memcpy(blk + (size_t)i * 64 * 128 + off, &halves.h[t >> (56 - 8 * i) & 0xff], 2);
       }
     }
   }
@@ -286,6 +291,16 @@ inline float host_bf16_value(uint16_t b) {
   return f;
 }
 
+// Row t of Q = V diag(lambda) Vinv, every entry summed over m in order.
+inline void q_row(int S, const double* V, const double* Vinv, const double* lambda, int t,
+                  double (&row)[kMaxStates]) {
+  for (int s = 0; s < S; ++s) row[s] = 0.0;
+  for (int m = 0; m < S; ++m) {
+    const double a = V[t * S + m] * lambda[m];
+    for (int s = 0; s < S; ++s) row[s] += a * Vinv[m * S + s];
+  }
+}
+
 // Bytes of the Q' operand for SP = 64 or 128 padded states: (SP / 64)^2
 // blocks of 64 x 64 three-term BF16 values.
 inline size_t qt_bytes(int SP) { return (size_t)(SP / 64) * (SP / 64) * kTcQtBytes; }
@@ -305,11 +320,11 @@ inline void build_qt_tile(int S, int SP, const double* V, const double* Vinv,
   std::memset(out, 0, qt_bytes(SP));
   const size_t term = 64 * 128;
   const int NB = SP / 64;
-  for (int s = 0; s < S; ++s)
-    for (int t = 0; t < S; ++t) {
-      double q = 0.0;  // Q[t][s]
-      for (int m = 0; m < S; ++m) q += V[t * S + m] * lambda[m] * Vinv[m * S + s];
-      float rem = (float)q;
+  double q[kMaxStates];
+  for (int t = 0; t < S; ++t) {
+    q_row(S, V, Vinv, lambda, t, q);
+    for (int s = 0; s < S; ++s) {
+      float rem = (float)q[s];
       const int on = rows ? t : s, ok = rows ? s : t;  // the entry's row and column
       const int n = on & 63, k = ok & 63;
       const size_t blk = (size_t)(ok >> 6) * NB * kTcQtBytes + (size_t)(on >> 6) * term;
@@ -320,6 +335,7 @@ inline void build_qt_tile(int S, int SP, const double* V, const double* Vinv,
         rem = rem - host_bf16_value(b);
       }
     }
+  }
 }
 
 // FP32 paths whose post-order pass stores U = P p per node instead of p
@@ -337,12 +353,11 @@ template <typename T>
 inline void build_q_matrix(int S, int SP, const double* V, const double* Vinv,
                            const double* lambda, T* out) {
   for (int i = 0; i < SP * SP; ++i) out[i] = T(0);
-  for (int t = 0; t < S; ++t)
-    for (int s = 0; s < S; ++s) {
-      double q = 0.0;
-      for (int m = 0; m < S; ++m) q += V[t * S + m] * lambda[m] * Vinv[m * S + s];
-      out[t * SP + s] = (T)q;
-    }
+  double q[kMaxStates];
+  for (int t = 0; t < S; ++t) {
+    q_row(S, V, Vinv, lambda, t, q);
+    for (int s = 0; s < S; ++s) out[t * SP + s] = (T)q[s];
+  }
 }
 
 // FP32 with 65..128 states runs on the tensor cores too (kernels_tcb.cuh):
