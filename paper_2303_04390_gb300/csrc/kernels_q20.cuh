@@ -15,10 +15,11 @@
 //
 // Measured (256 taxa x 5,000 patterns x 4 categories): post-order 0.366 ->
 // 0.299 ms, pre-order 0.590 -> 0.510 ms.  What bounds it now is latency at 8
-// warps per SM (ncu, a 20-node level: 8.0 clocks per warp and issue, 3.1 of
-// them for global loads and 1.4 for instructions) and the last wave of a
-// level.  Vectors in registers and the product unrolled over all 20 rows were
-// slower (0.70 ms: instruction fetch).
+// (pre-order) and 10 to 11 warps per SM and the last wave of a level (ncu:
+// pre-order 5.3 clocks per warp and issue, 1.1 of them for global and 0.8 for
+// shared loads, issue active 33 to 36%; post-order 9 to 10 clocks, 5 for global
+// loads, issue active 22 to 37%).  Vectors in registers and the product
+// unrolled over all 20 rows were slower (0.70 ms: instruction fetch).
 //
 // The pre-order step takes the numerator from the other side,
 //   num_x = gamma_r (a_x Q) . U_x = gamma_r a_x . (Q U_x),

@@ -25,7 +25,7 @@
 // sums over categories and the two ratios of a pattern are spread over its
 // lanes, one instruction for all of them.  256 taxa x 3,001 patterns x 4
 // categories: post-order 0.42 -> 0.19 ms, pre-order 0.98 -> 0.56 ms against
-// per-level launches that formed P p, dP p and P' a (ncu: FP64 pipe 64% and
+// per-level launches that formed P p, dP p and P' a (ncu: FP64 pipe 65% and
 // 70% of the time, 24 and 80 FP64 instructions a step; the rest is the third
 // block that some SMs hold and others do not).  Spreading a tile over a
 // cluster of 2, 4 or 8 blocks lost at every size (the cluster barrier: 0.84,

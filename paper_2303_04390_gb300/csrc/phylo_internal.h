@@ -119,10 +119,10 @@ constexpr int kP4MatKinds = 3;
 // How a pass of the level schedule runs.
 enum PassMode {
   kByLevel,  // one launch per level
-  kByTile,   // one launch: a pattern tile walks the tree (kernels_tree.cuh)
-  kWalk      // the same with every partial vector in shared memory
+  kByTile,   // a pattern tile walks runs of levels (kernels_tree.cuh)
+  kWalk      // one launch, every partial vector in shared memory
 };
-// Whole-pass launches, 4 padded states: tiles of one warp of (pattern,
+// These launches, 4 padded states: tiles of one warp of (pattern,
 // category) lanes.
 constexpr int kTreeWarps = 8;      // warps per block, kByTile
 constexpr int kWalkMaxWarps = 16;  // warps per block, kWalk
