@@ -1168,7 +1168,7 @@ cudaError_t launch_level_impl(const LevelArgs<T>& a, int SP, int RP, bool post,
   if (a.n_tiles <= 0 || a.n_level <= 0) return cudaSuccess;
   switch (SP) {
     case 4:
-      if constexpr (std::is_same<T, float>::value) return launch_p4_rp(a, RP, post, st);
+      if constexpr (std::is_same<T, float>::value) return launch_p4(a, post, st);
       else return cudaErrorInvalidValue;  // FP64: launch_tree_pass
     case 20: return launch_small_rp<T, 20>(a, RP, post, st);
     case 64:

@@ -5,7 +5,7 @@
 // root's Eq. 3; Eq. 4 with the fused Eq. 8 ratio and Eq. 7 tile sums).  The
 // mapping is chosen for S = 4, where a (pattern, category) pair carries too
 // little work to pay for per-pair shuffles:
-//  - a thread owns one pattern and all R <= RM categories, so the rescale
+//  - a thread owns one pattern and all R categories, so the rescale
 //    maximum, the sums over categories and the gradient ratio are local;
 //  - the thread issues every 16-byte load of its pattern (R vectors per
 //    input) before it computes, so each warp keeps 3 x R x 512 bytes in
@@ -82,11 +82,11 @@ __device__ __forceinline__ float max4(float2 lo, float2 hi) {
 // P' of the tip branches below a cherry child (i: 0, 1; j: 2, 3).  n holds
 // the node's own P' (post-order: U_k = P_k p_k) or Q (pre-order, one
 // matrix: the Eq. 8 numerator of a child whose U is stored).
-template <int RM, bool PRE, bool CH>
+template <int R, bool PRE, bool CH>
 struct P4Mats {
-  float4 m[2][(PRE ? kP4MatKinds : 1) * RM * 4];
-  float4 g[CH ? 4 : 1][RM * 4];
-  float4 n[PRE ? 4 : RM * 4];
+  float4 m[2][(PRE ? kP4MatKinds : 1) * R * 4];
+  float4 g[CH ? 4 : 1][R * 4];
+  float4 n[PRE ? 4 : R * 4];
 };
 
 // Power-of-two rescale of a vector whose largest magnitude is mx (finite,
@@ -151,15 +151,22 @@ __device__ __forceinline__ void p4_child(int y, int S, float4 v,
 #endif
 constexpr int kP4PreMinBlocks = PHYLO_P4_PRE_BLOCKS;
 
-// RM: categories unrolled (R <= RM); EX: R == RM, so that no per-category
-// test is left at run time.
-template <int RM, bool EX, bool PRE, bool CH>
+// R: the category count.  Every count has its own form.  A form with the count
+// at run time (3 in four unrolled categories; 5, 6 and 7 in eight) gave a wrong
+// Eq. 8 sum for the second child of a node with two tips at 5, 6 and 7, and with
+// fewer resident blocks asked for, an illegal address.  The same source compiled
+// for the CPU, under address and undefined-behaviour sanitizers, gave the right
+// sums and stayed in its arrays: no fault was found in it, so the device code of
+// that form (nvcc 13.0.88) is the likely cause, and it is not used.  1,024 taxa x
+// 10,000 patterns, both passes: 542 us with 3 categories, 631 with 4 (as before),
+// 811 with 5, 1,378 with 7, 1,800 with 8 (as before).
+template <int R, bool PRE, bool CH>
 __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
     level_p4_kernel(LevelArgs<float> a) {
-  __shared__ P4Mats<RM, PRE, CH> sm;
+  __shared__ P4Mats<R, PRE, CH> sm;
   __shared__ uint64_t bar;
   const int tid = threadIdx.x, lane = tid & 31;
-  const int R = EX ? RM : a.n_cat, C = a.n_patterns, S = a.n_states;
+  const int C = a.n_patterns, S = a.n_states;
   const int4 d = a.level_desc[blockIdx.y];
   const int k = d.x, bi = d.y, bj = d.z;
   const bool ci = d.w & kDescFlagCompact0, cj = d.w & kDescFlagCompact1;
@@ -169,9 +176,9 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
   const int c = blockIdx.x * kP4Threads + tid;
   const int tile = c >> 5;  // this warp's tile
   const bool valid = c < C;
-  const uint32_t mbytes = (uint32_t)R * 64;  // one matrix of every category
-  const uint32_t cbytes = (PRE ? kP4MatKinds : 1) * mbytes;  // a child's block
-  const size_t bstride = (size_t)kP4MatKinds * R * 16;      // floats per branch
+  constexpr uint32_t mbytes = R * 64;  // one matrix of every category
+  constexpr uint32_t cbytes = (PRE ? kP4MatKinds : 1) * mbytes;  // a child's block
+  constexpr size_t bstride = (size_t)kP4MatKinds * R * 16;  // floats per branch
   if (tid == 0) mbar_init_fenced(&bar, 1);
   __syncthreads();
   // The descriptor, the tree and the tip states are written by the host and
@@ -197,7 +204,7 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
   };
   if (a.mats_ready) issue_copies();
   // ---- every global load of this pattern, issued before any use ----------
-  float4 vi[RM], vj[RM], q[RM];
+  float4 vi[R], vj[R], q[R];
   int yi = -1, yj = -1, ei = 0, ej = 0;
   int ya[2] = {0, 0}, yb[2] = {0, 0};  // tip states below cherry children
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -216,18 +223,17 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
   pdl_wait_and_release();
   if (!a.mats_ready) issue_copies();
 #pragma unroll
-  for (int r = 0; r < RM; ++r) {
-    const bool on = valid && r < R;
+  for (int r = 0; r < R; ++r) {
     vi[r] = zero4; vj[r] = zero4; q[r] = zero4;
-    if (on && !ci && !hi_)
+    if (valid && !ci && !hi_)
       vi[r] = bi < a.n_tips ? __ldg(reinterpret_cast<const float4*>(a.tip_partials) + (size_t)bi * C + c)
                             : __ldg(reinterpret_cast<const float4*>(a.post) +
                                     p4_index(bi - a.n_tips, c, r, R, a.n_tiles));
-    if (on && !cj && !hj_)
+    if (valid && !cj && !hj_)
       vj[r] = bj < a.n_tips ? __ldg(reinterpret_cast<const float4*>(a.tip_partials) + (size_t)bj * C + c)
                             : __ldg(reinterpret_cast<const float4*>(a.post) +
                                     p4_index(bj - a.n_tips, c, r, R, a.n_tiles));
-    if (PRE && on && k != a.root)
+    if (PRE && valid && k != a.root)
       q[r] = __ldg(reinterpret_cast<const float4*>(a.pre) +
                    p4_index(k - a.n_tips, c, r, R, a.n_tiles));
   }
@@ -235,7 +241,7 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
     const float4 pr = make_float4(a.root_pit[0], S > 1 ? a.root_pit[1] : 0.f,
                                   S > 2 ? a.root_pit[2] : 0.f, S > 3 ? a.root_pit[3] : 0.f);
 #pragma unroll
-    for (int r = 0; r < RM; ++r) q[r] = pr;
+    for (int r = 0; r < R; ++r) q[r] = pr;
   }
   if (!PRE && valid) {  // a cherry's exponent is 0 (its partials are not rescaled)
     if (bi >= a.n_tips && !hi_) ei = a.escale[(size_t)(bi - a.n_tips) * a.escale_stride + c];
@@ -256,8 +262,8 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
   if constexpr (CH) {
     // a cherry child's partials from its two tip states
 #pragma unroll
-    for (int r = 0; r < RM; ++r) {
-      if (!(valid && r < R)) continue;
+    for (int r = 0; r < R; ++r) {
+      if (!valid) continue;
       if (hi_) {
         const float4 u = p4_col(sm.g[0] + r * 4, ya[0], S), w = p4_col(sm.g[1] + r * 4, yb[0], S);
         vi[r] = make_float4(u.x * w.x, u.y * w.y, u.z * w.z, u.w * w.w);
@@ -272,21 +278,18 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
   const bool su_i = bi >= a.n_tips && !hi_, su_j = bj >= a.n_tips && !hj_;
   if (!PRE) {
     // ---- Eq. 2: p_k = U_i o U_j for every category -------------------------
-    float2 plo[RM], phi[RM];
+    float2 plo[R], phi[R];
     float m = 0.f;
 #pragma unroll
-    for (int r = 0; r < RM; ++r) {
-      plo[r] = make_float2(0.f, 0.f); phi[r] = plo[r];
-      if (r < R) {
-        float2 ilo, ihi, jlo, jhi, d0, d1;
-        if (su_i) { ilo = lo2(vi[r]); ihi = hi2(vi[r]); }
-        else p4_child<false>(yi, S, vi[r], PTi + r * 4, nullptr, ilo, ihi, d0, d1);
-        if (su_j) { jlo = lo2(vj[r]); jhi = hi2(vj[r]); }
-        else p4_child<false>(yj, S, vj[r], PTj + r * 4, nullptr, jlo, jhi, d0, d1);
-        plo[r] = __fmul2_rn(ilo, jlo);
-        phi[r] = __fmul2_rn(ihi, jhi);
-        m = fmaxf(m, max4(plo[r], phi[r]));
-      }
+    for (int r = 0; r < R; ++r) {
+      float2 ilo, ihi, jlo, jhi, d0, d1;
+      if (su_i) { ilo = lo2(vi[r]); ihi = hi2(vi[r]); }
+      else p4_child<false>(yi, S, vi[r], PTi + r * 4, nullptr, ilo, ihi, d0, d1);
+      if (su_j) { jlo = lo2(vj[r]); jhi = hi2(vj[r]); }
+      else p4_child<false>(yj, S, vj[r], PTj + r * 4, nullptr, jlo, jhi, d0, d1);
+      plo[r] = __fmul2_rn(ilo, jlo);
+      phi[r] = __fmul2_rn(ihi, jhi);
+      m = fmaxf(m, max4(plo[r], phi[r]));
     }
     int e = 0;
     float f = 1.f;
@@ -299,14 +302,13 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
       if (valid) {  // U_k = P_k p_k, stored with p_k's exponent
         float4* out = reinterpret_cast<float4*>(a.post) + p4_index(k - a.n_tips, c, 0, R, a.n_tiles);
 #pragma unroll
-        for (int r = 0; r < RM; ++r)
-          if (r < R) {
-            const float2 lo = __fmul2_rn(plo[r], make_float2(f, f));
-            const float2 hi = __fmul2_rn(phi[r], make_float2(f, f));
-            float2 ulo, uhi;
-            mv4t(sm.n + r * 4, make_float4(lo.x, lo.y, hi.x, hi.y), ulo, uhi);
-            out[32 * r] = make_float4(ulo.x, ulo.y, uhi.x, uhi.y);
-          }
+        for (int r = 0; r < R; ++r) {
+          const float2 lo = __fmul2_rn(plo[r], make_float2(f, f));
+          const float2 hi = __fmul2_rn(phi[r], make_float2(f, f));
+          float2 ulo, uhi;
+          mv4t(sm.n + r * 4, make_float4(lo.x, lo.y, hi.x, hi.y), ulo, uhi);
+          out[32 * r] = make_float4(ulo.x, ulo.y, uhi.x, uhi.y);
+        }
         a.escale[(size_t)(k - a.n_tips) * a.escale_stride + c] = e;
       }
       return;
@@ -318,8 +320,8 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
       const float2 ph = make_float2(S > 2 ? a.root_pit[2] : 0.f, S > 3 ? a.root_pit[3] : 0.f);
       float L = 0.f;
 #pragma unroll
-      for (int r = 0; r < RM; ++r)
-        if (r < R) L = fmaf(a.cat_wt[r], dot22(pl, ph, plo[r], phi[r]) * f, L);
+      for (int r = 0; r < R; ++r)
+        L = fmaf(a.cat_wt[r], dot22(pl, ph, plo[r], phi[r]) * f, L);
       if (!(L > 0.f) || !isfinite(L)) atomicOr(a.err, ERR_ZERO_PARTIAL);
       term = (double)a.pattern_wt[c] * (log((double)L) + (double)e * 0.69314718055994530942);
     }
@@ -330,48 +332,46 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
   }
   // ---- Eq. 4 and Eq. 8: children's pre-order partials and the ratio ------
   const bool int_i = bi >= a.n_tips, int_j = bj >= a.n_tips;
-  float2 qilo[RM], qihi[RM], qjlo[RM], qjhi[RM];
+  float2 qilo[R], qihi[R], qjlo[R], qjhi[R];
   float Ni = 0.f, Nj = 0.f, Dn = 0.f, mi = 0.f, mj = 0.f;
 #pragma unroll
-  for (int r = 0; r < RM; ++r) {
+  for (int r = 0; r < R; ++r) {
     qilo[r] = make_float2(0.f, 0.f); qihi[r] = qilo[r]; qjlo[r] = qilo[r]; qjhi[r] = qilo[r];
-    if (r < R) {
-      const float2 ql = lo2(q[r]), qh = hi2(q[r]);
-      float2 uilo, uihi, wilo, wihi, ujlo, ujhi, wjlo, wjhi;
-      // a stored U needs no product here; the others give U and dP p (or columns)
-      if (su_i) { uilo = lo2(vi[r]); uihi = hi2(vi[r]); }
-      else p4_child<true>(yi, S, vi[r], PTi + r * 4, DTi + r * 4, uilo, uihi, wilo, wihi);
-      if (su_j) { ujlo = lo2(vj[r]); ujhi = hi2(vj[r]); }
-      else p4_child<true>(yj, S, vj[r], PTj + r * 4, DTj + r * 4, ujlo, ujhi, wjlo, wjhi);
-      const float2 ailo = __fmul2_rn(ql, ujlo), aihi = __fmul2_rn(qh, ujhi);  // a_i
-      const float2 ajlo = __fmul2_rn(ql, uilo), ajhi = __fmul2_rn(qh, uihi);  // a_j
-      const float w = a.cat_wt[r];
-      float ni, nj;
-      if (su_i || su_j) {
-        const float gam = (float)a.rates[r];
-        float2 lo, hi;
-        if (su_i) {  // gamma_r (a_i' Q) U_i
-          mtv4r(sm.n, ailo, aihi, lo, hi);
-          ni = gam * dot22(lo, hi, uilo, uihi);
-        }
-        if (su_j) {
-          mtv4r(sm.n, ajlo, ajhi, lo, hi);
-          nj = gam * dot22(lo, hi, ujlo, ujhi);
-        }
+    const float2 ql = lo2(q[r]), qh = hi2(q[r]);
+    float2 uilo, uihi, wilo, wihi, ujlo, ujhi, wjlo, wjhi;
+    // a stored U needs no product here; the others give U and dP p (or columns)
+    if (su_i) { uilo = lo2(vi[r]); uihi = hi2(vi[r]); }
+    else p4_child<true>(yi, S, vi[r], PTi + r * 4, DTi + r * 4, uilo, uihi, wilo, wihi);
+    if (su_j) { ujlo = lo2(vj[r]); ujhi = hi2(vj[r]); }
+    else p4_child<true>(yj, S, vj[r], PTj + r * 4, DTj + r * 4, ujlo, ujhi, wjlo, wjhi);
+    const float2 ailo = __fmul2_rn(ql, ujlo), aihi = __fmul2_rn(qh, ujhi);  // a_i
+    const float2 ajlo = __fmul2_rn(ql, uilo), ajhi = __fmul2_rn(qh, uihi);  // a_j
+    const float w = a.cat_wt[r];
+    float ni, nj;
+    if (su_i || su_j) {
+      const float gam = (float)a.rates[r];
+      float2 lo, hi;
+      if (su_i) {  // gamma_r (a_i' Q) U_i
+        mtv4r(sm.n, ailo, aihi, lo, hi);
+        ni = gam * dot22(lo, hi, uilo, uihi);
       }
-      if (!su_i) ni = dot22(ailo, aihi, wilo, wihi);
-      if (!su_j) nj = dot22(ajlo, ajhi, wjlo, wjhi);
-      Ni = fmaf(w, ni, Ni);
-      Nj = fmaf(w, nj, Nj);
-      Dn = fmaf(w, dot22(ailo, aihi, uilo, uihi), Dn);
-      if (int_i) {
-        mtv4r(Pi + r * 4, ailo, aihi, qilo[r], qihi[r]);
-        mi = fmaxf(mi, max4(qilo[r], qihi[r]));
+      if (su_j) {
+        mtv4r(sm.n, ajlo, ajhi, lo, hi);
+        nj = gam * dot22(lo, hi, ujlo, ujhi);
       }
-      if (int_j) {
-        mtv4r(Pj + r * 4, ajlo, ajhi, qjlo[r], qjhi[r]);
-        mj = fmaxf(mj, max4(qjlo[r], qjhi[r]));
-      }
+    }
+    if (!su_i) ni = dot22(ailo, aihi, wilo, wihi);
+    if (!su_j) nj = dot22(ajlo, ajhi, wjlo, wjhi);
+    Ni = fmaf(w, ni, Ni);
+    Nj = fmaf(w, nj, Nj);
+    Dn = fmaf(w, dot22(ailo, aihi, uilo, uihi), Dn);
+    if (int_i) {
+      mtv4r(Pi + r * 4, ailo, aihi, qilo[r], qihi[r]);
+      mi = fmaxf(mi, max4(qilo[r], qihi[r]));
+    }
+    if (int_j) {
+      mtv4r(Pj + r * 4, ajlo, ajhi, qjlo[r], qjhi[r]);
+      mj = fmaxf(mj, max4(qjlo[r], qjhi[r]));
     }
   }
   F2 gi = {0.f, 0.f}, gj = {0.f, 0.f};
@@ -389,12 +389,11 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
       else (void)p4_rescale(mi, f);
       float4* out = reinterpret_cast<float4*>(a.pre) + p4_index(bi - a.n_tips, c, 0, R, a.n_tiles);
 #pragma unroll
-      for (int r = 0; r < RM; ++r)
-        if (r < R) {
-          const float2 lo = __fmul2_rn(qilo[r], make_float2(f, f));
-          const float2 hi = __fmul2_rn(qihi[r], make_float2(f, f));
-          out[32 * r] = make_float4(lo.x, lo.y, hi.x, hi.y);
-        }
+      for (int r = 0; r < R; ++r) {
+        const float2 lo = __fmul2_rn(qilo[r], make_float2(f, f));
+        const float2 hi = __fmul2_rn(qihi[r], make_float2(f, f));
+        out[32 * r] = make_float4(lo.x, lo.y, hi.x, hi.y);
+      }
     }
     if (int_j) {
       float f = 1.f;
@@ -402,12 +401,11 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
       else (void)p4_rescale(mj, f);
       float4* out = reinterpret_cast<float4*>(a.pre) + p4_index(bj - a.n_tips, c, 0, R, a.n_tiles);
 #pragma unroll
-      for (int r = 0; r < RM; ++r)
-        if (r < R) {
-          const float2 lo = __fmul2_rn(qjlo[r], make_float2(f, f));
-          const float2 hi = __fmul2_rn(qjhi[r], make_float2(f, f));
-          out[32 * r] = make_float4(lo.x, lo.y, hi.x, hi.y);
-        }
+      for (int r = 0; r < R; ++r) {
+        const float2 lo = __fmul2_rn(qjlo[r], make_float2(f, f));
+        const float2 hi = __fmul2_rn(qjhi[r], make_float2(f, f));
+        out[32 * r] = make_float4(lo.x, lo.y, hi.x, hi.y);
+      }
     }
   }
   // Both children's tile sums in one butterfly: after the first exchange
@@ -428,31 +426,26 @@ __global__ void __launch_bounds__(kP4Threads, PRE ? kP4PreMinBlocks : 0)
   }
 }
 
-template <int RM, bool EX>
-cudaError_t launch_p4_ex(const LevelArgs<float>& a, bool post, cudaStream_t st) {
+template <int R>
+cudaError_t launch_p4(const LevelArgs<float>& a, bool post, cudaStream_t st) {
   dim3 grid((a.n_tiles + 1) / 2, a.n_level);
   if (a.level_cherry) {
-    if (post) return launch_pdl(level_p4_kernel<RM, EX, false, true>, grid, kP4Threads, 0, st, a);
-    return launch_pdl(level_p4_kernel<RM, EX, true, true>, grid, kP4Threads, 0, st, a);
+    if (post) return launch_pdl(level_p4_kernel<R, false, true>, grid, kP4Threads, 0, st, a);
+    return launch_pdl(level_p4_kernel<R, true, true>, grid, kP4Threads, 0, st, a);
   }
-  if (post) return launch_pdl(level_p4_kernel<RM, EX, false, false>, grid, kP4Threads, 0, st, a);
-  return launch_pdl(level_p4_kernel<RM, EX, true, false>, grid, kP4Threads, 0, st, a);
+  if (post) return launch_pdl(level_p4_kernel<R, false, false>, grid, kP4Threads, 0, st, a);
+  return launch_pdl(level_p4_kernel<R, true, false>, grid, kP4Threads, 0, st, a);
 }
 
-template <int RM>
-cudaError_t launch_p4(const LevelArgs<float>& a, bool post, cudaStream_t st) {
-  if (a.n_cat == RM) return launch_p4_ex<RM, true>(a, post, st);
-  if constexpr (RM > 2) return launch_p4_ex<RM, false>(a, post, st);
-  return cudaErrorInvalidValue;
-}
-
-// RP (next power of two >= R) selects the unrolled category count.
-inline cudaError_t launch_p4_rp(const LevelArgs<float>& a, int RP, bool post,
-                                cudaStream_t st) {
-  switch (RP) {
+inline cudaError_t launch_p4(const LevelArgs<float>& a, bool post, cudaStream_t st) {
+  switch (a.n_cat) {
     case 1: return launch_p4<1>(a, post, st);
     case 2: return launch_p4<2>(a, post, st);
+    case 3: return launch_p4<3>(a, post, st);
     case 4: return launch_p4<4>(a, post, st);
+    case 5: return launch_p4<5>(a, post, st);
+    case 6: return launch_p4<6>(a, post, st);
+    case 7: return launch_p4<7>(a, post, st);
     case 8: return launch_p4<8>(a, post, st);
     default: return cudaErrorInvalidValue;
   }
